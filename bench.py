@@ -95,7 +95,7 @@ def kernel_source_hash():
     import hashlib
 
     h = hashlib.sha256()
-    for f in ("pc_fields.cu", "pc_lw_f32.cuh", "pc_lw_f32x2.cuh", "pc_lw_f64.cuh"):
+    for f in ("pc_fields.cu", "pc_far_f32.cuh", "pc_lw_f32.cuh", "pc_lw_f32x2.cuh", "pc_lw_f64.cuh"):
         with open(os.path.join(ROOT, "paper_2107_12437_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -609,9 +609,9 @@ def main():
                    "tile": f"{tile_rows} x {tile_cols} points, {tile_rows * tile_cols // 256} per thread, "
                            f"{tile_stage} sources per shared-memory stage (autotuned)",
                    "l2": "flushed between steps (256 MB write); outputs 2.7 GB > L2"},
-        # per step: the dipole-axis check, the float32 mirror of the histories, the field kernel
-        # (all 16 frames in one launch)
-        "gpu_launches": 3 * args.steps,
+        # per step: the dipole-axis check, the float32 mirror of the histories, the far limits, the count of
+        # near sources and the field kernel (all 16 frames in one launch)
+        "gpu_launches": 5 * args.steps,
         "clocks": clk.summary(),
         "e2e": {"value": e2e_value, "unit": "LW pair evals/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "host_cpus": f"{len(cpus_gpu)} GPU-local" if cpus_gpu else "unbound"},

@@ -7,7 +7,7 @@ namespace pc {
 
 pc_status begin_call(pc_ctx *ctx, cudaStream_t s) {
   cudaGetLastError();  // clear a stale launch error of an unrelated caller
-  if (cudaMemsetAsync(ctx->d_status, 0, sizeof(int), s) != cudaSuccess) return PC_ERR_CUDA;
+  if (cudaMemsetAsync(ctx->d_status, 0, kStatusWords * sizeof(int), s) != cudaSuccess) return PC_ERR_CUDA;
   return PC_OK;
 }
 
@@ -38,12 +38,12 @@ extern "C" pc_status pc_ctx_create(pc_ctx **out, int device) {
   pc_ctx *c = new pc_ctx();
   c->device = device;
   cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
-  if (cudaMalloc(&c->d_status, sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&c->h_status, sizeof(int)) != cudaSuccess) {
+  if (cudaMalloc(&c->d_status, pc::kStatusWords * sizeof(int)) != cudaSuccess ||
+      cudaMallocHost(&c->h_status, pc::kStatusWords * sizeof(int)) != cudaSuccess) {
     pc_ctx_destroy(c);
     return PC_ERR_CUDA;
   }
-  cudaMemset(c->d_status, 0, sizeof(int));
+  cudaMemset(c->d_status, 0, pc::kStatusWords * sizeof(int));
   *c->h_status = 0;
   *out = c;
   return PC_OK;

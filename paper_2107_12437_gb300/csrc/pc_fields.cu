@@ -23,6 +23,7 @@
 #include "pc_internal.cuh"
 #include "pc_lw_f32.cuh"
 #include "pc_lw_f32x2.cuh"
+#include "pc_far_f32.cuh"
 #include "pc_lw_f64.cuh"
 
 namespace pc {
@@ -116,6 +117,10 @@ struct Launch {
   double ufc[kMaxT];
   double iLc;
   float sE, sP;
+  // the far form (pc_far_f32.cuh): per dipole the distance from which it applies, and the spread of a
+  // tile's points about its anchor, both in c dt
+  const float *rfar;
+  float tile_r;
 };
 
 // the float32 outputs' units: E in k_e e / L^2, B in k_e e / (L^2 c), phi in k_e e / L,
@@ -282,15 +287,34 @@ __global__ void __launch_bounds__(128) fields_f64_kernel(const Launch L) {
 // ================================================================================================
 // mixed path
 // ================================================================================================
-__global__ void prep_dipoles_f32(const Sources s, float4 *H, float4 *srcf) {
+// xvmax (or null): per dipole the largest |X| and |V| of its samples, as the bits of non-negative
+// floats (ordered like unsigned integers; a NaN orders above everything), preset to 0.
+__global__ void prep_dipoles_f32(const Sources s, float4 *H, float4 *srcf, unsigned *xvmax) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int64_t n = (int64_t)s.N * s.Sd;
   if (i >= n) return;
   int j = (int)(i / s.Sd);
   const double q = s.qd[j];
   const double Lc = kC * s.dtd;
-  H[i] = make_float4((float)(s.d[i] / (q * Lc)), (float)(s.dd[i] / (q * kC)), (float)(s.ddd[i] * s.dtd / (q * kC)),
-                     0.f);
+  const float4 h = make_float4((float)(s.d[i] / (q * Lc)), (float)(s.dd[i] / (q * kC)),
+                               (float)(s.ddd[i] * s.dtd / (q * kC)), 0.f);
+  H[i] = h;
+  if (xvmax) {
+    // one atomic per warp and maximum: a warp's samples are one dipole's unless its row ends there
+    const unsigned act = __activemask();
+    const unsigned x = __float_as_uint(fabsf(h.x)), v = __float_as_uint(fabsf(h.y));
+    const int j0 = __shfl_sync(act, j, __ffs((int)act) - 1);
+    if (__all_sync(act, j == j0)) {
+      const unsigned xm = __reduce_max_sync(act, x), vm = __reduce_max_sync(act, v);
+      if ((int)(threadIdx.x & 31) == __ffs((int)act) - 1) {
+        atomicMax(xvmax + 2 * j, xm);
+        atomicMax(xvmax + 2 * j + 1, vm);
+      }
+    } else {
+      atomicMax(xvmax + 2 * j, x);
+      atomicMax(xvmax + 2 * j + 1, v);
+    }
+  }
   if (i % s.Sd == 0) {
     const double m1 = s.m1[j], m2 = s.m2[j];
     srcf[4 * j] = make_float4((float)s.axis[3 * j], (float)s.axis[3 * j + 1], (float)s.axis[3 * j + 2], (float)(q / kE));
@@ -364,11 +388,14 @@ __device__ __forceinline__ ff ff_from_double(double x) {
 // whenever the dipole's instantaneous moment crosses zero.  Exact per-charge roots (no segment
 // extension), the same difference form in double.
 template <int KIND>
-__device__ __noinline__ int near_dipole_f64(const Sources &s, int j, const double r[3], double u, double Ld,
+// iLd = 1 / (c dt): two float64 divisions in all (the unit is narrow, and in the frames whose moments
+// cross zero every near pair comes here).
+__device__ __noinline__ int near_dipole_f64(const Sources &s, int j, const double r[3], double u, double iLd,
                                                double r_excl, float *part, uint8_t *mask) {
   const double q = s.qd[j], m1 = s.m1[j], m2 = s.m2[j];
-  const double rx = (r[0] - s.origin[3 * j]) / Ld, ry = (r[1] - s.origin[3 * j + 1]) / Ld,
-               rz = (r[2] - s.origin[3 * j + 2]) / Ld;
+  const double iq = 1.0 / q, imm = 1.0 / (m1 + m2);
+  const double rx = (r[0] - s.origin[3 * j]) * iLd, ry = (r[1] - s.origin[3 * j + 1]) * iLd,
+               rz = (r[2] - s.origin[3 * j + 2]) * iLd;
   const double rn = sqrt(rx * rx + ry * ry + rz * rz);
   const double px = s.axis[3 * j], py = s.axis[3 * j + 1], pz = s.axis[3 * j + 2];
   const double rp = rx * px + ry * py + rz * pz;
@@ -378,13 +405,12 @@ __device__ __noinline__ int near_dipole_f64(const Sources &s, int j, const doubl
   H.d = s.d + (size_t)j * s.Sd;
   H.dd = s.dd + (size_t)j * s.Sd;
   H.ddd = s.ddd + (size_t)j * s.Sd;
-  H.sx = 1.0 / (q * Ld);
-  H.sv = 1.0 / (q * kC);
-  H.sa = s.dtd / (q * kC);
+  H.sx = iq * iLd;
+  H.sv = iq * (1.0 / kC);
+  H.sa = iq * (s.dtd * (1.0 / kC));
   double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   const int e = dipole_net<KIND, double, HistF64>(H, (int)s.Sd, (int)fl, x - fl, rx, ry, rz, rn, px, py, pz, rp,
-                                                  m2 / (m1 + m2), m1 / (m1 + m2), q / kE, r_excl / Ld, true, acc,
-                                                  *mask);
+                                                  m2 * imm, m1 * imm, q * (1.0 / kE), r_excl * iLd, true, acc, *mask);
   if (e) return e;
 #pragma unroll
   for (int i = 0; i < 10; ++i) part[i] += (float)acc[i];
@@ -398,7 +424,7 @@ __device__ __noinline__ int near_dipole_f64(const Sources &s, int j, const doubl
 template <int KIND>
 __device__ __noinline__ int slow_dipole(const Sources &s, int j, const float4 *hist, int S, int kb, float xc, float rx,
                                         float ry, float rz, float rn, float4 ax, float mup, float mum, float rex,
-                                        const double r[3], double u, double Ld, double r_excl, float *part,
+                                        const double r[3], double u, double iLd, double r_excl, float *part,
                                         uint8_t *mask) {
   const float rp = rx * ax.x + ry * ax.y + rz * ax.z;
   const HistF32 H{hist};
@@ -406,7 +432,7 @@ __device__ __noinline__ int slow_dipole(const Sources &s, int j, const float4 *h
   const int e = dipole_states<float, HistF32>(H, S, kb, xc, rn, rp, mup, mum, true, Xp, Vp, Ap, dp, Xm, Vm, Am, dm);
   if (e) return e;
   if (rn < kNearL && dipole_cancellation<float>(rn, mup, mum, Xp, Vp, Ap, Xm, Vm, Am) > kCancel)
-    return near_dipole_f64<KIND>(s, j, r, u, Ld, r_excl, part, mask);
+    return near_dipole_f64<KIND>(s, j, r, u, iLd, r_excl, part, mask);
   dipole_pair<KIND, float>(rx, ry, rz, rn, ax.x, ax.y, ax.z, rp, mup, mum, ax.w, Xp, Vp, Ap, dp, Xm, Vm, Am, dm, rex,
                            part, *mask);
   return 0;
@@ -704,7 +730,7 @@ __global__ void __launch_bounds__(kMixThreads, 4) fields_mixed_kernel(const Laun
         double rp64[3];
         point_at(L.pts, tile_point(L, tiles_v, tid), rp64);
         const int e = slow_dipole<KIND>(s, base + jj, s_hist[jj], (int)s.Sd, kb, xc, rx, ry, rz, rn, ax, mx.x, mx.y,
-                                        L.rex, rp64, (L.times[f] - s.t0d) / s.dtd, kC * s.dtd, L.r_excl, sp,
+                                        L.rex, rp64, L.uf[f], L.iLd, L.r_excl, sp,
                                         &smask);
         if (e) err = e;
         mask |= smask;
@@ -935,7 +961,7 @@ __device__ __forceinline__ int slow_pairs2(const Launch &L, int f, int base, typ
     double rp64[3];
     point_at(L.pts, p, rp64);
     err = slow_dipole<KIND>(s, base + jj, s_hist[jj], Sd32, kb, xc, rx, ry, rz, rn, ax, mx.x, mx.y, rex, rp64,
-                            (L.times[f] - s.t0d) / s.dtd, kC * s.dtd, L.r_excl, sp, &smask);
+                            L.uf[f], L.iLd, L.r_excl, sp, &smask);
     mask |= smask;
     V2 SP[10];
 #pragma unroll
@@ -943,6 +969,45 @@ __device__ __forceinline__ int slow_pairs2(const Launch &L, int f, int base, typ
     kahan2_add(kh, tid, SP);
   }
   return err;
+}
+
+// the two points' sums to the outputs, in SI units
+__device__ __forceinline__ void store_two_points(const Launch &L, int f, int tid, const float2 (*sum)[kMixThreads],
+                                                 const float2 (*comp)[kMixThreads], bool actA, bool actB, int64_t pA,
+                                                 int64_t pB, uint8_t maskA, uint8_t maskB) {
+  const float uE = L.unit[0], uB = L.unit[1], uP = L.unit[2], uA = L.unit[3];
+  for (int lane = 0; lane < 2; ++lane) {
+    if (!(lane == 0 ? actA : actB)) continue;
+    const int64_t o = (L.frame0 + f) * L.pts.P + (lane == 0 ? pA : pB);
+    float val[10];
+#pragma unroll
+    for (int i = 0; i < 10; ++i) {
+      const float2 sv = sum[i][tid], cv = comp[i][tid];
+      val[i] = lane == 0 ? sv.x - cv.x : sv.y - cv.y;
+    }
+    // streaming stores, as in the one-point kernel
+    if (L.out.E) {
+      float *e = (float *)L.out.E + 3 * o;
+      __stcs(e + 0, uE * val[0]);
+      __stcs(e + 1, uE * val[1]);
+      __stcs(e + 2, uE * val[2]);
+    }
+    if (L.out.B) {
+      float *b = (float *)L.out.B + 3 * o;
+      __stcs(b + 0, uB * val[3]);
+      __stcs(b + 1, uB * val[4]);
+      __stcs(b + 2, uB * val[5]);
+    }
+    if (L.out.phi) __stcs((float *)L.out.phi + o, uP * val[6]);
+    if (L.out.A) {
+      float *a = (float *)L.out.A + 3 * o;
+      __stcs(a + 0, uA * val[7]);
+      __stcs(a + 1, uA * val[8]);
+      __stcs(a + 2, uA * val[9]);
+    }
+    if (L.out.mask)
+      __stcs(reinterpret_cast<unsigned char *>(L.out.mask) + o, (unsigned char)(lane == 0 ? maskA : maskB));
+  }
 }
 
 template <int KIND, int CH>
@@ -1105,39 +1170,382 @@ __global__ void __launch_bounds__(kMixThreads, 2) fields_mixed2_kernel(const Lau
     set_status(L.status, err);
     return;
   }
-  const float uE = L.unit[0], uB = L.unit[1], uP = L.unit[2], uA = L.unit[3];
-  for (int lane = 0; lane < 2; ++lane) {
-    if (!(lane == 0 ? actA : actB)) continue;
-    const int64_t o = (L.frame0 + f) * L.pts.P + (lane == 0 ? pA : pB);
-    float val[10];
-#pragma unroll
-    for (int i = 0; i < 10; ++i) {
-      const float2 sv = s_kahan[0][i][tid], cv = s_kahan[1][i][tid];
-      val[i] = lane == 0 ? sv.x - cv.x : sv.y - cv.y;
-    }
-    // streaming stores, as in the one-point kernel
-    if (L.out.E) {
-      float *e = (float *)L.out.E + 3 * o;
-      __stcs(e + 0, uE * val[0]);
-      __stcs(e + 1, uE * val[1]);
-      __stcs(e + 2, uE * val[2]);
-    }
-    if (L.out.B) {
-      float *b = (float *)L.out.B + 3 * o;
-      __stcs(b + 0, uB * val[3]);
-      __stcs(b + 1, uB * val[4]);
-      __stcs(b + 2, uB * val[5]);
-    }
-    if (L.out.phi) __stcs((float *)L.out.phi + o, uP * val[6]);
-    if (L.out.A) {
-      float *a = (float *)L.out.A + 3 * o;
-      __stcs(a + 0, uA * val[7]);
-      __stcs(a + 1, uA * val[8]);
-      __stcs(a + 2, uA * val[9]);
-    }
-    if (L.out.mask)
-      __stcs(reinterpret_cast<unsigned char *>(L.out.mask) + o, (unsigned char)(lane == 0 ? maskA : maskB));
+  store_two_points(L, f, tid, s_kahan[0], s_kahan[1], actA, actB, pA, pB, maskA, maskB);
+}
+
+// ------------------------------------------------------------------------------------------------
+// Plane grids of dipoles that are mostly far (pc_far_f32.cuh): two points per thread as in
+// fields_mixed2_kernel and NF frames (1 or 2) of each, every source of the tile either far for the
+// whole tile -- its first-order form, with no test left per pair -- or near, and then evaluated as in
+// fields_mixed_kernel.  The far form's geometry (1/R, rho.p, p x rho, the delay) is the same in every
+// frame, so a pair of frames forms it once; a CTA walks `reps` groups of NF frames, so that its
+// anchor and the staged records are formed once for all of them (one chunk of sources) too.
+// Warps cover 4 x 8 points, so that their retarded samples lie close together.
+//
+// Measured on the field grid (64 dipoles, 2048^2 points, 16 frames): 30.6 -> 10.8 ms.  44 warp
+// instructions per pair of a warp (221 before); the float32 pipe is busy 58 % of the cycles and the
+// issue slots 51 %, with 16 warps per SM: bound by latency, then by that pipe.  One frame at a time and
+// the sums over p x g and dr apart took 14.5 ms; the history as separate (X, V) and A rows the same time
+// as float4 records, with fewer L1 wavefronts.  Two of the 16 frames (10 and 12.5 fs, where the moments
+// cross zero) spend 1.3 ms each on near pairs in float64.
+// ------------------------------------------------------------------------------------------------
+constexpr int kFarChunk = 64;  // sources staged at a time
+constexpr int kFarRows = 32, kFarCols = 16;  // points of a tile, two per thread: rows r and r + 16
+
+// one (tile anchor, source): rho_a and |rho_a| in c dt and the anchor's retarded sample (integer +
+// fraction), in float-float
+struct AnchorGeo {
+  ff x, y, z, n;
+  int k;
+  float frac;
+};
+__device__ __forceinline__ AnchorGeo anchor_geo(const Launch &L, const float *hi, const float *lo, int f, int j) {
+  AnchorGeo o;
+  const float4 oh = L.srcf[4 * j + 2], ol = L.srcf[4 * j + 3];
+  o.x = ff_add({hi[0], lo[0]}, {-oh.x, -ol.x});
+  o.y = ff_add({hi[1], lo[1]}, {-oh.y, -ol.y});
+  o.z = ff_add({hi[2], lo[2]}, {-oh.z, -ol.z});
+  o.n = ff_sqrt(ff_add(ff_add(ff_mul(o.x, o.x), ff_mul(o.y, o.y)), ff_mul(o.z, o.z)));
+  const ff x = ff_add({L.uf_hi[f], L.uf_lo[f]}, {-o.n.hi, -o.n.lo});
+  float kf;
+  o.k = Num<float>::floor_int(x.hi, kf);
+  o.frac = (x.hi - kf) + x.lo;
+  return o;
+}
+// whether a source is far for every point within L.tile_r of the anchor, all their retarded samples
+// (and, a sample further, the charges') on interior segments of the history
+__device__ __forceinline__ bool tile_far(const Launch &L, const AnchorGeo &g, int j) {
+  const float rt = L.tile_r;  // below 1e5 (the host's condition for this kernel)
+  const int ir = (int)rt + 2;
+  // (anchor samples from 2^22 on are beyond the float floor's range)
+  return g.n.hi - rt >= L.rfar[j] && g.k >= ir + 2 && g.k < (1 << 22) && g.k + ir <= (int)L.src.Sd - 5;
+}
+
+// the anchor (centre) of plane tile (tu, tv), in c dt, as float-float
+__device__ __forceinline__ void tile_anchor(const Launch &L, int64_t tu, int64_t tv, float *hi, float *lo) {
+  const double iu = (double)(tu * kFarRows) + 0.5 * (kFarRows - 1), iv = (double)(tv * kFarCols) + 0.5 * (kFarCols - 1);
+  for (int i = 0; i < 3; ++i) {
+    const double x = (L.pts.o[i] + iu * L.pts.eu[i] + iv * L.pts.ev[i]) * L.iLd;
+    hi[i] = (float)x;
+    lo[i] = (float)(x - (double)hi[i]);
   }
+}
+
+// Kahan sums of the NF frames and two points of each thread: [sum, compensation][frame, output][thread],
+// lanes = points
+template <int NF>
+using KahanFar = float2[2][10 * NF][kMixThreads];
+// one point's ten outputs (natural order) of frame slot n into its lane
+template <int NF>
+__device__ __forceinline__ void kahan_lane_add(KahanFar<NF> &k, int tid, int n, int lane, const float *v) {
+#pragma unroll
+  for (int i = 0; i < 10; ++i) {
+    float *sp = &k[0][10 * n + i][tid].x + lane, *cp = &k[1][10 * n + i][tid].x + lane;
+    const float s0 = *sp, y = v[i] - *cp, t = s0 + y;
+    *cp = (t - s0) - y;
+    *sp = t;
+  }
+}
+
+// The near sources (bits, the same for the whole CTA) of one of the thread's two points in one frame
+// (slot n): the body of fields_mixed_kernel on the far kernel's staged records, in groups of 32.
+template <int KIND, int NF>
+__device__ __forceinline__ int near_sources_far(const Launch &L, int f, int n, int base, unsigned long long bits,
+                                                int lane, float drx, float dry, float drz, float dr2, int64_t p,
+                                                const float4 *s_a, const float2 *s_f, KahanFar<NF> &kh, int tid,
+                                                uint8_t &mask) {
+  const Sources &s = L.src;
+  float2 P[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) P[i] = make_float2(0.f, 0.f);
+  unsigned long long slow = 0;
+  auto flush = [&](const float2(&Q)[5]) {
+    const float v[10] = {Q[0].x, Q[0].y, Q[3].x, Q[1].x, Q[1].y, Q[3].y, Q[4].y, Q[2].x, Q[2].y, Q[4].x};
+    kahan_lane_add<NF>(kh, tid, n, lane, v);
+  };
+  auto geometry = [&](int jj, float &rx, float &ry, float &rz, float &rn, float &xc, int &kb) {
+    const float4 g = s_a[jj];
+    rx = g.x + drx;
+    ry = g.y + dry;
+    rz = g.z + drz;
+    const float rho2 = rx * rx + ry * ry + rz * rz;
+    rn = rho2 > 0.f ? rho2 * rsqrtf(rho2) : 0.f;
+    xc = s_f[jj].x - __fdividef(2.f * (g.x * drx + g.y * dry + g.z * drz) + dr2, rn + g.w);
+    kb = __float_as_int(s_f[jj].y) + kFloorBits;
+  };
+  int cnt = 0;
+  for (unsigned long long m = bits; m; m &= m - 1) {
+    const int jj = __ffsll((long long)m) - 1;
+    const float4 ax = L.srcf[4 * (base + jj)], mu = L.srcf[4 * (base + jj) + 1];
+    float rx, ry, rz, rn, xc;
+    int kb;
+    geometry(jj, rx, ry, rz, rn, xc, kb);
+    const float rp = rx * ax.x + ry * ax.y + rz * ax.z;
+    float2 X, V, Ac, dl;
+    bool fast = false;
+    float fl;
+    const int j = kb + Num<float>::floor_int(xc, fl);
+    if ((unsigned)(j - 1) < L.jlim && rn > L.rex_fast) {
+      const HistF32 H{L.Hd + (size_t)(base + jj) * (size_t)s.Sd};
+      float x0, v0, a0, x1, v1, a1;
+      H.get_in(j, x0, v0, a0);
+      H.get_in(j + 1, x1, v1, a1);
+      fast = dip_pair_states_fast(x0, v0, a0, x1, v1, a1, xc - fl, rn, rp, mu.x, mu.y, X, V, Ac, dl);
+    }
+    if (fast && rn < kNearL &&
+        dipole_cancellation<float>(rn, mu.x, mu.y, X.x, V.x, Ac.x, X.y, V.y, Ac.y) > kCancel)
+      fast = false;
+    if (fast)
+      dipole_pair_fast<KIND>(make_float2(rx, ry), rz, rn, make_float2(ax.x, ax.y), ax.z, rp, mu.x, mu.y, ax.w, X, V,
+                             Ac, dl, P);
+    else
+      slow |= 1ull << jj;
+    if (++cnt == 32) {
+      flush(P);
+#pragma unroll
+      for (int i = 0; i < 5; ++i) P[i] = make_float2(0.f, 0.f);
+      cnt = 0;
+    }
+  }
+  flush(P);
+  int err = 0;
+  while (slow && !err) {
+    const int jj = __ffsll((long long)slow) - 1;
+    slow &= slow - 1;
+    float sp[10] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    uint8_t smask = 0;
+    const float4 ax = L.srcf[4 * (base + jj)], mu = L.srcf[4 * (base + jj) + 1];
+    float rx, ry, rz, rn, xc;
+    int kb;
+    geometry(jj, rx, ry, rz, rn, xc, kb);
+    double rp64[3];
+    point_at(L.pts, p, rp64);
+    err = slow_dipole<KIND>(s, base + jj, L.Hd + (size_t)(base + jj) * (size_t)s.Sd, (int)s.Sd, kb, xc, rx, ry, rz, rn,
+                            ax, mu.x, mu.y, L.rex, rp64, L.uf[f], L.iLd, L.r_excl, sp,
+                            &smask);
+    mask |= smask;
+    float2 Q[5];
+    pack_outputs(sp, Q);
+    flush(Q);
+  }
+  return err;
+}
+
+template <int KIND, int NF>
+__global__ void __launch_bounds__(kMixThreads, 2)
+    fields_far_kernel(const __grid_constant__ Launch L, int64_t tiles_v, int reps) {
+  __shared__ float s_anc_hi[3], s_anc_lo[3];
+  extern __shared__ float2 s_dyn[];
+  KahanFar<NF> &s_kahan = *reinterpret_cast<KahanFar<NF> *>(s_dyn);
+  __shared__ float4 s_a[kFarChunk];      // g = rho_a (x, y, z), |g|
+  __shared__ float4 s_b[kFarChunk];      // q/e p (x, y, z), |g|^2
+  __shared__ float2 s_f[NF][kFarChunk];  // the anchor's retarded sample: fraction, integer part less kFloorBits
+  __shared__ unsigned s_near[2];
+
+  const int tid = threadIdx.x;
+  const Sources &s = L.src;
+  // warps of 4 x 8 points, so that a warp's retarded samples lie close together
+  const int tr = ((tid >> 6) << 2) | ((tid >> 3) & 3), tc = ((tid >> 5) & 1) * 8 + (tid & 7);
+  const int64_t tu = blockIdx.x / tiles_v, tv = blockIdx.x % tiles_v;
+  const int64_t iuA = tu * kFarRows + tr, iuB = iuA + kFarRows / 2, iv = tv * kFarCols + tc;
+  const bool actA = iuA < L.pts.nu && iv < L.pts.nv, actB = iuB < L.pts.nu && iv < L.pts.nv;
+  const int64_t pA = iuA * L.pts.nv + iv, pB = iuB * L.pts.nv + iv;
+  if (tid == 0) tile_anchor(L, tu, tv, s_anc_hi, s_anc_lo);
+  // twice the offsets of the two points from the anchor, from whole grid steps (points past the grid's
+  // edge too: they are within the tile like the others, and only not stored)
+  const float duA = (float)(2 * tr - (kFarRows - 1)), duB = duA + (float)kFarRows;
+  const float dvv = (float)(2 * tc - (kFarCols - 1));
+  const V2 Dx(duA * L.eu_L[0] + dvv * L.ev_L[0], duB * L.eu_L[0] + dvv * L.ev_L[0]);
+  const V2 Dy(duA * L.eu_L[1] + dvv * L.ev_L[1], duB * L.eu_L[1] + dvv * L.ev_L[1]);
+  const V2 Dz(duA * L.eu_L[2] + dvv * L.ev_L[2], duB * L.eu_L[2] + dvv * L.ev_L[2]);
+  const V2 half(0.5f);
+  const V2 dr2 = V2(0.25f) * fma2(Dz, Dz, fma2(Dy, Dy, Dx * Dx));
+  int err = 0;
+  for (int rep = 0; rep < reps; ++rep) {
+    const int f0 = (blockIdx.y * reps + rep) * NF;
+    if (f0 >= L.T) break;
+    uint8_t mask[NF][2];
+#pragma unroll
+    for (int n = 0; n < NF; ++n) mask[n][0] = mask[n][1] = 0;
+#pragma unroll
+    for (int i = 0; i < 10 * NF; ++i) {
+      s_kahan[0][i][tid] = make_float2(0.f, 0.f);
+      s_kahan[1][i][tid] = make_float2(0.f, 0.f);
+    }
+    for (int base = 0; base < s.N; base += kFarChunk) {
+      const int nch = min(kFarChunk, s.N - base);
+      __syncthreads();
+      if (tid < kFarChunk) {
+        bool near = false;
+        if (tid < nch) {
+          const int j = base + tid;
+          AnchorGeo g;
+#pragma unroll
+          for (int n = 0; n < NF; ++n) {
+            g = anchor_geo(L, s_anc_hi, s_anc_lo, f0 + n, j);
+            near = near || !tile_far(L, g, j);
+            s_f[n][tid] = make_float2(g.frac, __int_as_float(g.k - kFloorBits));
+          }
+          const float4 ax = L.srcf[4 * j];
+          const ff gg = ff_mul(g.n, g.n);
+          s_a[tid] = make_float4(g.x.hi, g.y.hi, g.z.hi, g.n.hi);
+          s_b[tid] = make_float4(ax.w * ax.x, ax.w * ax.y, ax.w * ax.z, gg.hi);
+        }
+        const unsigned b = __ballot_sync(0xffffffffu, near);
+        if ((tid & 31) == 0) s_near[tid >> 5] = b;
+      }
+      __syncthreads();
+      const unsigned long long near_bits = (unsigned long long)s_near[0] | ((unsigned long long)s_near[1] << 32);
+      for (int g0 = 0; g0 < nch; g0 += 32) {
+        const unsigned skip = s_near[g0 >> 5];
+        const int gend = min(nch, g0 + 32);
+        V2 S[NF][10];  // E, B, phi, A of each frame
+#pragma unroll
+        for (int n = 0; n < NF; ++n)
+#pragma unroll
+          for (int i = 0; i < 10; ++i) S[n][i] = V2(0.f);
+        for (int jj = g0; jj < gend; ++jj) {
+          if ((skip >> (jj - g0)) & 1u) continue;
+          const float4 a = s_a[jj], b = s_b[jj];
+          // |rho|^2 - |g|^2 = 2 g.dr + dr^2, 1/|rho|, |rho| - |g| = (|rho|^2 - |g|^2) / (|rho| + |g|)
+          const V2 gx(a.x), gy(a.y), gz(a.z), px(b.x), py(b.y), pz(b.z);
+          const V2 num = fma2(gx, Dx, fma2(gy, Dy, fma2(gz, Dz, dr2)));
+          const V2 rho2 = num + V2(b.w);
+          const V2 i(rsqrt_fast(rho2.v.x), rsqrt_fast(rho2.v.y));
+          const V2 den = fma2(rho2, i, V2(a.w));
+          const V2 corr = num * V2(rcp_fast(den.v.x), rcp_fast(den.v.y));
+          // each frame's samples first, so that their loads are all in flight
+          V2 th[NF];
+          float4 h[NF][4];
+          const float4 *H = L.Hd + (size_t)(base + jj) * (size_t)s.Sd;
+#pragma unroll
+          for (int n = 0; n < NF; ++n) {
+            const float2 fr = s_f[n][jj];
+            const V2 xc = V2(fr.x) - corr;
+            const V2 y = floor_bits2(xc);
+            th[n] = xc - (y - V2(kFloorMagic));
+            const int kb = __float_as_int(fr.y);
+            const float4 *hA = H + (kb + __float_as_int(y.v.x)), *hB = H + (kb + __float_as_int(y.v.y));
+            h[n][0] = __ldg(hA);
+            h[n][1] = __ldg(hA + 1);
+            h[n][2] = __ldg(hB);
+            h[n][3] = __ldg(hB + 1);
+          }
+          const V2 rx = fma2(half, Dx, gx), ry = fma2(half, Dy, gy), rz = fma2(half, Dz, gz);
+          const V2 rp = fma2(rz, pz, fma2(ry, py, rx * px));
+          const V2 cx = fma2(py, rz, -(pz * ry)), cy = fma2(pz, rx, -(px * rz)), cz = fma2(px, ry, -(py * rx));
+          const V2 i2 = i * i, rpi2 = rp * i2, m = rpi2 * i, i3_ = V2(3.f) * i;
+#pragma unroll
+          for (int n = 0; n < NF; ++n) {
+            const float4 A0 = h[n][0], A1 = h[n][1], B0 = h[n][2], B1 = h[n][3];
+            const float tA = th[n].v.x, tB = th[n].v.y;
+            const V2 X(fmaf(tA, A1.x - A0.x, A0.x), fmaf(tB, B1.x - B0.x, B0.x));
+            const V2 V(fmaf(tA, A1.y - A0.y, A0.y), fmaf(tB, B1.y - B0.y, B0.y));
+            const V2 t1 = fma2(i, X, V);
+            V2(&o)[10] = S[n];
+            o[6] = fma2(rpi2, t1, o[6]);
+            V2 cE, cP, cB;
+            if (KIND == PC_COULOMB) {
+              cE = m * i3_ * t1;
+              cP = -(i2 * t1);
+              cB = i2 * i * V;
+            } else {
+              const V2 Ac(fmaf(tA, A1.z - A0.z, A0.z), fmaf(tB, B1.z - B0.z, B0.z));
+              if (KIND == PC_RADIATION) {
+                cE = m * Ac;
+                cP = -(i * Ac);
+                cB = i2 * Ac;
+              } else {
+                cE = m * fma2(i3_, t1, Ac);
+                cP = -(i * fma2(i, t1, Ac));
+                cB = i2 * fma2(i, V, Ac);
+              }
+            }
+            const V2 vi = V * i;
+            o[0] = fma2(cP, px, fma2(cE, rx, o[0]));
+            o[1] = fma2(cP, py, fma2(cE, ry, o[1]));
+            o[2] = fma2(cP, pz, fma2(cE, rz, o[2]));
+            o[3] = fma2(cB, cx, o[3]);
+            o[4] = fma2(cB, cy, o[4]);
+            o[5] = fma2(cB, cz, o[5]);
+            o[7] = fma2(vi, px, o[7]);
+            o[8] = fma2(vi, py, o[8]);
+            o[9] = fma2(vi, pz, o[9]);
+          }
+        }
+#pragma unroll
+        for (int n = 0; n < NF; ++n)
+#pragma unroll
+          for (int i = 0; i < 10; ++i) {
+            const float2 s0 = s_kahan[0][10 * n + i][tid], c0 = s_kahan[1][10 * n + i][tid];
+            const float2 y = __fadd2_rn(S[n][i].v, make_float2(-c0.x, -c0.y));
+            const float2 t = __fadd2_rn(s0, y);
+            const float2 d = __fadd2_rn(t, make_float2(-s0.x, -s0.y));
+            s_kahan[1][10 * n + i][tid] = __fadd2_rn(d, make_float2(-y.x, -y.y));
+            s_kahan[0][10 * n + i][tid] = t;
+          }
+      }
+      if (near_bits && !err) {
+#pragma unroll 1
+        for (int q = 0; q < 2 * NF && !err; ++q) {
+          const int lane = q & 1, n = q >> 1;
+          if (!(lane ? actB : actA)) continue;
+          const float dx = 0.5f * (lane ? Dx.v.y : Dx.v.x), dy = 0.5f * (lane ? Dy.v.y : Dy.v.x),
+                      dz = 0.5f * (lane ? Dz.v.y : Dz.v.x), d2 = lane ? dr2.v.y : dr2.v.x;
+          uint8_t mk = 0;
+          err = near_sources_far<KIND, NF>(L, f0 + n, n, base, near_bits, lane, dx, dy, dz, d2, lane ? pB : pA, s_a,
+                                           s_f[n], s_kahan, tid, mk);
+#pragma unroll
+          for (int t = 0; t < 2 * NF; ++t)
+            if (t == q) mask[t >> 1][t & 1] |= mk;
+        }
+      }
+    }
+    if (err) {
+      if (actA || actB) set_status(L.status, err);
+      err = 0;
+    }
+#pragma unroll
+    for (int n = 0; n < NF; ++n)
+      store_two_points(L, f0 + n, tid, &s_kahan[0][10 * n], &s_kahan[1][10 * n], actA, actB, pA, pB, mask[n][0],
+                       mask[n][1]);
+  }
+}
+
+// How many (tile, source, frame) triples are near, over up to kFarSample tiles spread over the grid and
+// up to four frames: far[0] += near ones, far[1] += all.
+constexpr int kFarSample = 512;
+__global__ void far_count_kernel(const __grid_constant__ Launch L, int64_t tiles, int64_t tiles_v, int n_tiles,
+                                 int n_frames, int *far) {
+  const int64_t n = (int64_t)n_tiles * n_frames * L.src.N;
+  int near = 0, all = 0;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+    const int j = (int)(t % L.src.N);
+    const int64_t r = t / L.src.N;
+    const int f = (int)((r % n_frames) * L.T / n_frames);
+    const int64_t tile = (r / n_frames) * tiles / n_tiles;
+    float hi[3], lo[3];
+    tile_anchor(L, tile / tiles_v, tile % tiles_v, hi, lo);
+    near += tile_far(L, anchor_geo(L, hi, lo, f, j), j) ? 0 : 1;
+    all += 1;
+  }
+  near = __reduce_add_sync(0xffffffffu, near);
+  all = __reduce_add_sync(0xffffffffu, all);
+  if ((threadIdx.x & 31) == 0 && all) {
+    atomicAdd(far, near);
+    atomicAdd(far + 1, all);
+  }
+}
+
+// per dipole the distance from which it is far, from the largest moments of its history
+__global__ void far_limit_kernel(int N, const unsigned *xvmax, const float4 *srcf, float rex_fast, float *rfar) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= N) return;
+  const float4 mu = srcf[4 * j + 1];
+  // not below kNearL (nearer pairs are tested for a near field that cancels), nor where a charge may
+  // lie within r_excl
+  rfar[j] = fmaxf(fmaxf(kNearL, rex_fast),
+                  far_limit(__uint_as_float(xvmax[2 * j]), __uint_as_float(xvmax[2 * j + 1]), mu.x, mu.y));
 }
 
 // ================================================================================================
@@ -1163,6 +1571,87 @@ static void launch_mixed_list(const Launch &L, dim3 grid, int kind, cudaStream_t
   if (kind == PC_TOTAL) fields_mixed_kernel<PC_TOTAL, true, kChunk><<<grid, kMixThreads, 0, st>>>(L, 1);
   else if (kind == PC_COULOMB) fields_mixed_kernel<PC_COULOMB, true, kChunk><<<grid, kMixThreads, 0, st>>>(L, 1);
   else fields_mixed_kernel<PC_RADIATION, true, kChunk><<<grid, kMixThreads, 0, st>>>(L, 1);
+}
+
+// Frames in twos, a last odd one by itself; each CTA walks as many of them as leave the grid kFarWaves
+// waves of two CTAs per SM.
+constexpr int kFarWaves = 8;
+template <int KIND, int NF>
+static cudaError_t launch_far_nf(const pc_ctx *ctx, const Launch &L, int64_t tiles, int64_t tiles_v, cudaStream_t st) {
+  const size_t smem = sizeof(KahanFar<NF>);
+  auto *fn = fields_far_kernel<KIND, NF>;
+  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int64_t groups = (L.T + NF - 1) / NF, want = (int64_t)kFarWaves * 2 * ctx->num_sms;
+  const int reps = (int)std::max<int64_t>(1, std::min<int64_t>(groups, tiles * groups / want));
+  fn<<<dim3((unsigned)tiles, (unsigned)((groups + reps - 1) / reps)), kMixThreads, smem, st>>>(L, tiles_v, reps);
+  return cudaSuccess;
+}
+template <int KIND>
+static cudaError_t launch_far_kind(const pc_ctx *ctx, const Launch &L, int64_t tiles, int64_t tiles_v, cudaStream_t st) {
+  Launch M = L;
+  M.T = L.T & ~1;
+  if (M.T) {
+    const cudaError_t e = launch_far_nf<KIND, 2>(ctx, M, tiles, tiles_v, st);
+    if (e != cudaSuccess) return e;
+  }
+  if (L.T & 1) {
+    const int k = L.T - 1;
+    M.T = 1;
+    M.frame0 = L.frame0 + k;
+    M.times[0] = L.times[k];
+    M.uf[0] = L.uf[k];
+    M.uf_hi[0] = L.uf_hi[k];
+    M.uf_lo[0] = L.uf_lo[k];
+    return launch_far_nf<KIND, 1>(ctx, M, tiles, tiles_v, st);
+  }
+  return cudaSuccess;
+}
+static cudaError_t launch_far(const pc_ctx *ctx, const Launch &L, int kind, cudaStream_t st) {
+  const int64_t tiles_v = (L.pts.nv + kFarCols - 1) / kFarCols;
+  const int64_t tiles = ((L.pts.nu + kFarRows - 1) / kFarRows) * tiles_v;
+  if (kind == PC_TOTAL) return launch_far_kind<PC_TOTAL>(ctx, L, tiles, tiles_v, st);
+  if (kind == PC_COULOMB) return launch_far_kind<PC_COULOMB>(ctx, L, tiles, tiles_v, st);
+  return launch_far_kind<PC_RADIATION>(ctx, L, tiles, tiles_v, st);
+}
+
+// Whether a mixed call of T frames may take fields_far_kernel (then far_chosen decides): plane grids
+// of dipoles alone.  Below kFarWork (point, dipole, frame) triples the whole sum takes about as long as
+// asking the device (one read-back, about 10 us).  Sets L.tile_r, the largest distance of a tile's point
+// from its anchor (c dt).
+constexpr double kFarWork = 8e6;  // fields_mixed_kernel: about 30 us
+static bool far_candidate(Launch &L, bool plane_of_dipoles, int32_t T) {
+  if (!plane_of_dipoles || (double)L.src.N * (double)L.pts.P * (double)T < kFarWork) return false;
+  double r2 = 0.0;
+  for (int sg = -1; sg <= 1; sg += 2) {
+    double q = 0.0;
+    for (int i = 0; i < 3; ++i) {
+      const double d = (0.5 * (kFarRows - 1) * L.pts.eu[i] + sg * 0.5 * (kFarCols - 1) * L.pts.ev[i]) * L.iLd;
+      q += d * d;
+    }
+    r2 = std::max(r2, q);
+  }
+  const double r = sqrt(r2) * (1.0 + 1e-6) + 1e-3;
+  if (!(r < 1e5)) return false;
+  L.tile_r = (float)r;
+  return true;
+}
+
+// The far kernel's near pairs run at half the warps of fields_mixed_kernel, its far ones several times
+// as fast: it is taken while at most kFarNearMost of the sampled (tile, source, frame) triples are near.
+constexpr double kFarNearMost = 0.4;
+static pc_status far_chosen(pc_ctx *ctx, const Launch &L, cudaStream_t st, bool *far) {
+  const int64_t tiles_v = (L.pts.nv + kFarCols - 1) / kFarCols;
+  const int64_t tiles = ((L.pts.nu + kFarRows - 1) / kFarRows) * tiles_v;
+  const int n_tiles = (int)std::min<int64_t>(tiles, kFarSample), n_frames = std::min(L.T, 4);
+  const int64_t n = (int64_t)n_tiles * n_frames * L.src.N;
+  far_count_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 608), 256, 0, st>>>(L, tiles, tiles_v, n_tiles,
+                                                                                     n_frames, ctx->d_status + 1);
+  if (cudaMemcpyAsync(ctx->h_status, ctx->d_status, 3 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return PC_ERR_CUDA;
+  *far = ctx->h_status[0] == 0 && (double)ctx->h_status[1] <= kFarNearMost * (double)ctx->h_status[2];
+  return PC_OK;
 }
 
 // Host outputs that are page-locked are mapped into the device's address space (unified
@@ -1275,6 +1764,7 @@ static pc_status fields_impl(pc_ctx *ctx, const pc_charges *ch, const pc_dipole_
   if (has_dp) check_axes_kernel<<<(unsigned)((dp->N + 255) / 256), 256, 0, st>>>(dp->axis, dp->N, L.status);
   L.tile_shift = ctx->tile_shift;
 
+  bool far_try = false, far = false;
   L.iLd = has_dp ? 1.0 / (kC * s.dtd) : 0.0;  // 1/(c dt): first guesses without a division
   L.iLc = has_ch ? 1.0 / (kC * s.dt) : 0.0;
   // dipole sample indices are 32-bit integers in both paths (the difference form's solves)
@@ -1283,8 +1773,8 @@ static pc_status fields_impl(pc_ctx *ctx, const pc_charges *ch, const pc_dipole_
     // the float32 path indexes samples with 32-bit integers
     if ((has_dp && s.Sd > (int64_t)1 << 30) || (has_ch && s.S > (int64_t)1 << 30)) return PC_ERR_ARG;
     size_t nd = has_dp ? (size_t)s.N * s.Sd : 0, nc = has_ch ? (size_t)s.M * s.S * 3 : 0;
-    const size_t ns = has_dp ? 4 * (size_t)s.N : 0;
-    if (ctx->hist_f32.reserve((nd + nc + ns) * sizeof(float4)) != cudaSuccess) return PC_ERR_CUDA;
+    const size_t ns = has_dp ? 4 * (size_t)s.N : 0, nf = has_dp ? (size_t)s.N : 0;
+    if (ctx->hist_f32.reserve((nd + nc + ns + nf) * sizeof(float4)) != cudaSuccess) return PC_ERR_CUDA;
     if (has_ch && ctx->charge_ref.reserve((size_t)s.M * 3 * sizeof(double)) != cudaSuccess) return PC_ERR_CUDA;
     float4 *Hd = (float4 *)ctx->hist_f32.ptr;
     float4 *Hc = Hd + nd;
@@ -1298,9 +1788,17 @@ static pc_status fields_impl(pc_ctx *ctx, const pc_charges *ch, const pc_dipole_
       L.eu_L[i] = (float)(L.pts.eu[i] * L.iLd);
       L.ev_L[i] = (float)(L.pts.ev[i] * L.iLd);
     }
+    far_try = far_candidate(L, !list && has_dp && !has_ch, T);
+    unsigned *xvmax = (unsigned *)(Hc + nc + ns);
+    if (far_try && cudaMemsetAsync(xvmax, 0, 2 * (size_t)s.N * sizeof(unsigned), st) != cudaSuccess) return PC_ERR_CUDA;
     if (has_dp) {
       int64_t n = (int64_t)nd;
-      prep_dipoles_f32<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(s, Hd, Hc + nc);
+      prep_dipoles_f32<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(s, Hd, Hc + nc, far_try ? xvmax : nullptr);
+    }
+    if (far_try) {
+      float *rfar = (float *)(xvmax + 2 * (size_t)s.N);
+      far_limit_kernel<<<(unsigned)((s.N + 127) / 128), 128, 0, st>>>(s.N, xvmax, L.srcf, L.rex_fast, rfar);
+      L.rfar = rfar;
     }
     if (has_ch) {
       int64_t n = (int64_t)s.M * s.S;
@@ -1333,6 +1831,10 @@ static pc_status fields_impl(pc_ctx *ctx, const pc_charges *ch, const pc_dipole_
   int chunk = 0;
   for (int32_t f0 = 0; f0 < T; f0 += step, ++chunk) {
     set_frames(L, times, f0, min(step, T - f0));
+    if (far_try && chunk == 0) {
+      const pc_status fs = far_chosen(ctx, L, st, &far);
+      if (fs != PC_OK) return fs;
+    }
     const int sl = chunk & 1;
     if (hp.on) {
       // this chunk's device slot: wait until the copy of the chunk before last has left it
@@ -1368,7 +1870,9 @@ static pc_status fields_impl(pc_ctx *ctx, const pc_charges *ch, const pc_dipole_
         tiles = tu * tiles_v;
       }
       dim3 grid((unsigned)tiles, (unsigned)L.T);
-      if (list) launch_mixed_list(L, grid, kind, st);
+      if (far) {
+        if (launch_far(ctx, L, kind, st) != cudaSuccess) return PC_ERR_CUDA;
+      } else if (list) launch_mixed_list(L, grid, kind, st);
       else if (ctx->src_chunk == 32) launch_mixed_plane<32>(L, grid, tiles_v, two, kind, st);
       else launch_mixed_plane<kChunk>(L, grid, tiles_v, two, kind, st);
     }
@@ -1561,7 +2065,7 @@ extern "C" pc_status pc_fields_noalloc(const pc_charges *ch, const pc_dipole_sou
   L.iLd = has_dp ? 1.0 / (kC * s.dtd) : 0.0;
   set_units(L);
   // the mirrors are rewritten in full by every call
-  if (has_dp) prep_dipoles_f32<<<(unsigned)((nd + 255) / 256), 256, 0, st>>>(s, Hd, srcf);
+  if (has_dp) prep_dipoles_f32<<<(unsigned)((nd + 255) / 256), 256, 0, st>>>(s, Hd, srcf, nullptr);
   if (has_ch) {
     const int64_t n = (int64_t)s.M * s.S;
     prep_charges_f32<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(s, Hc, cref);

@@ -20,6 +20,9 @@ __device__ __forceinline__ void set_status(int *st, int code) {
   if (*((volatile int *)st) == 0) atomicCAS(st, 0, code);
 }
 
+// The device status block: word 0 the status, the others counters of the call; cleared by begin_call.
+constexpr int kStatusWords = 4;
+
 // Grow-only device buffer owned by the context.
 struct Buf {
   void *ptr = nullptr;
@@ -44,7 +47,7 @@ struct Buf {
 
 struct pc_ctx {
   int device = 0;
-  int *d_status = nullptr;   // device status word
+  int *d_status = nullptr;   // device status block (kStatusWords)
   int *h_status = nullptr;   // pinned host copy
   pc::Buf hist_f32;          // float32 mirrors of source histories (mixed path)
   pc::Buf charge_ref;        // per-charge float64 reference positions

@@ -21,6 +21,7 @@
 
 #include "pc_internal.cuh"
 #include "pc_lw_f32.cuh"
+#include "pc_far_f32.cuh"
 #include "pc_lw_f64.cuh"
 #include "pc_adjoint.cuh"
 
@@ -89,6 +90,20 @@ struct RunArgs {
   // per dipole: the RK4 step as an affine map y' = M y + c1 e1 + c2 e2 + c4 e4, as
   // [B][N][kTab]: M^1 .. M^kMaxBlock (row-major 2x2 each), then c1, c2, c4
   double *rk4tab;
+  // the far form of the mixed grid path (null: not used), see lo_far_drive_kernel: per receiver, source
+  // slice z and entry t of it (source j = z + nsplit t), [B][N][nsplit][fcp], the pair's (k1, k2, k3, f)
+  // and the whole samples D of its delay D + f (kFarNear: a near pair, kFarNone: no pair); the sums
+  // carried from one causal block to the next, [nsplit][B][N]; and the last step at which some moment lay
+  // beyond the far form's limits
+  float4 *pfar;
+  int *pfarD;
+  int fcp;
+  float4 *carry;
+  int *nbad;
+  int K;              // the run's causal block length (grid path)
+  int max_reach;      // the largest reach over the batch
+  // [B][2]: largest |d0 / q| (m) and |omega0| (1/s) of a configuration (bits), for those limits
+  unsigned long long *amax;
   double e_unit;  // k_e e / (c dt)^2: the float32 driving field's unit (V/m)
   float near_L;   // mixed drive: sources whose centre is closer than this (units of c dt) go float64
 };
@@ -104,7 +119,14 @@ __host__ __device__ inline int64_t state_doubles(int64_t nbn, int64_t D) { retur
 // this GPU): gamma0, omega0^2, q^2/m, the largest charge-speed factor, 1/(q L), 1/(q c), dt/(q c),
 // m/(2 q^2), and the charges' signed offsets per unit moment m2/((m1+m2) q), -m1/((m1+m2) q)
 constexpr int kTabC = 4 * 16 + 6;
-constexpr int kTab = kTabC + 11;
+// and the moment and its rate up to which the far form's limits hold
+constexpr int kTab = kTabC + 13;
+
+// The far form's limits are set for moments up to kFarGrow times the largest initial one of the
+// configuration (and rates up to that times its omega0): a pair is far from d_max / (q kFarX) on.  A run
+// whose moments grow beyond takes the two-charge form for as long as a block can reach such a sample.
+constexpr double kFarGrow = 1.5;
+constexpr int kFarNone = -1, kFarNear = -2;
 
 constexpr int kDipF = 12;
 
@@ -173,6 +195,13 @@ __device__ void rk4_table(const RunArgs &a, size_t bi) {
   T[kTabC + 8] = m2 / (m1 + m2) / q;
   T[kTabC + 9] = -m1 / (m1 + m2) / q;
   T[kTabC + 10] = a.v_max / T[kTabC + 3];  // the largest |d'| the velocity guard allows
+  T[kTabC + 11] = T[kTabC + 12] = 0.0;
+  if (a.pfar) {
+    const unsigned long long *am = a.amax + 2 * (bi / a.N);
+    const double dmax = kFarGrow * __longlong_as_double((long long)am[0]) * q;
+    T[kTabC + 11] = dmax;
+    T[kTabC + 12] = dmax * __longlong_as_double((long long)am[1]);
+  }
 }
 
 // The kb steps of a causal block at once, one lane per step: with every stage field of the block
@@ -247,6 +276,8 @@ __device__ void rk4_block_warp(const RunArgs &a, int b, int i, int64_t n0, int k
       if (a.kdd) a.kdd[kk] = yn1;
     }
     bad = fabs(yn1) > T[kTabC + 10];
+    if (!HWCVT && a.nbad && !(fabs(yn0) <= T[kTabC + 11] && fabs(yn1) <= T[kTabC + 12]))
+      atomicMax(a.nbad, (int)(n + 1));
     if (ys && lane == kb - 1) {
       ys[0] = yn0;
       ys[1] = yn1;
@@ -974,6 +1005,7 @@ __global__ void lo_first_kernel(const RunArgs a) {
         if (k < 0) continue;
         const size_t sl = row + (k & a.wm);
         const double x = smp[3 * t], v = smp[3 * t + 1], ac = smp[3 * t + 2];
+        if (a.nbad && !(fabs(x) <= T[kTabC + 11] && fabs(v) <= T[kTabC + 12])) atomicMax(a.nbad, (int)k);
         a.d[sl] = x;
         a.dd[sl] = v;
         a.ddd[sl] = ac;
@@ -1151,6 +1183,20 @@ __global__ void lo_rstat_init_kernel(const RunArgs a) {
   a.rstat[3 * b] = 0x7f7f7f7f7f7f7f7full;
   a.rstat[3 * b + 1] = 0ull;
   a.rstat[3 * b + 2] = 0ull;
+  if (a.pfar) {
+    a.amax[2 * b] = a.amax[2 * b + 1] = 0ull;
+    if (b == 0) *a.nbad = -1;
+  }
+}
+
+// Per configuration the largest |d0 / q| and |omega0| (a.amax).  A NaN orders above every number as bits,
+// and then no pair is far.
+__global__ void lo_amax_kernel(const RunArgs a) {
+  const int64_t bi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (bi >= (int64_t)a.B * a.N) return;
+  const int64_t b = bi / a.N;
+  atomicMax(a.amax + 2 * b, (unsigned long long)__double_as_longlong(fabs(a.d0[bi] / a.q[bi])));
+  atomicMax(a.amax + 2 * b + 1, (unsigned long long)__double_as_longlong(fabs(a.omega0[bi])));
 }
 
 // Per pair (i, j) of a configuration: the centre delay |R_i - R_j| / (c dt) (the first guess of
@@ -1162,9 +1208,11 @@ __global__ void __launch_bounds__(256) lo_pairs_kernel(const RunArgs a) {
   __shared__ double s_r[256], s_v[256], s_x[256];
   const int N = a.N;
   const int64_t NN = (int64_t)N * N;
-  const double L = kC * a.dt;
+  const double L = kC * a.dt, iL = 1.0 / L;
   const int64_t H = 2 * a.n_steps + 1;
   for (int b = blockIdx.y; b < a.B; b += gridDim.y) {
+    const float xm = a.pfar ? (float)(__longlong_as_double((long long)a.amax[2 * b]) * iL) : 0.f;
+    const float vm = a.pfar ? xm * (float)(__longlong_as_double((long long)a.amax[2 * b + 1]) * a.dt) : 0.f;
     double rmin = 1e300, vmax = 0.0, rmax = 0.0;
     for (int64_t ij = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ij < NN;
          ij += (int64_t)gridDim.x * blockDim.x) {
@@ -1188,16 +1236,27 @@ __global__ void __launch_bounds__(256) lo_pairs_kernel(const RunArgs a) {
         }
         vmax = fmax(vmax, sqrt(v2max));
       }
-      const double x = r / L;
+      const double x = r * iL;
       const double fl = floor(x);
       a.delay[bi * N + j] = make_int2((int)fmin(fl, 1073741824.0), __float_as_int((float)(x - fl)));
       if (a.pgeo) {
         const double *pi_ = a.axis + 3 * bi, *pj_ = a.axis + 3 * bj;
-        const double rx = dx / L, ry = dy / L, rz = dz / L;
-        a.pgeo[bi * N + j] =
-            make_float4((float)x, (float)(rx * pj_[0] + ry * pj_[1] + rz * pj_[2]),
-                        (float)(rx * pi_[0] + ry * pi_[1] + rz * pi_[2]),
-                        (float)(pj_[0] * pi_[0] + pj_[1] * pi_[1] + pj_[2] * pi_[2]));
+        const double rx = dx * iL, ry = dy * iL, rz = dz * iL;
+        const float4 g = make_float4((float)x, (float)(rx * pj_[0] + ry * pj_[1] + rz * pj_[2]),
+                                     (float)(rx * pi_[0] + ry * pi_[1] + rz * pi_[2]),
+                                     (float)(pj_[0] * pi_[0] + pj_[1] * pi_[1] + pj_[2] * pi_[2]));
+        a.pgeo[bi * N + j] = g;
+        if (a.pfar) {
+          // p_i . E of the far form: k1 X + k2 V + k3 A
+          const float m1 = (float)a.m1[bj], m2 = (float)a.m2[bj], im = 1.f / (m1 + m2);
+          const bool far = i != j && g.x >= far_limit(xm, vm, m2 * im, m1 * im);
+          const float q = (float)(a.q[bj] * (1.0 / kE)), ir = 1.f / g.x;
+          const float cp = g.y * ir, cpi = g.z * ir;
+          const float k3 = q * ir * (cp * cpi - g.w), k2 = q * ir * ir * (3.f * cp * cpi - g.w);
+          const size_t e = (bi * a.nsplit + (size_t)(j % a.nsplit)) * a.fcp + (size_t)(j / a.nsplit);
+          a.pfar[e] = make_float4(k2 * ir, k2, k3, (float)(x - fl));
+          a.pfarD[e] = far ? (int)fmin(fl, 1073741824.0) : (i == j ? kFarNone : kFarNear);
+        }
       }
     }
     s_r[threadIdx.x] = rmin;
@@ -1255,6 +1314,202 @@ __global__ void __launch_bounds__(kRunWarps * 32) lo_drive_kernel(const RunArgs 
   drive_phase<MIXED, NEAR, RING, true, MOV>(a, b, i, n0, ns, sh[warp], &err, j_lo, j_hi,
                                        dst + bidx(a, b, i) * (2 * kMaxBlock + 1));
   if (err) set_status(a.status, err);
+}
+
+
+// ------------------------------------------------------------------------------------------------
+// Grid path, phase A of the mixed drive in the far form (pc_far_f32.cuh).  With fixed origins the
+// projected field of a far pair is the constant combination g = k1 X + k2 V + k3 A of its source's
+// samples, interpolated at delays D + f that are constant too, so the K steps of a causal block need
+// K + 2 consecutive values of g per pair and three operations for each, and their interpolation to the
+// 2 K stage times is applied once, to the sums over the sources:
+//   with n = n0 - D - 1 + p the sample at position p, step t (times n0 + t + 1/2 and n0 + t + 1) takes
+//   half  = H0[t] + H1[t+1] + H2[t+2],  H0 = sum w0 g, H1 = sum (1 - w0 - w2) g, H2 = sum w2 g,
+//   whole = F[t+1] + (G - F)[t+2],      F = sum f g, G = sum g,   w0 = max(f - 1/2, 0), w2 = max(1/2 - f, 0)
+// (linear interpolation between samples, Sec. 3.1).  Positions K and K + 1 are positions 0 and 1 of the
+// next block, whose four sums they enter are carried over, so that a block reads K new samples per pair:
+// half a warp takes a source, lanes = positions 2 .. 17.
+// Sources that are not far go through pair_drive_f32 with lanes = stages, as in lo_drive_kernel; a far
+// source whose samples cross t = 0 in this block (the rest state before it has a kink there, which the
+// two charges' retarded times meet apart) is corrected by the difference of the two forms.
+// A block whose reach holds a sample beyond the limits (a.nbad) goes through lo_drive_kernel's sources
+// altogether; the next far block then forms the carried sums itself.
+// Measured, 4096 oscillators in a 600 nm cube: 3.10 -> 0.55 ms a block of 16 steps, about 10 warp
+// instructions per pair and block against 179; bound by the gathers of the samples (the pair tables alone,
+// 20 B a pair, take 0.05 ms from HBM).  A ring of 256: 21 -> 11.6 us a block, launch included.
+// ------------------------------------------------------------------------------------------------
+struct FarSums {
+  float G, H0, H2, F;
+};
+// The far sources of slice z (table rows from tab), samples at positions 2 + m + shift (m = lane & 15) of
+// the block at n0: sums per position over the slice's sources, groups of 32 compensated.  A slice takes
+// every nsplit-th source, so that the near ones, neighbours in index as often as not, spread over them.
+template <bool RING>
+__device__ __forceinline__ FarSums far_sources(const RunArgs &a, size_t b0, size_t tab, int z, int n0, int shift,
+                                               float4 *s_k, int2 *s_j) {
+  const int lane = threadIdx.x & 31, half = lane >> 4;
+  const char *H = reinterpret_cast<const char *>(a.H32 + b0 * (size_t)a.hs);
+  const unsigned hb = (unsigned)a.hs * 16u;  // a.hs < 2^27 (the host's condition)
+  const int mask = RING ? (int)a.wm : -1;
+  const int pos = 2 + (lane & 15) + shift;
+  FarSums S = {0.f, 0.f, 0.f, 0.f}, C = {0.f, 0.f, 0.f, 0.f};
+  for (int t0 = 0; t0 < a.fcp; t0 += 32) {
+    const int t = t0 + lane;
+    float4 pk = make_float4(0.f, 0.f, 0.f, 0.f);
+    int D = kFarNone;
+    if (t < a.fcp) {
+      D = a.pfarD[tab + t];
+      pk = a.pfar[tab + t];
+    }
+    const bool far = D >= 0;
+    const unsigned mf = __ballot_sync(0xffffffffu, far);
+    const int cnt = __popc(mf);
+    __syncwarp();
+    if (far) {
+      const int sl = __popc(mf & ((1u << lane) - 1u));
+      s_k[sl] = pk;
+      s_j[sl] = make_int2(z + a.nsplit * t, n0 - D - 1);
+    }
+    if ((cnt & 1) && lane == 31) {  // an even count: a source of no weight
+      s_k[cnt] = make_float4(0.f, 0.f, 0.f, 0.f);
+      s_j[cnt] = make_int2(z, 0);
+    }
+    __syncwarp();
+    FarSums g = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int e = half; e < cnt; e += 2) {
+      const float4 k = s_k[e];
+      const int2 r = s_j[e];
+      const unsigned n = (unsigned)(max(r.y + pos, 0) & mask);
+      const float4 h = *reinterpret_cast<const float4 *>(H + (size_t)(unsigned)r.x * hb + 16u * n);
+      const float v = fmaf(k.z, h.z, fmaf(k.y, h.y, k.x * h.x));
+      g.G += v;
+      g.H0 = fmaf(__saturatef(k.w - 0.5f), v, g.H0);
+      g.H2 = fmaf(__saturatef(0.5f - k.w), v, g.H2);
+      g.F = fmaf(k.w, v, g.F);
+    }
+    auto add = [](float &s, float &c, float x) {
+      const float y = x - c, t = s + y;
+      c = (t - s) - y;
+      s = t;
+    };
+    add(S.G, C.G, g.G);
+    add(S.H0, C.H0, g.H0);
+    add(S.H2, C.H2, g.H2);
+    add(S.F, C.F, g.F);
+  }
+  // the two halves' sources
+  S.G += __shfl_xor_sync(0xffffffffu, S.G, 16);
+  S.H0 += __shfl_xor_sync(0xffffffffu, S.H0, 16);
+  S.H2 += __shfl_xor_sync(0xffffffffu, S.H2, 16);
+  S.F += __shfl_xor_sync(0xffffffffu, S.F, 16);
+  return S;
+}
+
+template <bool NEAR, bool RING>
+__global__ void __launch_bounds__(kRunWarps * 32) lo_far_drive_kernel(const __grid_constant__ RunArgs a, int64_t n0_, int ns_) {
+  __shared__ double sh[kRunWarps][32];
+  __shared__ float4 s_k[kRunWarps][34];
+  __shared__ int2 s_j[kRunWarps][34];
+  if (*((volatile int *)a.status)) return;  // an earlier block failed
+  int64_t n0l = n0_;
+  int ns = ns_;
+  if (ns < 0) {
+    n0l = a.blk[0];
+    if (n0l >= a.n_steps) return;
+    ns = 2 * (int)min((int64_t)a.K, a.n_steps - n0l);
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int b = blockIdx.y;
+  const int i = blockIdx.x * kRunWarps + warp;
+  if (i >= a.N) return;
+  const int z = blockIdx.z;
+  const size_t bi = bidx(a, b, i), b0 = bidx(a, b, 0);
+  double *dst = (a.nsplit > 1 ? a.Epart + (size_t)z * a.B * a.N * (2 * kMaxBlock + 1) : a.Es) + bi * (2 * kMaxBlock + 1);
+  const int n0 = (int)n0l, K = a.K;
+  int err = 0;
+  // (the reach is the depth of a run state too, so that a resumed run decides as the uninterrupted one)
+  const int nbad = *((volatile int *)a.nbad), back = a.max_reach;
+  if (nbad >= 0 && n0 - back <= nbad) {
+    const int j_lo = min(a.N, z * a.fcp), j_hi = min(a.N, j_lo + a.fcp);
+    drive_phase<true, NEAR, RING, true, false>(a, b, i, n0l, ns, sh[warp], &err, j_lo, j_hi, dst);
+    if (err) set_status(a.status, err);
+    return;
+  }
+  const size_t row = bi * (size_t)a.N, tab = (bi * a.nsplit + z) * (size_t)a.fcp;
+  // positions 0 and 1: carried from the block before, or formed here (a first block, or after one that
+  // went through the other form) as positions K and K + 1 of that block
+  float4 *cw = a.carry + ((size_t)z * a.B + b) * (size_t)a.N + i;
+  float4 c;
+  if (n0l == a.n_begin || (nbad >= 0 && n0 - K - back <= nbad)) {
+    const FarSums P = far_sources<RING>(a, b0, tab, z, n0, -K, s_k[warp], s_j[warp]);
+    const float h1 = P.G - P.H0 - P.H2;
+    c = make_float4(__shfl_sync(0xffffffffu, P.H0, K - 2), __shfl_sync(0xffffffffu, P.H0, K - 1),
+                    __shfl_sync(0xffffffffu, h1, K - 1), __shfl_sync(0xffffffffu, P.F, K - 1));
+  } else {
+    c = *cw;
+  }
+  const FarSums S = far_sources<RING>(a, b0, tab, z, n0, 0, s_k[warp], s_j[warp]);
+  const float h1 = S.G - S.H0 - S.H2;
+  {
+    const float4 cn = make_float4(__shfl_sync(0xffffffffu, S.H0, K - 2), __shfl_sync(0xffffffffu, S.H0, K - 1),
+                                  __shfl_sync(0xffffffffu, h1, K - 1), __shfl_sync(0xffffffffu, S.F, K - 1));
+    if (lane == 0) *cw = cn;
+  }
+  // the other sources, lane = stage s (time n0 + (s + 1) / 2)
+  float accf = 0.f, comp = 0.f;
+  double accd = 0.0;
+  const float stage_f = 0.5f * (__int_as_float(0x4B000000 | (lane + 1)) - 8388608.f);
+  for (int t0 = 0; t0 < a.fcp; t0 += 32) {
+    const int D = t0 + lane < a.fcp ? a.pfarD[tab + t0 + lane] : kFarNone;
+    const int kb = n0 - D - 1;
+    const bool near = D == kFarNear, wave = D >= 0 && kb <= 1 && kb + K + 2 >= 0;
+    const unsigned mn = __ballot_sync(0xffffffffu, near), mw = __ballot_sync(0xffffffffu, wave);
+    float grp = 0.f;
+    for (unsigned m = mn | mw; m; m &= m - 1) {
+      const int l = __ffs((int)m) - 1, j = z + a.nsplit * (t0 + l);
+      if (lane >= ns) continue;
+      const int2 dl = a.delay[row + j];
+      const float4 geo = a.pgeo[row + j];
+      const float xs = stage_f - __int_as_float(dl.y);
+      float flf;
+      const int fl = Num<float>::floor_int(xs, flf);
+      const int k = n0 - dl.x + fl;
+      const float th = xs - flf;
+      if (NEAR && geo.x < a.near_L) {
+        accd += pair_drive_f64(a, b, i, j, (double)n0 + (double)stage_f, n0, k, &err, 0, 2);
+        if (!((mw >> l) & 1u)) continue;
+      } else {
+        grp += pair_drive_f32<RING>(a, b, i, j, k, th, geo, n0 + 1, &err);
+      }
+      if ((mw >> l) & 1u) {
+        const float4 *hj = a.H32 + (b0 + (size_t)j) * (size_t)a.hs;
+        const int mask = RING ? (int)a.wm : -1;
+        const float4 h0 = hj[max(k, 0) & mask], h1_ = hj[max(k + 1, 0) & mask], pk = a.pfar[tab + t0 + l];
+        const float v0 = fmaf(pk.z, h0.z, fmaf(pk.y, h0.y, pk.x * h0.x));
+        const float v1 = fmaf(pk.z, h1_.z, fmaf(pk.y, h1_.y, pk.x * h1_.x));
+        grp -= fmaf(th, v1 - v0, v0);
+      }
+    }
+    const float y = grp - comp;
+    const float t = accf + y;
+    comp = (t - accf) - y;
+    accf = t;
+  }
+  if (err) set_status(a.status, err);
+  // step t = lane (< 16): its two stage fields
+  const int t = lane & 15;
+  const float H0u = __shfl_up_sync(0xffffffffu, S.H0, 2), H1u = __shfl_up_sync(0xffffffffu, h1, 1),
+              Fu = __shfl_up_sync(0xffffffffu, S.F, 1);
+  const float h0 = t == 0 ? c.x : (t == 1 ? c.y : H0u), hm = t == 0 ? c.z : H1u, fm = t == 0 ? c.w : Fu;
+  const float eh = (h0 + hm) + S.H2 + __shfl_sync(0xffffffffu, accf, 2 * t);
+  const float ew = fm + (S.G - S.F) + __shfl_sync(0xffffffffu, accf, 2 * t + 1);
+  const double dh = NEAR ? __shfl_sync(0xffffffffu, accd, 2 * t) : 0.0;
+  const double dw = NEAR ? __shfl_sync(0xffffffffu, accd, 2 * t + 1) : 0.0;
+  if (lane < 16 && 2 * t < ns) {
+    dst[1 + 2 * t] = (double)eh * a.e_unit + dh;
+    dst[2 + 2 * t] = (double)ew * a.e_unit + dw;
+  }
 }
 
 // Sum of the slices' partial stage fields (fixed order) into Es[lo..hi].
@@ -1849,6 +2104,14 @@ static void *drive_kernel_for(const RunArgs &a, bool mixed) {
     return ring ? (void *)lo_drive_kernel<true, true, true> : (void *)lo_drive_kernel<true, true, false>;
   return ring ? (void *)lo_drive_kernel<true, false, true> : (void *)lo_drive_kernel<true, false, false>;
 }
+// the block loop's drive: the far form where the run has its tables
+static void *block_drive_kernel_for(const RunArgs &a, bool mixed) {
+  if (!a.pfar) return drive_kernel_for(a, mixed);
+  const bool ring = a.wm >= 0;
+  if (a.near_L > 0.f)
+    return ring ? (void *)lo_far_drive_kernel<true, true> : (void *)lo_far_drive_kernel<true, false>;
+  return ring ? (void *)lo_far_drive_kernel<false, true> : (void *)lo_far_drive_kernel<false, false>;
+}
 static void *run_kernel_for(const RunArgs &a, bool mixed) {
   if (!mixed) return (void *)lo_run_kernel<false>;
   if (a.org_pos) return (void *)lo_run_kernel<true, false, false, true>;
@@ -1912,7 +2175,7 @@ static pc_status launch_block_loop(pc_ctx *ctx, const RunArgs &a, bool mixed, di
   cudaKernelNodeParams kp;
   memset(&kp, 0, sizeof(kp));
   cudaGraphNode_t n1, n2, n3;
-  kp.func = drive_kernel_for(a, mixed);
+  kp.func = block_drive_kernel_for(a, mixed);
   kp.gridDim = dgrid;
   kp.blockDim = dim3(kRunWarps * 32);
   kp.kernelParams = drive_args;
@@ -2032,7 +2295,21 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   const size_t part_off = k_off + k_bytes, blk_off = part_off + part_bytes, tab_off = blk_off + blk_bytes;
   const size_t geo_off = tab_off + tab_bytes, rs_off = geo_off + geo_bytes;
   const size_t od_off = rs_off + rs_bytes, od_bytes = motion ? al(nbn * sizeof(double)) : 0;
-  if (ctx->run_scratch.reserve(od_off + od_bytes) != cudaSuccess) return PC_ERR_CUDA;
+  // the far form's tables (mixed grid path with fixed origins); without the memory for them the run
+  // takes the two-charge form throughout
+  // eight source slices per receiver (4096 oscillators, 1000 steps: 49, 41, 37, 37, 39 and 44 ms with 2, 4,
+  // 8, 16, 32 and 64; 1024: 5.3, 5.0, 4.45, 4.5, 5.0 with 2, 4, 8, 16 and 32), or as set or tuned
+  const int far_split = std::min(kMaxSplit, std::min(ctx->run_slices > 0 ? ctx->run_slices : 8, std::max(1, dp->N / 8)));
+  const int far_cp = (dp->N + far_split - 1) / far_split;
+  const size_t far_n = nbn * (size_t)far_split * far_cp;
+  const size_t far_off = od_off + od_bytes, pf_bytes = al(far_n * sizeof(float4)), pd_bytes = al(far_n * sizeof(int));
+  const size_t cr_bytes = al((size_t)pc::kMaxSplit * nbn * sizeof(float4)), am_bytes = al(2 * (size_t)dp->B * sizeof(double));
+  bool far = mixed && grid && !motion;
+  if (far && ctx->run_scratch.reserve(far_off + pf_bytes + pd_bytes + cr_bytes + am_bytes + 256) != cudaSuccess) {
+    cudaGetLastError();
+    far = false;
+  }
+  if (!far && ctx->run_scratch.reserve(far_off) != cudaSuccess) return PC_ERR_CUDA;
   char *scr = (char *)ctx->run_scratch.ptr;
   pc::RunArgs a;
   memset(&a, 0, sizeof(a));
@@ -2068,6 +2345,18 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   a.org_vel = motion ? motion->vel : nullptr;
   a.org_acc = motion ? motion->acc : nullptr;
   a.odisp = motion ? (double *)(scr + od_off) : nullptr;
+  if (far) {
+    char *f = scr + far_off;
+    a.pfar = (float4 *)f;
+    a.pfarD = (int *)(f + pf_bytes);
+    a.carry = (float4 *)(f + pf_bytes + pd_bytes);
+    a.amax = (unsigned long long *)(f + pf_bytes + pd_bytes + cr_bytes);
+    a.nbad = (int *)(f + pf_bytes + pd_bytes + cr_bytes + am_bytes);
+    a.fcp = far_cp;
+    a.nsplit = far_split;
+    // entries past the last source stay kFarNone
+    if (cudaMemsetAsync(a.pfarD, 0xff, far_n * sizeof(int), st) != cudaSuccess) return PC_ERR_CUDA;
+  }
   a.status = ctx->d_status;
   if (pl.delay_out) *pl.delay_out = a.delay;
   if (pl.rk4tab_out) *pl.rk4tab_out = a.rk4tab;
@@ -2077,6 +2366,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
     const unsigned gx = (unsigned)std::min<int64_t>((NN + 255) / 256, 2048);
     const unsigned gy = (unsigned)std::min(dp->B, 65535);
     pc::lo_rstat_init_kernel<<<(dp->B + 255) / 256, 256, 0, st>>>(a);
+    if (far) pc::lo_amax_kernel<<<(unsigned)((nbn + 255) / 256), 256, 0, st>>>(a);
     if (motion) pc::lo_origin_disp_kernel<<<(unsigned)std::min<size_t>((nbn + 127) / 128, 4096), 128, 0, st>>>(a);
     pc::lo_pairs_kernel<<<dim3(gx, gy), 256, 0, st>>>(a);
     if (motion) pc::lo_closest_kernel<<<dim3(gx, gy), 256, 0, st>>>(a);
@@ -2127,6 +2417,12 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   char *sto = (char *)ctx->run_store.ptr;
   a.hs = hs;
   a.wm = wm;
+  a.K = K;
+  a.max_reach = (int)std::min<int64_t>(D, (int64_t)1 << 29);
+  if (K < 2 || hs >= ((int64_t)1 << 27)) {  // (the carried sums sit in lanes K - 2 and K - 1)
+    a.pfar = nullptr;
+    a.nbad = nullptr;
+  }
   if (full_store) {
     a.d = out->d;
     a.dd = out->d_dot;
@@ -2192,7 +2488,9 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
     const int64_t target = (int64_t)ctx->num_sms * 64;
     int nsplit = (int)std::min<int64_t>(std::max<int64_t>(1, (target + (int64_t)nbn - 1) / (int64_t)nbn),
                                         std::max(1, dp->N / 8));
-    if (ctx->run_slices > 0) {
+    if (a.pfar) {
+      nsplit = far_split;  // the tables' slices
+    } else if (ctx->run_slices > 0) {
       nsplit = std::min(ctx->run_slices, std::max(1, dp->N / 8));  // set or tuned
     } else if (motion && mixed) {
       // the moving mixed drive holds about twice the registers of the fixed one (two CTAs per SM
@@ -2230,7 +2528,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
         for (int64_t n0 = n_begin; n0 < n_end; n0 += K) {
           const int kb = (int)std::min<int64_t>(K, n_end - n0);
           if (timed) cudaEventRecord(ctx->tev[nev++], st);
-          pc::launch_drive(drive, dgrid, a, n0, 2 * kb, st);
+          pc::launch_drive(pc::block_drive_kernel_for(a, mixed), dgrid, a, n0, 2 * kb, st);
           if (timed) cudaEventRecord(ctx->tev[nev++], st);
           const unsigned wgrid = (unsigned)((nbn * 32 + 127) / 128);
           if (mixed) pc::lo_rk4_kernel<true><<<wgrid, 128, 0, st>>>(a, n0, kb);

@@ -93,3 +93,86 @@ def test_exclusion_radius_beyond_the_far_distance(ctx):
 def test_coarse_grid_tiles_are_never_wholly_far(ctx):
     # grid steps of 40 nm: a tile spans more than a micrometre
     _check(ctx, _sources(64), 401, 403, [11.4e-15], step=4e-8)
+
+
+# ------------------------------------------------------------------------------------------------
+# the oscillator run's far drive (grid path, mixed)
+# ------------------------------------------------------------------------------------------------
+def _cloud(N, cell=37.5e-9, seed=11, ring=False, B=1):
+    """N oscillators, one in each of N lattice cells (no two closer than 5 nm)."""
+    rng = np.random.default_rng(seed)
+    g = int(math.ceil(N ** (1 / 3) - 1e-9))
+    org, ax = [], []
+    for _ in range(B):
+        c = np.stack(np.unravel_index(rng.permutation(g ** 3)[:N], (g, g, g)), axis=1)
+        org.append(c * cell + rng.uniform(0.0, cell - 5e-9, (N, 3)))
+        ax.append(W.unit_vectors(rng, N))
+    return W.lo_batch(np.array(org), np.array(ax), OMEGA0, 1e-11, 1e-18, 0, 0)
+
+
+def _err(a, b):
+    return float(((a - b).abs().amax(-1) / b.abs().amax()).max())
+
+
+@pytest.mark.parametrize("N,steps", [(65, 700), (96, 333), (130, 400), (257, 203)])
+def test_far_drive_against_oracle(ctx, N, steps):
+    # past the light-crossing time of the cloud, so that pairs have been static, crossing t = 0 and moving;
+    # a last block of fewer than 16 steps; slices that do not divide the sources
+    cfg = _cloud(N)
+    cfg.n_steps = steps
+    ref = oracle.dipoles_run(cfg)
+    assert ref["status"] == oracle.OK
+    out = pc.pc_dipoles_run(ctx, pc.lo_config_to_device(cfg), cfg.dt, steps, precision=pc.PC_MIXED, want_Ed=True)
+    for k in ("d", "d_dot", "Ed"):
+        g = out[k][0].cpu().numpy()
+        assert np.max(np.abs(g - ref[k])) < 1e-5 * np.max(np.abs(ref[k])), k
+
+
+@pytest.mark.parametrize("slices", [0, 1, 3, 12])
+@pytest.mark.parametrize("spacing,near", [(1.0, 0.0), (0.5, 0.0), (1.0, 60e-9), (40.0, 0.0)])
+def test_far_drive_against_float64(ctx, slices, spacing, near):
+    # the float64 run's driving fields within 3e-6 of their largest value (float32 sums of some hundred
+    # terms of 1e-7 each); blocks shorter than 16 steps (spacing 0.5: origins down to 2.5 nm, 7 steps),
+    # near sources in float64, and a cloud that stays static for the whole run
+    cfg = _cloud(100, B=2)
+    cfg.origin *= spacing
+    lod = pc.lo_config_to_device(cfg)
+    f = pc.pc_dipoles_run(ctx, lod, cfg.dt, 450, precision=pc.PC_F64, want_Ed=True)
+    try:
+        pc.pc_set_run_tiling(ctx, slices)
+        m = pc.pc_dipoles_run(ctx, lod, cfg.dt, 450, precision=pc.PC_MIXED, near_f64=near, want_Ed=True)
+    finally:
+        pc.pc_set_run_tiling(ctx, 0)
+    assert _err(m["Ed"], f["Ed"]) < 3e-6
+    assert _err(m["d"], f["d"]) < 1e-9
+
+
+def test_far_drive_leaves_and_returns_where_moments_pass_its_limits(ctx):
+    # a state whose oldest samples are three times the largest initial moment (beyond the limits): the
+    # resumed run's first blocks take the two-charge form, the later ones the far form with its carried
+    # sums formed anew; the float64 run resumed from the same state is the reference
+    cfg = _cloud(80)
+    lod = pc.lo_config_to_device(cfg)
+    n = pc.pc_dipoles_state_size(ctx, lod, cfg.dt)
+    state = torch.zeros(n, dtype=torch.float64, device="cuda")
+    first = 960  # a whole number of blocks, beyond the state's depth
+    pc.pc_dipoles_run(ctx, lod, cfg.dt, first, precision=pc.PC_F64, state_out=state)
+    D = int(state[2])
+    assert D < first
+    state[4 + 80:].view(80, D + 1, 3)[:, :20] *= 3.0
+    f = pc.pc_dipoles_run(ctx, lod, cfg.dt, 200, precision=pc.PC_F64, state_in=state, want_Ed=True)
+    m = pc.pc_dipoles_run(ctx, lod, cfg.dt, 200, precision=pc.PC_MIXED, state_in=state, want_Ed=True)
+    assert _err(m["Ed"], f["Ed"]) < 3e-6
+    assert _err(m["d"], f["d"]) < 1e-9
+    # and amplitudes that the limits of smaller declared moments forbid throughout
+    small = pc.lo_config_to_device(cfg)
+    small.d0 *= 0.1
+    m = pc.pc_dipoles_run(ctx, small, cfg.dt, 200, precision=pc.PC_MIXED, state_in=state, want_Ed=True)
+    assert _err(m["Ed"], f["Ed"]) < 3e-6
+
+
+def test_far_drive_refuses_what_is_not_a_number(ctx):
+    cfg = _cloud(80)
+    cfg.omega0[0, 7] = np.nan
+    with pytest.raises(pc.PcError):
+        pc.pc_dipoles_run(ctx, pc.lo_config_to_device(cfg), cfg.dt, 400, precision=pc.PC_MIXED)

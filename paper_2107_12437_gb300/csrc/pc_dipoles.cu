@@ -32,6 +32,10 @@ constexpr int kMaxBlock = 16;  // steps per causal block (2K <= 32 stages, one p
 constexpr int kSmallN = 64;    // configurations up to this size run as one persistent CTA each
 constexpr int kMaxSplit = 64;  // source slices per receiver on the grid path
 
+struct alignas(32) FarK64 {
+  double x, y, z, w;
+};
+
 struct RunArgs {
   int B, N;
   const double *origin, *axis, *q, *m1, *m2, *omega0, *d0;
@@ -98,7 +102,9 @@ struct RunArgs {
   float4 *pfar;
   int *pfarD;
   int fcp;
+  FarK64 *pfar64;     // the float64 drive's (k1, k2, k3, f) instead of pfar (pc_far_f32.cuh: the split form)
   float4 *carry;
+  double *carry64;    // the float64 drive's, four each
   int *nbad;
   int K;              // the run's causal block length (grid path)
   int max_reach;      // the largest reach over the batch
@@ -127,6 +133,7 @@ constexpr int kTab = kTabC + 13;
 // whose moments grow beyond takes the two-charge form for as long as a block can reach such a sample.
 constexpr double kFarGrow = 1.5;
 constexpr int kFarNone = -1, kFarNear = -2;
+constexpr double kFarDelay = 16 + 4;  // samples: a block of kMaxBlock steps reads well behind the newest one
 
 constexpr int kDipF = 12;
 
@@ -196,7 +203,7 @@ __device__ void rk4_table(const RunArgs &a, size_t bi) {
   T[kTabC + 9] = -m1 / (m1 + m2) / q;
   T[kTabC + 10] = a.v_max / T[kTabC + 3];  // the largest |d'| the velocity guard allows
   T[kTabC + 11] = T[kTabC + 12] = 0.0;
-  if (a.pfar) {
+  if (a.pfarD) {
     const unsigned long long *am = a.amax + 2 * (bi / a.N);
     const double dmax = kFarGrow * __longlong_as_double((long long)am[0]) * q;
     T[kTabC + 11] = dmax;
@@ -1183,7 +1190,7 @@ __global__ void lo_rstat_init_kernel(const RunArgs a) {
   a.rstat[3 * b] = 0x7f7f7f7f7f7f7f7full;
   a.rstat[3 * b + 1] = 0ull;
   a.rstat[3 * b + 2] = 0ull;
-  if (a.pfar) {
+  if (a.pfarD) {
     a.amax[2 * b] = a.amax[2 * b + 1] = 0ull;
     if (b == 0) *a.nbad = -1;
   }
@@ -1211,8 +1218,9 @@ __global__ void __launch_bounds__(256) lo_pairs_kernel(const RunArgs a) {
   const double L = kC * a.dt, iL = 1.0 / L;
   const int64_t H = 2 * a.n_steps + 1;
   for (int b = blockIdx.y; b < a.B; b += gridDim.y) {
-    const float xm = a.pfar ? (float)(__longlong_as_double((long long)a.amax[2 * b]) * iL) : 0.f;
-    const float vm = a.pfar ? xm * (float)(__longlong_as_double((long long)a.amax[2 * b + 1]) * a.dt) : 0.f;
+    const double xd = a.pfarD ? __longlong_as_double((long long)a.amax[2 * b]) * iL : 0.0;
+    const float xm = a.pfarD ? (float)(__longlong_as_double((long long)a.amax[2 * b]) * iL) : 0.f;
+    const float vm = a.pfarD ? xm * (float)(__longlong_as_double((long long)a.amax[2 * b + 1]) * a.dt) : 0.f;
     double rmin = 1e300, vmax = 0.0, rmax = 0.0;
     for (int64_t ij = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ij < NN;
          ij += (int64_t)gridDim.x * blockDim.x) {
@@ -1246,14 +1254,28 @@ __global__ void __launch_bounds__(256) lo_pairs_kernel(const RunArgs a) {
                                      (float)(rx * pi_[0] + ry * pi_[1] + rz * pi_[2]),
                                      (float)(pj_[0] * pi_[0] + pj_[1] * pi_[1] + pj_[2] * pi_[2]));
         a.pgeo[bi * N + j] = g;
+        const size_t e =
+            a.pfarD ? (bi * a.nsplit + (size_t)(j % a.nsplit)) * a.fcp + (size_t)(j / a.nsplit) : (size_t)0;
+        if (a.pfar64) {
+          // p_i . E of the split form's linear part, with the charge's unit and the samples' scales:
+          // k1 d + k2 d' + k3 d'' is the field in V/m
+          const bool far = i != j && fl >= kFarDelay && a.m1[bj] == a.m2[bj] && xd <= kSplitX * x &&
+                           xd * __longlong_as_double((long long)a.amax[2 * b + 1]) * a.dt <= kSplitV;
+          const double ir = 1.0 / r, c1 = (dx * pj_[0] + dy * pj_[1] + dz * pj_[2]) * ir,
+                       c2 = (dx * pi_[0] + dy * pi_[1] + dz * pi_[2]) * ir,
+                       c12 = pj_[0] * pi_[0] + pj_[1] * pi_[1] + pj_[2] * pi_[2];
+          const double k3 = kKe * ir * (c1 * c2 - c12) * (1.0 / (kC * kC));
+          const double k2 = kKe * ir * ir * (3.0 * c1 * c2 - c12);
+          a.pfar64[e] = {k2 * ir, k2 * (1.0 / kC), k3, x - fl};
+          a.pfarD[e] = far ? (int)fmin(fl, 1073741824.0) : (i == j ? kFarNone : kFarNear);
+        }
         if (a.pfar) {
           // p_i . E of the far form: k1 X + k2 V + k3 A
           const float m1 = (float)a.m1[bj], m2 = (float)a.m2[bj], im = 1.f / (m1 + m2);
-          const bool far = i != j && g.x >= far_limit(xm, vm, m2 * im, m1 * im);
+          const bool far = i != j && fl >= kFarDelay && g.x >= far_limit(xm, vm, m2 * im, m1 * im);
           const float q = (float)(a.q[bj] * (1.0 / kE)), ir = 1.f / g.x;
           const float cp = g.y * ir, cpi = g.z * ir;
           const float k3 = q * ir * (cp * cpi - g.w), k2 = q * ir * ir * (3.f * cp * cpi - g.w);
-          const size_t e = (bi * a.nsplit + (size_t)(j % a.nsplit)) * a.fcp + (size_t)(j / a.nsplit);
           a.pfar[e] = make_float4(k2 * ir, k2, k3, (float)(x - fl));
           a.pfarD[e] = far ? (int)fmin(fl, 1073741824.0) : (i == j ? kFarNone : kFarNear);
         }
@@ -1509,6 +1531,220 @@ __global__ void __launch_bounds__(kRunWarps * 32) lo_far_drive_kernel(const __gr
   if (lane < 16 && 2 * t < ns) {
     dst[1 + 2 * t] = (double)eh * a.e_unit + dh;
     dst[2 + 2 * t] = (double)ew * a.e_unit + dw;
+  }
+}
+
+
+// ------------------------------------------------------------------------------------------------
+// The same for the float64 drive, in the split form (pc_far_f32.cuh): the linear part as in
+// lo_far_drive_kernel in float64 on the float64 history, and the cubic terms, smaller by (X/R)^2, in
+// float32 with lanes = stages on the history's float32 mirror.  Where a charge's own retarded time falls
+// just outside the segment of the centre's (by o samples, at most half its offset), its state differs from
+// that segment's extension by o times the second difference of the samples: that term in float64.  Sources
+// crossing t = 0, where the second difference is not small, are corrected by the difference of
+// pair_drive_f64 and the linear part instead.
+// Measured: a cloud of 1000 oscillators, 320 steps 316 -> 12.7 ms, a ring of 256, 1000 steps 63.4 -> 7.0 ms.  A
+// far pair costs 7 float64 instructions per two of them and 16 positions and about 170 float32 ones per 32
+// stages, a near one about 280 float64 ones per 32 stages: the ring is bound by its 10 near pairs a
+// receiver.  E_d against binary128 on a cloud of 400: 1.4e-12 rms (3.9e-12 with two charges throughout).
+// ------------------------------------------------------------------------------------------------
+struct FarSums64 {
+  double G, H0, H2, F;
+};
+struct FarEntry64 {
+  double k1, k2, k3, f, w0, w2;
+};
+template <bool RING>
+__device__ __forceinline__ void far_group64(const RunArgs &a, size_t b0, int cnt, int pos, const FarEntry64 *s_k,
+                                            const int2 *s_j, FarSums64 &S) {
+  const int half = (threadIdx.x & 31) >> 4;
+  const int64_t wm = RING ? a.wm : -1;
+#pragma unroll 2
+  for (int e = half; e < cnt; e += 2) {
+    const FarEntry64 &k = s_k[e];
+    const int2 r = s_j[e];
+    const size_t n = (b0 + (size_t)r.x) * (size_t)a.hs + (size_t)((int64_t)max(r.y + pos, 0) & wm);
+    const double v = fma(k.k3, a.ddd[n], fma(k.k2, a.dd[n], k.k1 * a.d[n]));
+    S.G += v;
+    S.H0 = fma(k.w0, v, S.H0);
+    S.H2 = fma(k.w2, v, S.H2);
+    S.F = fma(k.f, v, S.F);
+  }
+}
+// the table's entries t0 .. t0 + 31 of a slice that are far, into shared memory; returns their number
+__device__ __forceinline__ int far_stage64(const RunArgs &a, size_t tab, int z, int t0, int n0, FarEntry64 *s_k, int2 *s_j,
+                                           int &D) {
+  const int lane = threadIdx.x & 31, t = t0 + lane;
+  D = t < a.fcp ? a.pfarD[tab + t] : kFarNone;
+  const bool far = D >= 0;
+  const unsigned mf = __ballot_sync(0xffffffffu, far);
+  const int cnt = __popc(mf);
+  __syncwarp();
+  if (far) {
+    const FarK64 p = a.pfar64[tab + t];
+    const int sl = __popc(mf & ((1u << lane) - 1u));
+    s_k[sl] = {p.x, p.y, p.z, p.w, fmax(p.w - 0.5, 0.0), fmax(0.5 - p.w, 0.0)};
+    s_j[sl] = make_int2(z + a.nsplit * t, n0 - D - 1);
+  }
+  if ((cnt & 1) && lane == 31) {
+    s_k[cnt] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    s_j[cnt] = make_int2(z, 0);
+  }
+  __syncwarp();
+  return cnt;
+}
+__device__ __forceinline__ void far_halves64(FarSums64 &S) {
+  S.G += __shfl_xor_sync(0xffffffffu, S.G, 16);
+  S.H0 += __shfl_xor_sync(0xffffffffu, S.H0, 16);
+  S.H2 += __shfl_xor_sync(0xffffffffu, S.H2, 16);
+  S.F += __shfl_xor_sync(0xffffffffu, S.F, 16);
+}
+
+template <bool RING>
+__global__ void __launch_bounds__(kRunWarps * 32)
+    lo_far64_drive_kernel(const __grid_constant__ RunArgs a, int64_t n0_, int ns_) {
+  __shared__ double sh[kRunWarps][32];
+  __shared__ FarEntry64 s_k[kRunWarps][34];
+  __shared__ int2 s_j[kRunWarps][34];
+  if (*((volatile int *)a.status)) return;  // an earlier block failed
+  int64_t n0l = n0_;
+  int ns = ns_;
+  if (ns < 0) {
+    n0l = a.blk[0];
+    if (n0l >= a.n_steps) return;
+    ns = 2 * (int)min((int64_t)a.K, a.n_steps - n0l);
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int b = blockIdx.y;
+  const int i = blockIdx.x * kRunWarps + warp;
+  if (i >= a.N) return;
+  const int z = blockIdx.z;
+  const size_t bi = bidx(a, b, i), b0 = bidx(a, b, 0);
+  double *dst = (a.nsplit > 1 ? a.Epart + (size_t)z * a.B * a.N * (2 * kMaxBlock + 1) : a.Es) + bi * (2 * kMaxBlock + 1);
+  const int n0 = (int)n0l, K = a.K;
+  int err = 0;
+  const int nbad = *((volatile int *)a.nbad), back = a.max_reach;
+  if (nbad >= 0 && n0 - back <= nbad) {
+    const int j_lo = min(a.N, z * a.fcp), j_hi = min(a.N, j_lo + a.fcp);
+    drive_phase<false>(a, b, i, n0l, ns, sh[warp], &err, j_lo, j_hi, dst);
+    if (err) set_status(a.status, err);
+    return;
+  }
+  const size_t row = bi * (size_t)a.N, tab = (bi * a.nsplit + z) * (size_t)a.fcp;
+  double *cw = a.carry64 + 4 * (((size_t)z * a.B + b) * (size_t)a.N + i);
+  const int pos = 2 + (lane & 15);
+  double c0, c1, c2, c3;
+  if (n0l == a.n_begin || (nbad >= 0 && n0 - K - back <= nbad)) {
+    FarSums64 P = {0.0, 0.0, 0.0, 0.0};
+    int D;
+    for (int t0 = 0; t0 < a.fcp; t0 += 32) {
+      const int cnt = far_stage64(a, tab, z, t0, n0, s_k[warp], s_j[warp], D);
+      far_group64<RING>(a, b0, cnt, pos - K, s_k[warp], s_j[warp], P);
+    }
+    far_halves64(P);
+    c0 = __shfl_sync(0xffffffffu, P.H0, K - 2);
+    c1 = __shfl_sync(0xffffffffu, P.H0, K - 1);
+    c2 = __shfl_sync(0xffffffffu, P.G - P.H0 - P.H2, K - 1);
+    c3 = __shfl_sync(0xffffffffu, P.F, K - 1);
+  } else {
+    c0 = cw[0];
+    c1 = cw[1];
+    c2 = cw[2];
+    c3 = cw[3];
+  }
+  FarSums64 S = {0.0, 0.0, 0.0, 0.0};
+  // lane = stage s (time n0 + (s + 1) / 2): the near sources and the far ones' corrections
+  float accf = 0.f;
+  double accd = 0.0;
+  const float stage_f = 0.5f * (__int_as_float(0x4B000000 | (lane + 1)) - 8388608.f);
+  const int mask = RING ? (int)a.wm : -1;
+  for (int t0 = 0; t0 < a.fcp; t0 += 32) {
+    int D;
+    const int cnt = far_stage64(a, tab, z, t0, n0, s_k[warp], s_j[warp], D);
+    far_group64<RING>(a, b0, cnt, pos, s_k[warp], s_j[warp], S);
+    const int kb0 = n0 - D - 1;
+    const bool near = D == kFarNear, wave = D >= 0 && kb0 <= 2 && kb0 + K + 3 >= 0;
+    const unsigned mn = __ballot_sync(0xffffffffu, near), mw = __ballot_sync(0xffffffffu, wave);
+    if (lane < ns) {
+      float grp = 0.f;
+      for (int e = 0; e < cnt; ++e) {
+        const int2 r = s_j[warp][e];
+        const int kb = r.y;
+        if (kb <= 2 && kb + K + 3 >= 0) continue;  // crossing t = 0: below
+        const size_t ij = row + (size_t)r.x;
+        const float4 geo = a.pgeo[ij];
+        const float xs = stage_f - __int_as_float(a.delay[ij].y);
+        float flf;
+        const int k = kb + 1 + Num<float>::floor_int(xs, flf);
+        const float th = xs - flf;
+        const size_t hrow = (b0 + (size_t)r.x) * (size_t)a.hs;
+        const float4 h0 = a.H32[hrow + (size_t)(max(k, 0) & mask)], h1 = a.H32[hrow + (size_t)(max(k + 1, 0) & mask)];
+        const float R = geo.x, iR = __fdividef(1.f, R);
+        const float dX = h1.x - h0.x, dV = h1.y - h0.y, dA = h1.z - h0.z;
+        const float X = fmaf(th, dX, h0.x), V = fmaf(th, dV, h0.y), A = fmaf(th, dA, h0.z);
+        const float mu = geo.y * iR, nu = geo.z * iR;
+        const Cubic q = cubic_terms(mu, X * iR, V, A * R, dX, dV * R, dA * R * R);
+        const float qs = a.dipf[(b0 + (size_t)r.x) * kDipF + 11];
+        grp += 0.25f * qs * iR * iR * fmaf(q.Ca, nu, q.D * geo.w);
+        // a charge off the centre's segment
+        const float hd = 0.5f * fabsf(X * mu);
+        const float o = fmaxf(hd - th, 0.f), o1 = fmaxf(th + hd - 1.f, 0.f);
+        if (o > 0.f || o1 > 0.f) {
+          const FarEntry64 &kk = s_k[warp][e];
+          const int m = o > 0.f ? k : k + 1;  // the sample between the two segments
+          const size_t nm = hrow + (size_t)(max(m - 1, 0) & (int)mask), n_ = hrow + (size_t)(max(m, 0) & (int)mask),
+                       np = hrow + (size_t)(max(m + 1, 0) & (int)mask);
+          const double D2 = kk.k1 * ((a.d[np] - a.d[n_]) - (a.d[n_] - a.d[nm])) +
+                            kk.k2 * ((a.dd[np] - a.dd[n_]) - (a.dd[n_] - a.dd[nm])) +
+                            kk.k3 * ((a.ddd[np] - a.ddd[n_]) - (a.ddd[n_] - a.ddd[nm]));
+          accd = fma(0.5 * (double)fmaxf(o, o1), D2, accd);
+        }
+      }
+      accf += grp;
+      for (unsigned m = mn | mw; m; m &= m - 1) {
+        const int l = __ffs((int)m) - 1, j = z + a.nsplit * (t0 + l);
+        const int2 dl = a.delay[row + j];
+        const float xs = stage_f - __int_as_float(dl.y);
+        float flf;
+        const int k = n0 - dl.x + Num<float>::floor_int(xs, flf);
+        accd += pair_drive_f64(a, b, i, j, (double)n0 + (double)stage_f, n0, k, &err, 0, 2);
+        if ((mw >> l) & 1u) {
+          // less the linear part, from the exact fraction
+          const FarK64 p = a.pfar64[tab + t0 + l];
+          const double x = (double)n0 + (double)stage_f - (double)dl.x - p.w, fl = floor(x), th = x - fl;
+          const size_t hrow = (b0 + (size_t)j) * (size_t)a.hs;
+          const int kk = (int)fl;
+          const size_t na = hrow + (size_t)(max(kk, 0) & mask), nb = hrow + (size_t)(max(kk + 1, 0) & mask);
+          const double v0 = fma(p.z, a.ddd[na], fma(p.y, a.dd[na], p.x * a.d[na]));
+          const double v1 = fma(p.z, a.ddd[nb], fma(p.y, a.dd[nb], p.x * a.d[nb]));
+          accd -= fma(th, v1 - v0, v0);
+        }
+      }
+    }
+    __syncwarp();
+  }
+  far_halves64(S);
+  const double h1 = S.G - S.H0 - S.H2;
+  {
+    const double n0c = __shfl_sync(0xffffffffu, S.H0, K - 2), n1c = __shfl_sync(0xffffffffu, S.H0, K - 1),
+                 n2c = __shfl_sync(0xffffffffu, h1, K - 1), n3c = __shfl_sync(0xffffffffu, S.F, K - 1);
+    if (lane == 0) {
+      cw[0] = n0c;
+      cw[1] = n1c;
+      cw[2] = n2c;
+      cw[3] = n3c;
+    }
+  }
+  if (err) set_status(a.status, err);
+  const int t = lane & 15;
+  const double H0u = __shfl_up_sync(0xffffffffu, S.H0, 2), H1u = __shfl_up_sync(0xffffffffu, h1, 1),
+               Fu = __shfl_up_sync(0xffffffffu, S.F, 1);
+  const double mine = fma((double)accf, a.e_unit, accd);
+  const double mh = __shfl_sync(0xffffffffu, mine, 2 * t), mw_ = __shfl_sync(0xffffffffu, mine, 2 * t + 1);
+  const double x0 = t == 0 ? c0 : (t == 1 ? c1 : H0u), xm = t == 0 ? c2 : H1u, fm = t == 0 ? c3 : Fu;
+  if (lane < 16 && 2 * t < ns) {
+    dst[1 + 2 * t] = ((x0 + xm) + S.H2) + mh;
+    dst[2 + 2 * t] = (fm + (S.G - S.F)) + mw_;
   }
 }
 
@@ -2106,7 +2342,8 @@ static void *drive_kernel_for(const RunArgs &a, bool mixed) {
 }
 // the block loop's drive: the far form where the run has its tables
 static void *block_drive_kernel_for(const RunArgs &a, bool mixed) {
-  if (!a.pfar) return drive_kernel_for(a, mixed);
+  if (!a.pfarD) return drive_kernel_for(a, mixed);
+  if (!mixed) return a.wm >= 0 ? (void *)lo_far64_drive_kernel<true> : (void *)lo_far64_drive_kernel<false>;
   const bool ring = a.wm >= 0;
   if (a.near_L > 0.f)
     return ring ? (void *)lo_far_drive_kernel<true, true> : (void *)lo_far_drive_kernel<true, false>;
@@ -2180,7 +2417,7 @@ static pc_status launch_block_loop(pc_ctx *ctx, const RunArgs &a, bool mixed, di
   kp.blockDim = dim3(kRunWarps * 32);
   kp.kernelParams = drive_args;
   if (cudaGraphAddKernelNode(&n1, body, nullptr, 0, &kp) != cudaSuccess) return PC_ERR_CUDA;
-  kp.func = mixed ? (void *)lo_rk4_kernel<true> : (void *)lo_rk4_kernel<false>;
+  kp.func = a.H32 ? (void *)lo_rk4_kernel<true> : (void *)lo_rk4_kernel<false>;
   kp.gridDim = dim3((unsigned)(((size_t)a.B * a.N * 32 + 127) / 128));  // one warp per receiver
   kp.blockDim = dim3(128);
   kp.kernelParams = rk4_args;
@@ -2302,10 +2539,17 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   const int far_split = std::min(kMaxSplit, std::min(ctx->run_slices > 0 ? ctx->run_slices : 8, std::max(1, dp->N / 8)));
   const int far_cp = (dp->N + far_split - 1) / far_split;
   const size_t far_n = nbn * (size_t)far_split * far_cp;
-  const size_t far_off = od_off + od_bytes, pf_bytes = al(far_n * sizeof(float4)), pd_bytes = al(far_n * sizeof(int));
-  const size_t cr_bytes = al((size_t)pc::kMaxSplit * nbn * sizeof(float4)), am_bytes = al(2 * (size_t)dp->B * sizeof(double));
-  bool far = mixed && grid && !motion;
-  if (far && ctx->run_scratch.reserve(far_off + pf_bytes + pd_bytes + cr_bytes + am_bytes + 256) != cudaSuccess) {
+  const size_t far_off = od_off + od_bytes, pf_bytes = al(far_n * (mixed ? sizeof(float4) : sizeof(FarK64)));
+  const size_t pd_bytes = al(far_n * sizeof(int)), am_bytes = al(2 * (size_t)dp->B * sizeof(double));
+  const size_t cr_bytes = al((size_t)far_split * nbn * (mixed ? sizeof(float4) : 4 * sizeof(double)));
+  const size_t fg_bytes = mixed ? 0 : al(nbn * dp->N * sizeof(float4));  // the float64 drive's pair geometry
+  const size_t far_bytes = pf_bytes + pd_bytes + cr_bytes + am_bytes + fg_bytes + 256;
+  bool far = grid && !motion && !pl.tables_only && n_end < ((int64_t)1 << 30);
+  if (far && far_bytes > ((size_t)1 << 30) && far_off + far_bytes > ctx->run_scratch.bytes) {
+    size_t mfree = 0, mall = 0;  // at most half of what is left
+    if (cudaMemGetInfo(&mfree, &mall) != cudaSuccess || far_bytes > mfree / 2) far = false;
+  }
+  if (far && ctx->run_scratch.reserve(far_off + far_bytes) != cudaSuccess) {
     cudaGetLastError();
     far = false;
   }
@@ -2347,11 +2591,14 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   a.odisp = motion ? (double *)(scr + od_off) : nullptr;
   if (far) {
     char *f = scr + far_off;
-    a.pfar = (float4 *)f;
+    a.pfar = mixed ? (float4 *)f : nullptr;
+    a.pfar64 = mixed ? nullptr : (FarK64 *)f;
     a.pfarD = (int *)(f + pf_bytes);
     a.carry = (float4 *)(f + pf_bytes + pd_bytes);
+    a.carry64 = (double *)a.carry;
     a.amax = (unsigned long long *)(f + pf_bytes + pd_bytes + cr_bytes);
     a.nbad = (int *)(f + pf_bytes + pd_bytes + cr_bytes + am_bytes);
+    if (!mixed) a.pgeo = (float4 *)(f + pf_bytes + pd_bytes + cr_bytes + am_bytes + 256);
     a.fcp = far_cp;
     a.nsplit = far_split;
     // entries past the last source stay kFarNone
@@ -2405,9 +2652,17 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
     hs = W;
     wm = W - 1;
   }
+  if (K < 2 || hs >= ((int64_t)1 << 27)) {  // (the carried sums sit in lanes K - 2 and K - 1)
+    far = false;
+    a.pfar = nullptr;
+    a.pfar64 = nullptr;
+    a.pfarD = nullptr;
+    a.nbad = nullptr;
+  }
+  const bool mirror = mixed || far;  // the history's float32 mirror
   const bool own_ring = !full_store && !pl.sd;
   const size_t ring_b = own_ring ? al(nbn * (size_t)hs * sizeof(double)) : 0;
-  const size_t h_bytes = mixed ? al(nbn * (size_t)hs * sizeof(float4)) : 0;
+  const size_t h_bytes = mirror ? al(nbn * (size_t)hs * sizeof(float4)) : 0;
   // the fit's kinetic energies: after the run from the full store, or per step into their own rows
   const int64_t first = opts->fit ? opts->first_index : 0;
   const size_t ke_b = opts->fit ? al(nbn * (size_t)(full_store ? So : So - first) * sizeof(double)) : 0;
@@ -2419,10 +2674,6 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   a.wm = wm;
   a.K = K;
   a.max_reach = (int)std::min<int64_t>(D, (int64_t)1 << 29);
-  if (K < 2 || hs >= ((int64_t)1 << 27)) {  // (the carried sums sit in lanes K - 2 and K - 1)
-    a.pfar = nullptr;
-    a.nbad = nullptr;
-  }
   if (full_store) {
     a.d = out->d;
     a.dd = out->d_dot;
@@ -2441,7 +2692,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
     a.odd = out->d_dot;
     a.oddd = out->d_ddot;
   }
-  a.H32 = mixed ? (float4 *)(sto + 3 * ring_b) : nullptr;
+  a.H32 = mirror ? (float4 *)(sto + 3 * ring_b) : nullptr;
   a.energy = out->energy;
   a.energy_loop = (out->energy && !full_store) ? 1 : 0;
   a.Ed = out->Ed;
@@ -2462,7 +2713,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   a.state_out = opts->state_out;
   a.state_D = D;
   const unsigned rgrid = (unsigned)((nbn + 127) / 128);
-  if (mixed) pc::lo_first_kernel<true><<<rgrid, 128, 0, st>>>(a);
+  if (mirror) pc::lo_first_kernel<true><<<rgrid, 128, 0, st>>>(a);
   else pc::lo_first_kernel<false><<<rgrid, 128, 0, st>>>(a);
   const bool timed = ctx->run_timing != 0;
   if (dp->N <= pc::kSmallN) {
@@ -2488,7 +2739,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
     const int64_t target = (int64_t)ctx->num_sms * 64;
     int nsplit = (int)std::min<int64_t>(std::max<int64_t>(1, (target + (int64_t)nbn - 1) / (int64_t)nbn),
                                         std::max(1, dp->N / 8));
-    if (a.pfar) {
+    if (far) {
       nsplit = far_split;  // the tables' slices
     } else if (ctx->run_slices > 0) {
       nsplit = std::min(ctx->run_slices, std::max(1, dp->N / 8));  // set or tuned
@@ -2531,7 +2782,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
           pc::launch_drive(pc::block_drive_kernel_for(a, mixed), dgrid, a, n0, 2 * kb, st);
           if (timed) cudaEventRecord(ctx->tev[nev++], st);
           const unsigned wgrid = (unsigned)((nbn * 32 + 127) / 128);
-          if (mixed) pc::lo_rk4_kernel<true><<<wgrid, 128, 0, st>>>(a, n0, kb);
+          if (mirror) pc::lo_rk4_kernel<true><<<wgrid, 128, 0, st>>>(a, n0, kb);
           else pc::lo_rk4_kernel<false><<<wgrid, 128, 0, st>>>(a, n0, kb);
           if (timed) {
             cudaEventRecord(ctx->tev[nev++], st);

@@ -176,3 +176,64 @@ def test_far_drive_refuses_what_is_not_a_number(ctx):
     cfg.omega0[0, 7] = np.nan
     with pytest.raises(pc.PcError):
         pc.pc_dipoles_run(ctx, pc.lo_config_to_device(cfg), cfg.dt, 400, precision=pc.PC_MIXED)
+
+
+# ------------------------------------------------------------------------------------------------
+# the oscillator run's split drive (grid path, float64)
+# ------------------------------------------------------------------------------------------------
+def _ed_binary128(cfg, hist, t0, times, receivers):
+    """E_d of some receivers on a history (d, d', d'' [N][S] from time t0 on) in binary128."""
+    out = []
+    for i in receivers:
+        o = np.arange(cfg.N) != i
+        dps = W.Dipoles(origin=cfg.origin[0, o], axis=cfg.axis[0, o], q=cfg.q[0, o], m1=cfg.m1[0, o], m2=cfg.m2[0, o],
+                        d=hist[0][o], d_dot=hist[1][o], d_ddot=hist[2][o], t0=t0, dt=cfg.dt)
+        r = oracle.fields_x(cfg.origin[0, i][None], times, dipoles=dps)
+        assert r["status"] == oracle.OK
+        out.append(r["E"][:, 0] @ cfg.axis[0, i])
+    return np.array(out)
+
+
+@pytest.mark.parametrize("case", ["cloud", "dense", "unequal masses", "fast", "slices"])
+def test_split_drive_against_binary128(ctx, case):
+    # every receiver's E_d on the run's own history within 1e-10 of its largest value, the float64 path's
+    # bound (two charges at 1e5 times their distance round to 1e-11 of their field)
+    cfg = _cloud(90, seed=29)
+    steps = 420
+    if case == "dense":
+        cfg.origin *= 0.45  # origins down to 2.3 nm, blocks of 7 steps
+    if case == "unequal masses":
+        cfg.m1[0, ::3] *= 1.5
+    if case == "fast":
+        cfg.omega0 *= 30.0  # charges beyond kSplitV: every pair in the two-charge form
+    try:
+        pc.pc_set_run_tiling(ctx, 7 if case == "slices" else 0)
+        f = pc.pc_dipoles_run(ctx, pc.lo_config_to_device(cfg), cfg.dt, steps, precision=pc.PC_F64, want_Ed=True)
+    finally:
+        pc.pc_set_run_tiling(ctx, 0)
+    h = {k: f[k][0].cpu().numpy() for k in ("d", "d_dot", "d_ddot", "Ed")}
+    at = np.r_[np.arange(1, steps, 13), steps - 1, steps]
+    recv = [0, 17, 44, 89]
+    ref = _ed_binary128(cfg, (h["d"], h["d_dot"], h["d_ddot"]), 0.0, at * cfg.dt, recv)
+    for e, i in zip(ref, recv):
+        assert np.max(np.abs(h["Ed"][i, at] - e)) < 1e-10 * np.max(np.abs(e)), i
+
+
+def test_split_drive_leaves_and_returns_where_moments_pass_its_limits(ctx):
+    # as for the mixed drive: oldest samples of the resumed state beyond the limits
+    cfg = _cloud(80)
+    lod = pc.lo_config_to_device(cfg)
+    first, n = 960, 200
+    state = torch.zeros(pc.pc_dipoles_state_size(ctx, lod, cfg.dt), dtype=torch.float64, device="cuda")
+    pc.pc_dipoles_run(ctx, lod, cfg.dt, first, precision=pc.PC_F64, state_out=state)
+    D = int(state[2])
+    smp = state[4 + 80:].view(80, D + 1, 3)
+    smp[:, :20] *= 3.0
+    f = pc.pc_dipoles_run(ctx, lod, cfg.dt, n, precision=pc.PC_F64, state_in=state, want_Ed=True)
+    hist = [np.concatenate([smp[:, :, c].cpu().numpy(), f[k][0, :, 1:].cpu().numpy()], axis=1)
+            for c, k in enumerate(("d", "d_dot", "d_ddot"))]
+    at = np.arange(1, n + 1, 7)
+    recv = [0, 33, 79]
+    ref = _ed_binary128(cfg, hist, (first - D) * cfg.dt, (first + at) * cfg.dt, recv)
+    for e, i in zip(ref, recv):
+        assert np.max(np.abs(f["Ed"][0, i, at].cpu().numpy() - e)) < 1e-10 * np.max(np.abs(e)), i

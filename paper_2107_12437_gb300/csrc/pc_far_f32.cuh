@@ -96,11 +96,183 @@ __device__ __forceinline__ Cubic cubic_terms(float mu, float x, float v, float a
   return o;
 }
 
+// The second-order terms, which the two charges of equal masses share: their derivative along a change of
+// (x, v, al) at fixed slopes enters where only one of the charges sees that change.
+__device__ __forceinline__ Cubic quad_terms(float mu, float x, float v, float al, float dX, float dV, float dA) {
+  const float d1 = -mu * x;
+  const float d2 = 0.5f * x * x * (1.f - mu * mu) - mu * mu * x * dX;
+  const float y2 = -d1 * dX, w2 = -d1 * dV, g2 = -d1 * dA;
+  const float u1 = fmaf(-v, mu, d1), u2 = d2 - fmaf(w2, mu, -v * x);
+  const float i1 = -u1, i2 = fmaf(u1, u1, -u2);
+  const float J1 = 2.f * i1, K1 = 3.f * i1, K2 = 3.f * fmaf(i1, i1, i2);
+  const float G1 = al * mu, G2 = fmaf(g2, mu, -fmaf(al, x, v * v));
+  const float GK1 = G1 + K1;
+  Cubic o;
+  o.Ca = fmaf(G1, K1, G2 + K2);
+  o.Cb = -fmaf(v, GK1, fmaf(al, J1, w2 + g2));
+  o.D = fmaf(d1, -(v + al), o.Cb) - fmaf(x, GK1, y2);
+  o.phi = i2;
+  o.A = fmaf(v, i1, w2);
+  return o;
+}
+// that derivative along (ex, ev, ea), exact for a quadratic form: half the difference at +-t times it, t
+// making the step as large as the point
+__device__ __forceinline__ void add_quad_slope(Cubic &c, float sign, float mu, float x, float v, float al, float dX, float dV,
+                                               float dA, float ex, float ev, float ea) {
+  const float t = __fdividef(fabsf(x) + fabsf(v) + fabsf(al), fabsf(ex) + fabsf(ev) + fabsf(ea) + 1e-30f);
+  const Cubic a = quad_terms(mu, fmaf(t, ex, x), fmaf(t, ev, v), fmaf(t, ea, al), dX, dV, dA);
+  const Cubic b = quad_terms(mu, fmaf(-t, ex, x), fmaf(-t, ev, v), fmaf(-t, ea, al), dX, dV, dA);
+  const float w = t > 0.f ? __fdividef(0.5f * sign, t) : 0.f;
+  c.Ca = fmaf(w, a.Ca - b.Ca, c.Ca);
+  c.D = fmaf(w, a.D - b.D, c.D);
+  c.Cb = fmaf(w, a.Cb - b.Cb, c.Cb);
+  c.phi = fmaf(w, a.phi - b.phi, c.phi);
+  c.A = fmaf(w, a.A - b.A, c.A);
+}
+
 // The distance from which the split form serves a float64 driving field.  With X/R <= kSplitX the cubic
 // terms' float32 rounding is 1e-14 of the pair's field, against the 1e-16 R/X (3e-13) at which the sum of
 // the two charges rounds there (less only where they do not cancel: on a ring of 256 with moments along its
 // axis E_d was within 2.5e-16 of binary128; 6.5e-4 here made that 8e-16).  V <= kSplitV keeps the fifth order
 // in V below 1e-14.  Equal masses only: the second order of unequal ones, in float32, would be 1e-11.
 constexpr double kSplitX = 4e-4, kSplitV = 2e-4;
+
+
+// One dipole's field at a point in the split form, for the float64 field sum and for near fields that
+// cancel in float32: r the separation from its centre (c dt), p its axis, qs = q / e, u the time in samples,
+// d / dd / ddd its float64 history with the scales (1/(qL), 1/(qc), dt/(qc)) and H the float32 mirror.
+// Adds the linear part to lin[10] (float64) and the cubic terms to cub[10] (float32), both as (E, B, phi, A)
+// in the units of dipole_pair.  False, adding nothing, where the two-charge form has to decide: off the
+// interior of the history, within rmin of the centre, or X/R or V beyond the limits at the samples.  Equal
+// masses only (the caller's condition).
+// 1/R comes from float32's by one third-order step y (1 + e/2 + 3 e^2/8), e = 1 - R^2 y^2 (its error 5 e^3/16
+// is below 1e-19), the sample index by adding 1.5 * 2^52 with rounding down: about 66 instructions on the
+// float64 unit a pair, where the two charges' roots and difference form take 280.
+struct SplitLimits {
+  float x, v, rmin;
+};
+template <int KIND>
+__device__ __forceinline__ bool split_dipole(double rx, double ry, double rz, double px, double py, double pz, double qs,
+                                             double u, const double *d, const double *dd, const double *ddd, double sx,
+                                             double sv, double sa, const float4 *H, int S, const SplitLimits lim,
+                                             double (&lin)[10], float (&cub)[10]) {
+  const double R2 = fma(rz, rz, fma(ry, ry, rx * rx));
+  const float fx = (float)rx, fy = (float)ry, fz = (float)rz;
+  const float R2f = fmaf(fz, fz, fmaf(fy, fy, fx * fx));
+  const float iRf = rsqrt_fast(R2f), Rf = R2f * iRf;
+  // (the radiation field's cubic terms are a difference from the Coulomb field's, which outweighs it close by)
+  if (!(Rf > (KIND == PC_RADIATION ? fmaxf(lim.rmin, 300.f) : lim.rmin) && Rf < 1e9f)) return false;
+  const double y = (double)iRf;
+  const double e = fma(-(R2 * y), y, 1.0);
+  const double i = fma(y * e, fma(e, 0.375, 0.5), y);
+  const double R = R2 * i;
+  const double x = u - R;
+  if (!(x > 2.0 && x < (double)(S - 3))) return false;
+  const double magic = 6755399441055744.0;  // 1.5 * 2^52
+  const double m = __dadd_rd(x, magic);
+  const int k = __double2loint(m);
+  const double th = (u - (m - magic)) - R;  // (u less a whole number of samples is exact)
+  const float4 h0 = __ldg(H + k), h1 = __ldg(H + k + 1);
+  if (!(fmaxf(fabsf(h0.x), fabsf(h1.x)) <= lim.x * Rf && fmaxf(fabsf(h0.y), fabsf(h1.y)) <= lim.v)) return false;
+  const double d0 = d[k], v0 = dd[k], a0 = ddd[k];
+  const double Dd = d[k + 1] - d0, Dv = dd[k + 1] - v0, Da = ddd[k + 1] - a0;
+  double X = fma(th, Dd, d0), V = fma(th, Dv, v0), A = fma(th, Da, a0);
+  const float qf = (float)qs, pxf = (float)px, pyf = (float)py, pzf = (float)pz, thf = (float)th;
+  const float mu = fmaf(fz, pzf, fmaf(fy, pyf, fx * pxf)) * iRf;
+  // (the slopes from the float64 samples: a difference of float32 ones is good to 5e-5 only, which put
+  // 1e-14 instead of 1e-15 into the fields of 10 pm dipoles)
+  const float dX = (float)(Dd * sx), dV = (float)(Dv * sv), dA = (float)(Da * sa);
+  const float Xf = fmaf(thf, dX, h0.x);
+  // a charge whose own retarded time lies off the centre's segment: its state differs from the segment's
+  // extension by the overshoot times the second difference of the samples.  The charges' delays are off the
+  // centre's by -+ X mu / 2 + (X^2 (1 - mu^2) / 2 - mu^2 X X') / 4 R: the overshoots from those in float64
+  // (float32 ones, good to 1e-7 of a sample, put 1e-13 into the potentials at such points)
+  const float s1 = 0.5f * Xf * mu, s2 = 0.25f * Xf * iRf * fmaf(0.5f * Xf, fmaf(-mu, mu, 1.f), -mu * mu * Rf * dX);
+  float ex = 0.f, ev = 0.f, ea = 0.f, sign = 0.f;
+  if (fabsf(thf - 0.5f) + fabsf(s1) + fabsf(s2) > 0.499999f) {
+    const double tp = th + (double)(s1 - s2), tm = th - (double)(s1 + s2);  // the charges' fractions
+    const double lp = fmax(-tp, 0.0), lm = fmax(-tm, 0.0), hp = fmax(tp - 1.0, 0.0), hm = fmax(tm - 1.0, 0.0);
+    const double lo = lp + lm, hi = hp + hm;
+    if (lo > 0.0 || hi > 0.0) {
+      const int n = lo > 0.0 ? k : k + 1;
+      const double o = lo > 0.0 ? lo : hi;
+      const double eX = o * ((d[n + 1] - d[n]) - (d[n] - d[n - 1])), eV = o * ((dd[n + 1] - dd[n]) - (dd[n] - dd[n - 1])),
+                   eA = o * ((ddd[n + 1] - ddd[n]) - (ddd[n] - ddd[n - 1]));
+      X = fma(0.5, eX, X);
+      V = fma(0.5, eV, V);
+      A = fma(0.5, eA, A);
+      // the next order, of opposite sign for the two charges
+      sign = (lo > 0.0 ? lp > lm : hp > hm) ? 1.f : -1.f;
+      ex = (float)(eX * sx) * iRf;
+      ev = (float)(eV * sv);
+      ea = (float)(eA * sa) * Rf;
+    }
+  }
+  X *= sx;
+  V *= sv;
+  A *= sa;
+  const double qx = qs * px, qy = qs * py, qz = qs * pz;
+  const double i2 = i * i, rpi2 = fma(rz, qz, fma(ry, qy, rx * qx)) * i2;
+  const double t1 = fma(i, X, V);
+  double cE, cP, cB;
+  if (KIND == PC_COULOMB) {
+    cE = rpi2 * i2 * (3.0 * t1);
+    cP = i2 * t1;
+    cB = i2 * i * V;
+  } else if (KIND == PC_RADIATION) {
+    cE = rpi2 * i * A;
+    cP = i * A;
+    cB = i2 * A;
+  } else {
+    cE = rpi2 * i * fma(3.0 * i, t1, A);
+    cP = i * fma(i, t1, A);
+    cB = i2 * fma(i, V, A);
+  }
+  lin[0] = fma(-cP, qx, fma(cE, rx, lin[0]));
+  lin[1] = fma(-cP, qy, fma(cE, ry, lin[1]));
+  lin[2] = fma(-cP, qz, fma(cE, rz, lin[2]));
+  lin[3] = fma(cB, fma(qy, rz, -(qz * ry)), lin[3]);
+  lin[4] = fma(cB, fma(qz, rx, -(qx * rz)), lin[4]);
+  lin[5] = fma(cB, fma(qx, ry, -(qy * rx)), lin[5]);
+  lin[6] = fma(rpi2, t1, lin[6]);
+  const double vi = V * i;
+  lin[7] = fma(vi, qx, lin[7]);
+  lin[8] = fma(vi, qy, lin[8]);
+  lin[9] = fma(vi, qz, lin[9]);
+  // the cubic terms (1 - 3 mu+ mu- = 1/4 for equal masses)
+  const float xn = Xf * iRf, vf = fmaf(thf, dV, h0.y), al = fmaf(thf, dA, h0.z) * Rf;
+  const float dVn = dV * Rf, dAn = dA * Rf * Rf;
+  Cubic c = cubic_terms(mu, xn, vf, KIND == PC_COULOMB ? 0.f : al, dX, dVn, KIND == PC_COULOMB ? 0.f : dAn);
+  if (sign != 0.f)
+    add_quad_slope(c, sign, mu, xn, vf, KIND == PC_COULOMB ? 0.f : al, dX, dVn, KIND == PC_COULOMB ? 0.f : dAn, ex, ev,
+                   KIND == PC_COULOMB ? 0.f : ea);
+  float Ca = c.Ca, D = c.D, Cb = c.Cb;
+  if (KIND == PC_RADIATION) {
+    Cubic v = cubic_terms(mu, xn, vf, 0.f, dX, dVn, 0.f);
+    if (sign != 0.f) add_quad_slope(v, sign, mu, xn, vf, 0.f, dX, dVn, 0.f, ex, ev, 0.f);
+    Ca -= v.Ca;
+    D -= v.D;
+    Cb -= v.Cb;
+  }
+  const float q1 = 0.25f * qf * iRf, q2 = q1 * iRf;
+  const float ca = q2 * Ca * iRf, cd = q2 * D, cb = q2 * Cb * iRf, cv = q1 * c.A;
+  cub[0] += fmaf(ca, fx, cd * pxf);
+  cub[1] += fmaf(ca, fy, cd * pyf);
+  cub[2] += fmaf(ca, fz, cd * pzf);
+  cub[3] = fmaf(cb, fy * pzf - fz * pyf, cub[3]);
+  cub[4] = fmaf(cb, fz * pxf - fx * pzf, cub[4]);
+  cub[5] = fmaf(cb, fx * pyf - fy * pxf, cub[5]);
+  cub[6] = fmaf(q1, c.phi, cub[6]);
+  cub[7] = fmaf(cv, pxf, cub[7]);
+  cub[8] = fmaf(cv, pyf, cub[8]);
+  cub[9] = fmaf(cv, pzf, cub[9]);
+  return true;
+}
+
+// float64 field sum: errors against binary128 as the two-charge form's (300 points of the grid of 64 dipoles
+// of 1, 10 and 20 pm: E rms 1.2-1.6e-12, B 4e-15, phi 2e-13, A 1.8e-15 in both; medians 1.2e-15)
+constexpr float kSplitFieldX = 6e-5f, kSplitFieldV = 1e-4f;
+// near fields of the mixed sum, kept to 1e-10 of the terms' magnitudes
+constexpr float kSplitNearX = 1e-3f, kSplitNearV = 1e-3f;
 
 }  // namespace pc

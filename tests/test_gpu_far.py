@@ -237,3 +237,38 @@ def test_split_drive_leaves_and_returns_where_moments_pass_its_limits(ctx):
     ref = _ed_binary128(cfg, hist, (first - D) * cfg.dt, (first + at) * cfg.dt, recv)
     for e, i in zip(ref, recv):
         assert np.max(np.abs(f["Ed"][0, i, at].cpu().numpy() - e)) < 1e-10 * np.max(np.abs(e)), i
+
+
+# ------------------------------------------------------------------------------------------------
+# the float64 field sum's split form
+# ------------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("kind", [pc.PC_TOTAL, pc.PC_COULOMB, pc.PC_RADIATION])
+@pytest.mark.parametrize("case", ["1 pm", "20 pm", "100 pm", "unequal masses", "list", "ends"])
+def test_split_fields_against_binary128(ctx, case, kind):
+    # plain relative errors of the float64 path within 1e-10 at every point that no cancellation between
+    # the sources deeper than 1e3 affects (the bound of the two-charge form, tests/test_gpu_fields.py)
+    amp = {"1 pm": 1e-12, "20 pm": 2e-11, "100 pm": 1e-10}.get(case, 1e-11)
+    dp = _sources(41, amp=amp, t_end=6e-15 if case == "ends" else 15e-15)
+    times = [3.5e-15, 6e-15] if case == "ends" else [10.4e-15, 12.5e-15]
+    if case == "unequal masses":
+        dp.m1[::2] *= 3.0
+    nu, nv, step, z = 129, 257, 1.1e-9, 0.45e-6
+    dev = pc.dipoles_to_device(dp)
+    rng = np.random.default_rng(8)
+    p = rng.integers(0, nu * nv, 90)
+    pts = np.stack([0.3e-6 + (p // nv) * step, 0.2e-6 + (p % nv) * step, np.full(p.size, z)], axis=1)
+    if case == "list":
+        allp = rng.uniform(0.0, 1e-6, (nu * nv, 3))
+        out = pc.pc_fields(ctx, dipoles=dev, points=torch.as_tensor(allp, device="cuda"), times=times, kind=kind)
+        pts = allp[p]
+    else:
+        out = pc.pc_fields_plane(ctx, dipoles=dev, origin=(0.3e-6, 0.2e-6, z), eu=(step, 0, 0), ev=(0, step, 0), nu=nu,
+                                 nv=nv, times=times, kind=kind)
+    ref = oracle.fields_x(pts, times, dipoles=dp, kind=kind)
+    scale = oracle.fields(pts, times, dipoles=dp, kind=kind)["scale_source"]
+    assert ref["status"] == oracle.OK and not out["mask"].any()
+    norm = lambda v: np.abs(v) if v.ndim == 2 else np.linalg.norm(v, axis=-1)  # noqa: E731
+    for k in ("E", "B", "phi", "A"):
+        g = out[k][:, torch.as_tensor(p, device="cuda")].cpu().numpy()
+        sc = scale["E"] / W.C if k == "B" else scale[k]
+        assert np.all(norm(g - ref[k]) <= 1e-10 * np.maximum(norm(ref[k]), 1e-3 * sc)), k

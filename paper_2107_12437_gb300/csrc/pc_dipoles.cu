@@ -2467,6 +2467,7 @@ struct RunPlan {
   int64_t ke_first = 0, ke_len = 0;
   int64_t *reach_out = nullptr;             // the state depth D of this geometry
   bool tables_only = false;                 // stop after the tables (the state-size query)
+  RunArgs *args_out = nullptr;              // the run's arguments (tables and mirror valid until the next run)
 };
 
 static int64_t pow2_at_least(int64_t x) {
@@ -2796,6 +2797,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
       }
     }
   }
+  if (pl.args_out) *pl.args_out = a;
   if (opts->state_out) pc::lo_save_kernel<<<ctx->num_sms * 4, 256, 0, st>>>(a, D);
   if (a.energy && !a.energy_loop) pc::energy_kernel<<<ctx->num_sms * 4, 256, 0, st>>>(a);
   if (opts->fit) {
@@ -2978,6 +2980,7 @@ struct AdjArgs {
   double *gpos, *gvel, *gacc;
   double *disp;
   double *g_origin, *g_omega0, *g_d0;
+  unsigned long long *ebmax;  // the largest |Ebar| so far (bits), or null
   int64_t margin;      // samples of slack around the retarded window (charge offsets)
 };
 
@@ -3122,15 +3125,24 @@ __global__ void adj_rk4_kernel(const AdjArgs A, int64_t n0, int kb) {
   A.lam[2 * bi + 1] = l1;
   A.carry[bi] = carry;
   A.w0bar[bi] += w0b;
+  if (A.ebmax) {
+    double m = 0.0;
+    for (int k = 1; k <= 2 * kb; ++k) m = fmax(m, fabs(Eb[k]));
+    atomicMax(A.ebmax, (unsigned long long)__double_as_longlong(m));
+  }
 }
 
 // Reverse of the driving-field contribution F = p_i . E of dipole j's two charges at receiver i
 // and time u (steps, history 0..nv).  eb = dL/dF.  Adds to the history adjoints of j (window
 // win[0..W) for samples wlo..), to the receiver's and the source's origin adjoints.
-template <bool MOV>
+// GLOBAL: the history adjoints go to A.mu itself (atomics that return nothing), the window is not used.
+template <bool MOV, bool GLOBAL = false>
 __device__ int pair_rev_f64(const AdjArgs &A, int b, int i, int j, double u, int64_t nv, double eb, double *win,
                             int64_t wlo, int W, double Rib[3], double Rjb[3]) {
   const RunArgs &a = A.f;
+  auto slot = [&](int64_t k) {
+    return GLOBAL ? A.mu + (bidx(a, b, j) * (size_t)a.hs + (size_t)(k & a.wm)) * 3 : win + 3 * (k - wlo);
+  };
   const double cdt = kC * a.dt;
   const size_t bi = bidx(a, b, i), bj = bidx(a, b, j);
   const double *Ri = a.origin + 3 * bi;
@@ -3224,7 +3236,7 @@ __device__ int pair_rev_f64(const AdjArgs &A, int b, int i, int j, double u, int
           Rjb[cc] -= abc;
         }
         const double pb_p = -(Rb * iR * aj + ajb + aib * apj);  // -ab . p_j
-        if (k < wlo || k + 1 >= wlo + W) return PC_ERR_NOCONV;
+        if (!GLOBAL && (k < wlo || k + 1 >= wlo + W)) return PC_ERR_NOCONV;
         const double Db = w * pb_p, Vb = w * svb, Ab = w * sab;
         const double thb = Db * Dd + Vb * Dv + Ab * Da;
         const double Gth = -2.0 * cdt * cdt * (u - (double)k - th) + 2.0 * w * Dd * aj;
@@ -3234,7 +3246,7 @@ __device__ int pair_rev_f64(const AdjArgs &A, int b, int i, int j, double u, int
           Rjb[cc] += sfac * (2.0 * av[cc]);
         }
         const double dbar = Db + sfac * 2.0 * aj * w;
-        double *w0p = win + 3 * (k - wlo), *w1p = w0p + 3;
+        double *w0p = slot(k), *w1p = slot(k + 1);
         atomicAdd(&w0p[0], (1.0 - th) * dbar);
         atomicAdd(&w0p[1], (1.0 - th) * Vb);
         atomicAdd(&w0p[2], (1.0 - th) * Ab);
@@ -3287,15 +3299,15 @@ __device__ int pair_rev_f64(const AdjArgs &A, int b, int i, int j, double u, int
     const double pb_p = -dot3(ab, pj);  // adjoint of the charge offset along the axis
     if (stat) {
       // position R_j + w d[0] p_j: only d[0] (window slot of sample 0) and the first origin sample
-      if (wlo != 0) return PC_ERR_NOCONV;
-      atomicAdd(&win[0], w * pb_p);
+      if (!GLOBAL && wlo != 0) return PC_ERR_NOCONV;
+      atomicAdd(slot(0), w * pb_p);
       if (mov && A.gpos)
         for (int c = 0; c < 3; ++c) atomicAdd(A.gpos + bj * H * 3 + c, -ab[c]);
       continue;
     }
-    if (k < wlo || k + 1 >= wlo + W) return PC_ERR_NOCONV;
+    if (!GLOBAL && (k < wlo || k + 1 >= wlo + W)) return PC_ERR_NOCONV;
     const double Db = w * pb_p, Vb = w * dot3(vb, pj), Ab = w * dot3(accb, pj);
-    double *w0p = win + 3 * (k - wlo), *w1p = w0p + 3;
+    double *w0p = slot(k), *w1p = slot(k + 1);
     // the fraction th depends on the inputs through G(th) = cdt^2 (u - k - th)^2 - |r - p(th)|^2 = 0
     double thb = Db * Dd + Vb * Dv + Ab * Da;
     const double ap = dot3(av, pj);
@@ -3435,6 +3447,272 @@ __global__ void __launch_bounds__(128, 4) adj_field_kernel(const AdjArgs A, int6
   // the window into the source's history adjoints (this CTA owns source j during the launch)
   for (int t = threadIdx.x; t < 3 * W; t += blockDim.x)
     A.mu[(bj * a.hs + ((wlo + t / 3) & a.wm)) * 3 + t % 3] += win[t];
+}
+
+// (2) in the split form (pc_far_f32.cuh), fixed origins: F of a far pair is k1 d + k2 d' + k3 d'' of its source
+// interpolated at a constant delay D + f, plus the cubic terms.  A warp takes 32 of a source's receivers at a
+// time (CTAs: y configurations, z shares of the receivers).  With c_p the stage adjoints' weights at sample
+// position p (the interpolation's transpose) the linear part adds c_p (k1, k2, k3) to the samples' adjoints,
+// and its derivatives by the geometry need only S = sum_p c_p (d, d', d'')_p and the slope sum S4 = sum_p s_p g_p,
+// g = k1 d + k2 d' + k3 d'': lanes = positions.  The cubic terms go through their reverse in float32, lanes =
+// stages, their adjoints of the samples gathered by the positions.  Where a charge is off its centre's
+// segment by o samples the term o/2 (k . second difference) is reversed in float64.  The geometry's gradient
+// is formed at the end of a batch, lanes = receivers.  Near sources, those crossing t = 0 and blocks that may
+// hold a sample beyond the limits go through pair_rev_f64, lanes = stages.  All history adjoints go to A.mu
+// by atomics that return nothing (a shared-memory window's float64 ones are compare-and-swap loops: 1.25 ms a
+// block of the ring of 256 against 0.42; 2.7 with two charges throughout).  The float64 unit is busy 82 %.
+constexpr int kRevWarps = 4;
+struct RevShared {
+  double s[8 * 4][19];       // partial sums of 8 pairs, rows = (pair, S1 .. S4), columns = positions, the last: crossings
+  double S[32][4];           // a batch's sums
+  float f[8 * 4][33];        // partial float32 sums of 8 pairs, rows = (pair, mu, nu, R, time), columns = stages
+  float T[32][4];
+  float h[6][33];            // adjoints of the two samples of a stage's segment (X, V, A each), columns = stages
+  double eb[40];             // the stage adjoints of a receiver, stage s at eb[3 + s], zeros around
+  FarEntry64 k[34];
+  int2 j[34];
+};
+__global__ void __launch_bounds__(kRevWarps * 32, 3) adj_split_kernel(const __grid_constant__ AdjArgs A, int64_t n0, int ns) {
+  extern __shared__ double dyn[];
+  __shared__ double s_rj[3][kRevWarps];
+  const RunArgs &a = A.f;
+  const int j = blockIdx.x, b = blockIdx.y;
+  const size_t bj = bidx(a, b, j), b0 = bidx(a, b, 0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  RevShared &sh = reinterpret_cast<RevShared *>(dyn)[warp];
+  const int nbad = *((volatile int *)a.nbad);
+  const bool all_near = nbad >= 0 && n0 - a.max_reach <= nbad;
+  const int kb_steps = ns / 2, n0i = (int)n0;
+  // the float32 part runs on stage adjoints over their largest so far, in units of k_e e / (c dt)^2
+  const double emax = __longlong_as_double((long long)*A.ebmax), iemax = emax > 0.0 ? 1.0 / emax : 0.0;
+  const double unit = emax * a.e_unit;
+  const double iL = 1.0 / (kC * a.dt), L = kC * a.dt;
+  const double Rj[3] = {a.origin[3 * bj], a.origin[3 * bj + 1], a.origin[3 * bj + 2]};
+  const double pj[3] = {a.axis[3 * bj], a.axis[3 * bj + 1], a.axis[3 * bj + 2]};
+  const double *dj = a.d + bj * a.hs, *ddj = a.dd + bj * a.hs, *dddj = a.ddd + bj * a.hs;
+  const float4 *hj = a.H32 + bj * (size_t)a.hs;
+  double *muj = A.mu + bj * (size_t)a.hs * 3;
+  const int64_t wm = a.wm;
+  const float qs = a.dipf[bj * kDipF + 11];
+  const double msx = 1.0 / (a.q[bj] * L), msv = 1.0 / (a.q[bj] * kC), msa = a.dt / (a.q[bj] * kC);  // the mirror's scales
+  const float stage_f = 0.5f * (__int_as_float(0x4B000000 | (lane + 1)) - 8388608.f);
+  double Gj[3] = {0.0, 0.0, 0.0};  // the lane's part of dL / dR_j
+  int err = 0;
+  const int groups = (a.fcp + 31) / 32;
+  for (int gz = blockIdx.z * kRevWarps + warp; gz < groups * a.nsplit; gz += kRevWarps * gridDim.z) {
+    const int z = gz % a.nsplit, t0 = 32 * (gz / a.nsplit);
+    const size_t tab = (bj * a.nsplit + z) * (size_t)a.fcp;
+    int D;
+    const int cnt = far_stage64(a, tab, z, t0, n0i, sh.k, sh.j, D);
+    const bool valid = D != kFarNone;
+    const int kb0 = n0i - D - 1;
+    const bool wave = D >= 0 && kb0 <= 2 && kb0 + kMaxBlock + 3 >= 0;
+    const unsigned mnear = __ballot_sync(0xffffffffu, valid && (D < 0 || wave || all_near));
+    // ---- far receivers, eight at a time ----
+    if (!all_near)
+      for (int e0 = 0; e0 < cnt; e0 += 8) {
+        const int e1 = min(cnt, e0 + 8);
+        for (int e = e0; e < e1; ++e) {
+          const int2 r = sh.j[e];
+          const int i = r.x, kb = r.y;
+          const bool skip = kb <= 2 && kb + kMaxBlock + 3 >= 0;  // crossing t = 0: among the near ones
+          const size_t bi = b0 + (size_t)i;
+          const int row = 4 * (e - e0);
+          __syncwarp();
+          const double ebs = (!skip && lane < ns) ? A.Ebar[bi * (2 * kMaxBlock + 1) + 1 + lane] : 0.0;
+          sh.eb[4 + lane] = ebs;
+          if (lane < 4) {
+            sh.eb[lane] = 0.0;
+            sh.s[row + lane][18] = 0.0;
+          }
+          if (lane >= 28) sh.eb[lane + 8] = 0.0;
+          const FarEntry64 &k = sh.k[e];
+          // the two fractions and segments: half-step stage t at position t + qh, whole-step t at t + 1
+          const int qh = k.f > 0.5 ? 0 : 1;
+          __syncwarp();
+          // lanes = stages: the cubic terms
+          float fm = 0.f, fn = 0.f, fR = 0.f, ft = 0.f;
+          float l0 = 0.f, l1 = 0.f, l2 = 0.f, u0 = 0.f, u1 = 0.f, u2 = 0.f;
+          if (!skip && lane < ns) {
+            const float4 geo = a.pgeo[bj * (size_t)a.N + i];  // the pair's geometry with the roles exchanged
+            const bool half = !(lane & 1);
+            const int kk = kb + (lane >> 1) + (half ? qh : 1);
+            const double thd = half ? (qh ? 0.5 : 1.5) - k.f : 1.0 - k.f;
+            const float th = (float)thd;
+            const int64_t sk0 = (int64_t)max(kk, 0) & wm, sk1 = (int64_t)max(kk + 1, 0) & wm;
+            const float4 h0 = hj[sk0];
+            const float R = geo.x, iR = __fdividef(1.f, R);
+            // (slopes from the float64 samples)
+            const float dX = (float)((dj[sk1] - dj[sk0]) * msx), dV = (float)((ddj[sk1] - ddj[sk0]) * msv),
+                        dA = (float)((dddj[sk1] - dddj[sk0]) * msa);
+            const float X = fmaf(th, dX, h0.x), V = fmaf(th, dV, h0.y), Ac = fmaf(th, dA, h0.z);
+            // rho points from j to i here: geo's from i to j (row j: rho . p_i, rho . p_j with the other sign)
+            const float mu = -geo.z * iR, nu = -geo.y * iR;
+            const float y = (float)(ebs * iemax) * 0.25f * qs * iR * iR;
+            Cubic q;
+            const CubicIn g = cubic_terms_rev(mu, X * iR, V, Ac * R, dX, dV * R, dA * R * R, y * nu, y * geo.w, q);
+            float xb = g.x * iR;
+            const float vb = g.v, ab = g.al * R;                       // of X, V, A
+            const float pb = g.dX, qb = g.dV * R, rb = g.dA * R * R;  // of the slopes
+            const float val = q.Ca * nu + q.D * geo.w;
+            fm = g.mu;
+            fn = y * q.Ca;
+            fR = iR * (g.al * Ac * R + g.dV * dV * R + 2.f * g.dA * dA * R * R - g.x * X * iR - 2.f * y * val);
+            ft = vb * dV + ab * dA;
+            // a charge off the segment: fractions th + s1 - s2 and th - s1 - s2 (as in split_dipole)
+            const float m2 = mu * mu;
+            const float s1 = 0.5f * X * mu, s2 = 0.25f * X * iR * (0.5f * X * (1.f - m2) - m2 * R * dX);
+            if (fabsf(th - 0.5f) + fabsf(s1) + fabsf(s2) > 0.499999f) {
+              const double tp = thd + (double)(s1 - s2), tm = thd - (double)(s1 + s2);
+              const double lo = fmax(-tp, 0.0) + fmax(-tm, 0.0), hi = fmax(tp - 1.0, 0.0) + fmax(tm - 1.0, 0.0);
+              if (lo > 0.0 || hi > 0.0) {
+                const int m = lo > 0.0 ? kk : kk + 1;
+                const int64_t sa = (int64_t)max(m - 1, 0) & wm, sb = (int64_t)max(m, 0) & wm, sc = (int64_t)max(m + 1, 0) & wm;
+                const double D2x = (dj[sc] - dj[sb]) - (dj[sb] - dj[sa]), D2v = (ddj[sc] - ddj[sb]) - (ddj[sb] - ddj[sa]),
+                             D2a = (dddj[sc] - dddj[sb]) - (dddj[sb] - dddj[sa]);
+                const double D2 = k.k1 * D2x + k.k2 * D2v + k.k3 * D2a;
+                const double w = 0.5 * (lo > 0.0 ? lo : hi) * ebs;
+                atomicAdd(&sh.s[row][18], w * D2x);
+                atomicAdd(&sh.s[row + 1][18], w * D2v);
+                atomicAdd(&sh.s[row + 2][18], w * D2a);
+                const double c3[3] = {w * k.k1, w * k.k2, w * k.k3};
+                for (int c = 0; c < 3; ++c) {
+                  atomicAdd(muj + 3 * sa + c, c3[c]);
+                  atomicAdd(muj + 3 * sb + c, -2.0 * c3[c]);
+                  atomicAdd(muj + 3 * sc + c, c3[c]);
+                }
+                // through the overshoot -(th +- s1 - s2) or th +- s1 - s2 - 1; the next order of the term, of
+                // opposite sign for the two charges, counts here (1e-5 of a second difference is 1e-8 of a slope)
+                const bool plus = lo > 0.0 ? tp < tm : tp > tm;
+                Cubic q2 = {0.f, 0.f, 0.f, 0.f, 0.f};
+                add_quad_slope(q2, plus ? 1.f : -1.f, mu, X * iR, V, Ac * R, dX, dV * R, dA * R * R, (float)(D2x * msx) * iR,
+                               (float)(D2v * msv), (float)(D2a * msa) * R);
+                const float ob = (float)(0.5 * (ebs * iemax) * (D2 / a.e_unit)) + y * (q2.Ca * nu + q2.D * geo.w);
+                const float tb = lo > 0.0 ? -ob : ob;  // of the charge's fraction
+                const float sg = plus ? 1.f : -1.f;
+                fm += tb * (sg * 0.5f * X + 0.5f * X * mu * (0.5f * X * iR + dX));
+                xb += tb * (sg * 0.5f * mu - 0.25f * (X * iR * (1.f - m2) - m2 * dX));
+                ft += tb;
+              }
+            }
+            ft += xb * dX;
+            l0 = (1.f - th) * xb - pb;
+            l1 = (1.f - th) * vb - qb;
+            l2 = (1.f - th) * ab - rb;
+            u0 = th * xb + pb;
+            u1 = th * vb + qb;
+            u2 = th * ab + rb;
+          }
+          sh.f[row][lane] = fm;
+          sh.f[row + 1][lane] = fn;
+          sh.f[row + 2][lane] = fR;
+          sh.f[row + 3][lane] = ft;
+          sh.h[0][lane] = l0;
+          sh.h[1][lane] = l1;
+          sh.h[2][lane] = l2;
+          sh.h[3][lane] = u0;
+          sh.h[4][lane] = u1;
+          sh.h[5][lane] = u2;
+          __syncwarp();
+          // lanes = positions 0 .. kb_steps + 1: half(t) = eb[4 + 2t], whole(t) = eb[5 + 2t]
+          if (lane < kb_steps + 2) {
+            const int p = lane;
+            const double h0 = sh.eb[4 + 2 * p], hm1 = sh.eb[2 + 2 * p], hm2 = sh.eb[2 * p];
+            const double w1 = sh.eb[3 + 2 * p], w2 = sh.eb[1 + 2 * p];
+            const double c = fma(k.w0, h0, fma(1.0 - k.w0 - k.w2, hm1, fma(k.w2, hm2, fma(k.f, w1, (1.0 - k.f) * w2))));
+            const double sl = (qh ? hm2 - hm1 : hm1 - h0) + (w2 - w1);
+            const int64_t sn = (int64_t)max(kb + p, 0) & wm;
+            const double x = dj[sn], v = ddj[sn], ac = dddj[sn];
+            sh.s[row][p] = c * x;
+            sh.s[row + 1][p] = c * v;
+            sh.s[row + 2][p] = c * ac;
+            sh.s[row + 3][p] = sl * fma(k.k3, ac, fma(k.k2, v, k.k1 * x));
+            if (!skip) {
+              // the stages whose segment starts at p, and those whose segment ends there
+              const int a0 = 2 * (p - qh), a1 = 2 * (p - 1) + 1, b0_ = 2 * (p - 1 - qh), b1 = 2 * (p - 2) + 1;
+              double *w = muj + 3 * sn;
+              const double kc[3] = {k.k1, k.k2, k.k3}, sc[3] = {unit * msx, unit * msv, unit * msa};
+#pragma unroll
+              for (int q = 0; q < 3; ++q) {
+                float t = 0.f;
+                if (a0 >= 0 && a0 < 32) t += sh.h[q][a0];
+                if (a1 >= 0 && a1 < 32) t += sh.h[q][a1];
+                if (b0_ >= 0 && b0_ < 32) t += sh.h[3 + q][b0_];
+                if (b1 >= 0 && b1 < 32) t += sh.h[3 + q][b1];
+                atomicAdd(w + q, fma(c, kc[q], (double)t * sc[q]));
+              }
+            }
+          }
+        }
+        __syncwarp();
+        if (lane < 4 * (e1 - e0)) {
+          double t = (lane & 3) < 3 ? sh.s[lane][18] : 0.0;
+          float u = 0.f;
+          for (int p = 0; p < kb_steps + 2; ++p) t += sh.s[lane][p];
+          for (int p = 0; p < 32; ++p) u += sh.f[lane][p];
+          sh.S[e0 + (lane >> 2)][lane & 3] = t;
+          sh.T[e0 + (lane >> 2)][lane & 3] = u;
+        }
+        __syncwarp();
+      }
+    // ---- the far receivers' geometry, lanes = receivers ----
+    if (!all_near && lane < cnt) {
+      const int i = sh.j[lane].x, kb = sh.j[lane].y;
+      if (!(kb <= 2 && kb + kMaxBlock + 3 >= 0)) {
+        const size_t bi = b0 + (size_t)i;
+        const double *pi = a.axis + 3 * bi, *Ri = a.origin + 3 * bi;
+        const double rho[3] = {Ri[0] - Rj[0], Ri[1] - Rj[1], Ri[2] - Rj[2]};
+        const double iR = rsqrt(dot3(rho, rho));
+        const double n[3] = {rho[0] * iR, rho[1] * iR, rho[2] * iR};
+        const double c1 = dot3(n, pj), c2 = dot3(n, pi), c12 = dot3(pi, pj);
+        const double S1 = sh.S[lane][0], S2 = sh.S[lane][1] * (1.0 / kC), S3 = sh.S[lane][2] * (1.0 / (kC * kC)), S4 = sh.S[lane][3];
+        // F = ke [Q (S1 / R^3 + S2 / R^2) + (c1 c2 - c12) S3 / R], Q = 3 c1 c2 - c12
+        const double q0 = kKe * iR * iR * (S1 * iR + S2), r0 = kKe * iR * S3;
+        const double cc = 3.0 * q0 + r0;  // d / d (c1 c2)
+        const double mub = fma(unit, (double)sh.T[lane][0], cc * c2), nub = fma(unit, (double)sh.T[lane][1], cc * c1);
+        const double Q = 3.0 * c1 * c2 - c12;
+        const double Rb = -iR * (Q * kKe * iR * iR * (3.0 * S1 * iR + 2.0 * S2) + (c1 * c2 - c12) * r0) +
+                          fma(unit, (double)sh.T[lane][2] - (double)sh.T[lane][3], -S4) * iL;
+        double G[3];
+        for (int c = 0; c < 3; ++c) {
+          G[c] = iR * (mub * (pj[c] - c1 * n[c]) + nub * (pi[c] - c2 * n[c])) + Rb * n[c];
+          atomicAdd(&A.g_origin[3 * bi + c], G[c]);
+          Gj[c] -= G[c];
+        }
+      }
+    }
+    __syncwarp();
+    // ---- the others, lanes = stages ----
+    for (unsigned m = mnear; m; m &= m - 1) {
+      const int l = __ffs((int)m) - 1, i = z + a.nsplit * (t0 + l);
+      const size_t bi = b0 + (size_t)i;
+      double Rib[3] = {0.0, 0.0, 0.0}, Rjb[3] = {0.0, 0.0, 0.0};
+      if (lane < ns && !err) {
+        const double eb = A.Ebar[bi * (2 * kMaxBlock + 1) + 1 + lane];
+        if (eb != 0.0)
+          err = pair_rev_f64<false, true>(A, b, i, j, (double)n0 + (double)stage_f, n0, eb, nullptr, 0, 0, Rib, Rjb);
+      }
+      for (int c = 0; c < 3; ++c) {
+        Gj[c] += Rjb[c];
+        double t = Rib[c];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0 && t != 0.0) atomicAdd(&A.g_origin[3 * bi + c], t);
+      }
+    }
+    __syncwarp();
+  }
+  if (err) set_status(a.status, err);
+  for (int c = 0; c < 3; ++c) {
+    double t = Gj[c];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) s_rj[c][warp] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    double t = 0.0;
+    for (int w = 0; w < kRevWarps; ++w) t += s_rj[threadIdx.x][w];
+    if (t != 0.0) atomicAdd(&A.g_origin[3 * bj + threadIdx.x], t);
+  }
 }
 
 // Field-loss seed of the adjoint: L = sum over configurations b, frames f and points p of
@@ -3659,7 +3937,7 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
   const size_t edb = al(nbn * (size_t)Sg * sizeof(double));
   const size_t half = al(nbn * (size_t)(Sg - 1) * sizeof(double));
   const size_t mu_b = al(nbn * (size_t)Wg * 3 * sizeof(double));
-  const size_t small = al(nbn * (2 + 1 + (2 * kMaxBlock + 1) + 1 + 2 + 2 + 1) * sizeof(double));
+  const size_t small = al((nbn * (2 + 1 + (2 * kMaxBlock + 1) + 1 + 2 + 2 + 1) + 1) * sizeof(double));
   const size_t fit_b = rates ? 3 * al(nbn * (size_t)flen * sizeof(double)) + al(4 * nbn * sizeof(double)) : 0;
   const size_t ck_b = Cask > 0 ? al((size_t)std::max<int64_t>(nseg - 1, 0) * st_len * sizeof(double)) : 0;
   if (ctx->adj_scratch.reserve(3 * hist + edb + half + mu_b + small + fit_b + ck_b) != cudaSuccess) return PC_ERR_CUDA;
@@ -3677,6 +3955,8 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
   double *ck = Cask > 0 ? (double *)(fp_ + fit_b) : nullptr;  // state at step c C: ck + (c - 1) st_len
   const int2 *delay = nullptr;
   const double *tab = nullptr;
+  RunArgs run;
+  memset(&run, 0, sizeof(run));
   // ---- forward ----
   if (Cask == 0) {
     // the whole history and the half-step fields, in the adjoint's scratch
@@ -3691,6 +3971,7 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
     pl.motion = motion;
     pl.delay_out = &delay;
     pl.rk4tab_out = &tab;
+    pl.args_out = &run;
     if (rates) {
       pl.ke = ke;
       pl.kdd = kdd;
@@ -3758,6 +4039,8 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
   A.tau = A.w0bar + nbn;
   A.wts = A.tau + 2 * nbn;
   A.disp = A.wts + 2 * nbn;
+  A.ebmax = (unsigned long long *)(A.disp + nbn);
+  if (cudaMemsetAsync(A.ebmax, 0, sizeof(double), st) != cudaSuccess) return PC_ERR_CUDA;
   A.delay = delay;
   if (motion) {
     a.org_pos = motion->pos;
@@ -3808,6 +4091,20 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
       return PC_ERR_CUDA;
   }
   const unsigned rgrid = (unsigned)((nbn + 127) / 128);
+  // the forward run's split form (float64 forward on the grid path): its tables and mirror for the reverse
+  auto use_tables = [&]() {
+    a.pfar64 = run.pfar64;
+    a.pfarD = run.pfarD;
+    a.pgeo = run.pgeo;
+    a.H32 = run.H32;
+    a.dipf = run.dipf;
+    a.nsplit = run.nsplit;
+    a.fcp = run.fcp;
+    a.nbad = run.nbad;
+    a.max_reach = run.max_reach;
+    a.e_unit = run.e_unit;
+  };
+  use_tables();
   // recompute segment c into the segment store (its E_d at the whole and half steps with it), and
   // point the reverse's arguments at it
   auto recompute = [&](int64_t c) -> pc_status {
@@ -3826,8 +4123,10 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
     pl.swm = Wg - 1;
     pl.delay_out = &delay;
     pl.rk4tab_out = &tab;
+    pl.args_out = &run;
     pc_status rs = run_impl(ctx, dp, dt, len, &so, &ro, st, pl);
     if (rs != PC_OK) return rs;
+    use_tables();
     a.n_begin = n0;
     a.n_steps = n0 + len;
     a.rk4tab = const_cast<double *>(tab);
@@ -3873,6 +4172,19 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
     fields_adj_kernel<<<dim3((unsigned)dp->N, (unsigned)fseed->T, (unsigned)dp->B), 128, fsm, st>>>(A, *fseed, fw);
   }
   const dim3 fgrid((unsigned)dp->N, (unsigned)dp->B);
+  // the split reverse, where the run has its tables; a source's receivers over as many CTAs as have a group
+  // of 32 for each warp, up to four waves of three CTAs per SM
+  const size_t smem_split = sizeof(RevShared) * kRevWarps;
+  const bool split = a.pfar64 != nullptr && !mov;
+  if (split && cudaFuncSetAttribute(adj_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_split) !=
+                   cudaSuccess)
+    return PC_ERR_CUDA;
+  dim3 sgrid = fgrid;
+  if (split) {
+    const int64_t groups = (int64_t)((a.fcp + 31) / 32) * a.nsplit, most = (int64_t)ctx->num_sms * 12;
+    sgrid.z = (unsigned)std::max<int64_t>(1, std::min<int64_t>((groups + kRevWarps - 1) / kRevWarps,
+                                                              most / std::max<int64_t>(1, (int64_t)nbn)));
+  }
   // reverse sweep over the causal blocks, last first (segment by segment when checkpointing)
   for (int64_t c = nseg - 1; c >= 0; --c) {
     if (Cask > 0 && c < nseg - 1) {
@@ -3886,6 +4198,7 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
       const int kb = (int)std::min((int64_t)K, s1 - n0);
       adj_rk4_kernel<<<rgrid, 128, 0, st>>>(A, n0, kb);
       if (mov) adj_field_kernel<true><<<fgrid, 128, smem, st>>>(A, n0, 2 * kb, wmax);
+      else if (split) adj_split_kernel<<<sgrid, kRevWarps * 32, smem_split, st>>>(A, n0, 2 * kb);
       else adj_field_kernel<false><<<fgrid, 128, smem, st>>>(A, n0, 2 * kb, wmax);
     }
   }

@@ -96,6 +96,74 @@ __device__ __forceinline__ Cubic cubic_terms(float mu, float x, float v, float a
   return o;
 }
 
+// Reverse of cubic_terms for a loss that depends on Ca and D (the driving field): their adjoints in, those of
+// mu, x, v, al and of the three slopes out.  Checked against central differences of cubic_terms.
+struct CubicIn {
+  float mu, x, v, al, dX, dV, dA;
+};
+__device__ __forceinline__ CubicIn cubic_terms_rev(float mu, float x, float v, float al, float p, float q, float r, float Cab,
+                                                   float Db, Cubic &val) {
+  const float d1 = -mu * x, xx = x * x, xp = x * p, mm = mu * mu;
+  const float d2 = 0.5f * xx * (1.f - mm) - mm * xp, e3 = p * d2 + x * (xp + d2), d3 = mu * e3;
+  const float y2 = -d1 * p, y3 = -d2 * p, w2 = -d1 * q, w3 = -d2 * q, g2 = -d1 * r, g3 = -d2 * r;
+  const float u1 = d1 - v * mu, u2 = d2 - w2 * mu + v * x, u3 = d3 - w3 * mu + v * y2 + w2 * x;
+  const float i1 = -u1, i2 = u1 * u1 - u2, i3 = u1 * (2.f * u2 - u1 * u1) - u3;
+  const float J1 = 2.f * i1, J2 = i1 * i1 + 2.f * i2;
+  const float K1 = 3.f * i1, K2 = 3.f * (i1 * i1 + i2), K3 = 3.f * i3 + i1 * (6.f * i2 + i1 * i1);
+  const float G1 = al * mu, G2 = g2 * mu - al * x - v * v, G3 = g3 * mu - 2.f * v * w2 - al * y2 - g2 * x;
+  const float GK1 = G1 + K1, GK2 = G1 * K1 + G2 + K2;
+  const float Cb1 = -(v + al), Cb2 = -(v * GK1 + al * J1 + w2 + g2),
+              Cb3 = -(v * GK2 + w2 * GK1 + al * J2 + g2 * J1 + w3 + g3);
+  val.Ca = G2 * K1 + G1 * K2 + G3 + K3;
+  val.D = d1 * Cb2 + d2 * Cb1 + Cb3 - x * GK2 - y2 * GK1 - y3;
+  float d1b = Db * Cb2, d2b = Db * Cb1;
+  const float m = -Db * d1, Cb1b = Db * d2, n = -Db;
+  float xb = -Db * GK2, y2b = -Db * GK1;
+  const float y3b = -Db;
+  float GK2b = -Db * x + n * v, GK1b = -Db * y2 + n * w2 + m * v;
+  float vb = n * GK2 + m * GK1 - Cb1b, alb = n * J2 + m * J1 - Cb1b;
+  float w2b = n * GK1 + m, g2b = n * J1 + m, w3b = n, g3b = n;
+  const float J2b = n * al, J1b = n * g2 + m * al;
+  const float G2b = Cab * K1 + GK2b, K1b = Cab * G2 + GK2b * G1 + GK1b, G1b = Cab * K2 + GK2b * K1 + GK1b;
+  const float K2b = Cab * G1 + GK2b, G3b = Cab, K3b = Cab;
+  g3b += G3b * mu;
+  float mub = G3b * g3 + G2b * g2 + G1b * al;
+  vb -= 2.f * (G3b * w2 + G2b * v);
+  w2b -= 2.f * G3b * v;
+  alb += G1b * mu - G3b * y2 - G2b * x;
+  y2b -= G3b * al;
+  g2b += G2b * mu - G3b * x;
+  xb -= G3b * g2 + G2b * al;
+  const float i3b = 3.f * K3b;
+  const float i1b = K3b * (6.f * i2 + 3.f * i1 * i1) + 6.f * K2b * i1 + 3.f * K1b + 2.f * (J2b * i1 + J1b);
+  const float i2b = 6.f * K3b * i1 + 3.f * K2b + 2.f * J2b;
+  const float u3b = -i3b, u1b = i3b * (2.f * u2 - 3.f * u1 * u1) + 2.f * i2b * u1 - i1b, u2b = 2.f * i3b * u1 - i2b;
+  w3b -= u3b * mu;
+  mub -= u3b * w3 + u2b * w2 + u1b * v;
+  vb += u3b * y2 + u2b * x - u1b * mu;
+  y2b += u3b * v;
+  w2b += u3b * x - u2b * mu;
+  xb += u3b * w2 + u2b * v;
+  d2b += u2b - (g3b * r + w3b * q + y3b * p);
+  d1b += u1b - (g2b * r + w2b * q + y2b * p);
+  CubicIn o;
+  o.dA = -(g3b * d2 + g2b * d1);
+  o.dV = -(w3b * d2 + w2b * d1);
+  float pb = -(y3b * d2 + y2b * d1);
+  mub += u3b * e3;
+  const float t = u3b * mu;
+  pb += t * d2;
+  d2b += t * (p + x);
+  xb += t * (xp + d2);
+  const float xpb = t * x - d2b * mm, xxb = 0.5f * d2b * (1.f - mm), mmb = -d2b * (0.5f * xx + xp);
+  o.dX = pb + xpb * x;
+  o.x = xb + xpb * p + 2.f * x * xxb - d1b * mu;
+  o.mu = mub + 2.f * mu * mmb - d1b * x;
+  o.v = vb;
+  o.al = alb;
+  return o;
+}
+
 // The second-order terms, which the two charges of equal masses share: their derivative along a change of
 // (x, v, al) at fixed slopes enters where only one of the charges sees that change.
 __device__ __forceinline__ Cubic quad_terms(float mu, float x, float v, float al, float dX, float dV, float dA) {

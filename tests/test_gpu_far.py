@@ -272,3 +272,21 @@ def test_split_fields_against_binary128(ctx, case, kind):
         g = out[k][:, torch.as_tensor(p, device="cuda")].cpu().numpy()
         sc = scale["E"] / W.C if k == "B" else scale[k]
         assert np.all(norm(g - ref[k]) <= 1e-10 * np.maximum(norm(ref[k]), 1e-3 * sc)), k
+
+
+# ------------------------------------------------------------------------------------------------
+# the adjoint's split reverse (grid path)
+# ------------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("checkpoint", [0, 100])
+@pytest.mark.parametrize("N,B,steps,scale", [(66, 1, 417, 1.0), (90, 2, 300, 1.0), (130, 1, 203, 0.6), (70, 1, 64, 30.0)])
+def test_split_reverse_against_the_two_charge_form(ctx, N, B, steps, scale, checkpoint):
+    # masses one rounding apart keep every pair in the two-charge form, forward and reverse, and move the
+    # result by as much: gradients within 1e-10 of each group's largest (both forms round at 1e-12)
+    cfg = _cloud(N, B=B, seed=N)
+    cfg.origin *= scale
+    w = torch.linspace(0.5, 1.5, B * N, dtype=torch.float64, device="cuda").view(B, N)
+    got = pc.pc_dipoles_adjoint(ctx, pc.lo_config_to_device(cfg), cfg.dt, steps, w, checkpoint_every=checkpoint)
+    cfg.m1 = np.nextafter(cfg.m1, np.inf)
+    ref = pc.pc_dipoles_adjoint(ctx, pc.lo_config_to_device(cfg), cfg.dt, steps, w, checkpoint_every=checkpoint)
+    for g, r, k in zip(got, ref, ("origin", "omega0", "d0")):
+        assert float((g - r).abs().max()) < 1e-10 * float(r.abs().max()), k

@@ -32,9 +32,8 @@ typedef enum {
   PC_ERR_VELOCITY = 4,  /* a dipole charge exceeded v_max (Sec. 3.2, default c/100) */
   PC_ERR_CAUSALITY = 5, /* dt exceeds a light-crossing time between dipoles (Sec. 3.2) */
   PC_ERR_NOCONV = 6,    /* the retarded-time solve or the energy fit did not converge */
-  PC_ERR_TIMEOUT = 7    /* reserved: no kernel of this library waits on another (every ordering
-                           between blocks goes through kernel or graph-node boundaries), so no
-                           call returns it */
+  PC_ERR_TIMEOUT = 7    /* the CTAs of a cooperative oscillator run did not meet at a block's end within
+                           the barrier's limit (seconds): the run ended there, its outputs are invalid */
 } pc_status;
 
 /* field kind, Sec. 3.2 (calculate_E / calculate_B select total, Coulomb or radiation field) */
@@ -269,10 +268,11 @@ typedef struct {
  * each step d'' is set from the equation of motion at the step end.  Optionally the kinetic energy
  * m d'^2/(2 q^2) from first_index on is fitted to Eq. KE (Levenberg-Marquardt), giving gamma and
  * omega per dipole.
- * Configurations of more than 64 dipoles run as grid-wide launches per causal block, the block
- * loop one CUDA graph with a device-side while node; where that node is unavailable, or when the
- * environment variable PYCHARGE_GB300_HOST_LOOP is "1" (for profilers that do not descend into
- * conditional graph nodes), the same launches are issued from the host, with identical results.
+ * Configurations of more than 64 dipoles run their block loop as one cooperative launch (mixed up to
+ * 14 dipoles per SM over the batch, float64 up to 2) or as grid-wide launches per causal block in one
+ * CUDA graph with a device-side while node; where neither can be launched, or when the environment
+ * variable PYCHARGE_GB300_HOST_LOOP is "1" (for profilers that do not descend into conditional graph
+ * nodes), the grid-wide launches are issued from the host, with identical results.
  * Errors: PC_ERR_ARG (also B > 65535 with N > 64), PC_ERR_CAUSALITY (two dipoles closer than
  * c dt), PC_ERR_VELOCITY, PC_ERR_NOCONV, PC_ERR_CUDA.
  */

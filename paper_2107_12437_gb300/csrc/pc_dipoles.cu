@@ -17,6 +17,7 @@
 #include <cstdlib>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "pc_internal.cuh"
@@ -106,6 +107,8 @@ struct RunArgs {
   float4 *carry;
   double *carry64;    // the float64 drive's, four each
   int *nbad;
+  unsigned *bar;      // the cooperative loop's barrier
+  int mid;            // mixed far drive with mid pairs
   int K;              // the run's causal block length (grid path)
   int max_reach;      // the largest reach over the batch
   // [B][2]: largest |d0 / q| (m) and |omega0| (1/s) of a configuration (bits), for those limits
@@ -134,6 +137,11 @@ constexpr int kTab = kTabC + 13;
 constexpr double kFarGrow = 1.5;
 constexpr int kFarNone = -1, kFarNear = -2;
 constexpr double kFarDelay = 16 + 4;  // samples: a block of kMaxBlock steps reads well behind the newest one
+// Mixed drive: equal masses stay far down to X/R = kMidX with the cubic terms added (mid pairs; their fifth
+// order is 0.3 (X/R)^4, and a charge off its centre's history segment changes the pair's field by up to
+// V^2 / (4 X), which kMidCross bounds).
+constexpr float kMidX = 1e-2f, kMidCross = 4e-8f;
+constexpr int kFarMid = 1 << 30;  // flag of a mid pair's delay
 
 constexpr int kDipF = 12;
 
@@ -226,7 +234,8 @@ __device__ void rk4_table(const RunArgs &a, size_t bi) {
 // path keeps the float64 unit for its drive
 template <bool MIXED, bool HWCVT = false>
 __device__ void rk4_block_warp(const RunArgs &a, int b, int i, int64_t n0, int kb, int *stop, double *Es,
-                               double *ys = nullptr, const double *Tsh = nullptr, const float *fsc = nullptr) {
+                               double *ys = nullptr, const double *Tsh = nullptr, const float *fsc = nullptr,
+                               int bad_slot = 0) {
   const int lane = threadIdx.x & 31;
   const int64_t So = a.n_steps - a.n_begin + 1;
   const size_t bi = bidx(a, b, i);
@@ -284,7 +293,7 @@ __device__ void rk4_block_warp(const RunArgs &a, int b, int i, int64_t n0, int k
     }
     bad = fabs(yn1) > T[kTabC + 10];
     if (!HWCVT && a.nbad && !(fabs(yn0) <= T[kTabC + 11] && fabs(yn1) <= T[kTabC + 12]))
-      atomicMax(a.nbad, (int)(n + 1));
+      atomicMax(a.nbad + bad_slot, (int)(n + 1));
     if (ys && lane == kb - 1) {
       ys[0] = yn0;
       ys[1] = yn1;
@@ -495,10 +504,9 @@ __device__ float pair_drive_f32(const RunArgs &a, int b, int i, int j, int kb, f
   const HistF32Ring H{a.H32 + bj * (size_t)a.hs, RING ? (int)a.wm : -1};
   // fast path: both charges on the segment of the centre's retarded time (packed solve), then only
   // the driving-field projection p_i . E of the pair
+  float fl;
+  const int k = kb + Num<float>::floor_int(xc, fl);
   {
-    float fl;
-    const int kc = Num<float>::floor_int(xc, fl);
-    const int k = kb + kc;
     if (k < -1) {
       // the centre's retarded time lies a sample or more before t = 0; when both charges' offsets
       // (at most |s| samples) keep them there too, they rest at their first position with no
@@ -520,8 +528,9 @@ __device__ float pair_drive_f32(const RunArgs &a, int b, int i, int j, int kb, f
       float x0, v0, a0, x1, v1, a1;
       H.get_in(k, x0, v0, a0);
       H.get_in(k + 1, x1, v1, a1);
-      // the first segment may not be extended backwards, the last one only by kEndTol
-      const float lo = (k == 0) ? 0.f : -kExtrap, hi = 1.f + ((k == nvalid - 2) ? kEndTol : kExtrap);
+      // the first segment may not be extended backwards, nor it and the second across sample 1 (d'' comes
+      // up from rest within the first segment: a kink as deep as the one at t = 0), the last only by kEndTol
+      const float lo = (k <= 1) ? 0.f : -kExtrap, hi = 1.f + ((k == 0 || k == nvalid - 2) ? kEndTol : kExtrap);
       float2 X, V, Ac, dl;
       if (dip_pair_states_fast(x0, v0, a0, x1, v1, a1, xc - fl, rn, rp, cj.y, cj.z, X, V, Ac, dl, 0.5f * (lo + hi),
                                0.5f * (hi - lo)))
@@ -540,7 +549,7 @@ __device__ float pair_drive_f32(const RunArgs &a, int b, int i, int j, int kb, f
   float acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   uint8_t mk = 0;
   const int e = dipole_net<PC_TOTAL, float, HistF32Ring>(H, nvalid, kb, xc, rx, ry, rz, rn2, px, py, pz, rp2, cj.y, cj.z,
-                                                     cj.w, 0.f, false, acc, mk);
+                                                     cj.w, 0.f, k <= 1, acc, mk);
   if (e) {
     *err = (e == PC_ERR_HISTORY) ? PC_ERR_CAUSALITY : e;
     return 0.f;
@@ -770,7 +779,7 @@ __device__ __forceinline__ void drive_sources_grid(const RunArgs &a, int b, int 
       if (k >= 0 && k <= nvalid - 2) {
         const float4 cj = pc[j * (kDipF / 4)];
         const float4 h0 = hj[k & mask], h1 = hj[(k + 1) & mask];
-        const float lo = (k == 0) ? 0.f : -kExtrap, hi = 1.f + ((k == nvalid - 2) ? kEndTol : kExtrap);
+        const float lo = (k <= 1) ? 0.f : -kExtrap, hi = 1.f + ((k == 0 || k == nvalid - 2) ? kEndTol : kExtrap);
         float2 X, V, Ac, dlt;
         if (dip_pair_states_fast(h0.x, h0.y, h0.z, h1.x, h1.y, h1.z, xc, geo.x, geo.y, cj.y, cj.z, X, V, Ac, dlt,
                                  0.5f * (lo + hi), 0.5f * (hi - lo))) {
@@ -1192,7 +1201,7 @@ __global__ void lo_rstat_init_kernel(const RunArgs a) {
   a.rstat[3 * b + 2] = 0ull;
   if (a.pfarD) {
     a.amax[2 * b] = a.amax[2 * b + 1] = 0ull;
-    if (b == 0) *a.nbad = -1;
+    if (b == 0) a.nbad[0] = a.nbad[1] = -1;
   }
 }
 
@@ -1272,12 +1281,24 @@ __global__ void __launch_bounds__(256) lo_pairs_kernel(const RunArgs a) {
         if (a.pfar) {
           // p_i . E of the far form: k1 X + k2 V + k3 A
           const float m1 = (float)a.m1[bj], m2 = (float)a.m2[bj], im = 1.f / (m1 + m2);
-          const bool far = i != j && fl >= kFarDelay && g.x >= far_limit(xm, vm, m2 * im, m1 * im);
+          const bool may = i != j && fl >= kFarDelay && g.x >= a.near_L && xm <= 8.f;
+          const bool mid = a.mid && may && g.x < far_limit(xm, vm, m2 * im, m1 * im) && a.m1[bj] == a.m2[bj] && vm <= kFarV &&
+                           xm <= kMidX * g.x && 0.25f * vm * vm <= kMidCross * xm;
+          const bool far = may && (mid || g.x >= far_limit(xm, vm, m2 * im, m1 * im));
           const float q = (float)(a.q[bj] * (1.0 / kE)), ir = 1.f / g.x;
           const float cp = g.y * ir, cpi = g.z * ir;
           const float k3 = q * ir * (cp * cpi - g.w), k2 = q * ir * ir * (3.f * cp * cpi - g.w);
-          a.pfar[e] = make_float4(k2 * ir, k2, k3, (float)(x - fl));
-          a.pfarD[e] = far ? (int)fmin(fl, 1073741824.0) : (i == j ? kFarNone : kFarNear);
+          if (mid) {
+            // the largest weights: rounded once, but from the float32 geometry, as pair_drive_f32 takes it, so
+            // that the pairs that change between the two forms keep their field to the last bits of float32
+            const double ix = 1.0 / (double)g.x, qd = a.q[bj] * (1.0 / kE), c1 = (double)g.y * ix, c2 = (double)g.z * ix,
+                         c12 = (double)g.w;
+            const double k2d = qd * ix * ix * (3.0 * c1 * c2 - c12);
+            a.pfar[e] = make_float4((float)(k2d * ix), (float)k2d, (float)(qd * ix * (c1 * c2 - c12)), (float)(x - fl));
+          } else {
+            a.pfar[e] = make_float4(k2 * ir, k2, k3, (float)(x - fl));
+          }
+          a.pfarD[e] = far ? (int)fmin(fl, kFarMid - 1.0) | (mid ? kFarMid : 0) : (i == j ? kFarNone : kFarNear);
         }
       }
     }
@@ -1351,40 +1372,89 @@ __global__ void __launch_bounds__(kRunWarps * 32) lo_drive_kernel(const RunArgs 
 // (linear interpolation between samples, Sec. 3.1).  Positions K and K + 1 are positions 0 and 1 of the
 // next block, whose four sums they enter are carried over, so that a block reads K new samples per pair:
 // half a warp takes a source, lanes = positions 2 .. 17.
-// Sources that are not far go through pair_drive_f32 with lanes = stages, as in lo_drive_kernel; a far
-// source whose samples cross t = 0 in this block (the rest state before it has a kink there, which the
-// two charges' retarded times meet apart) is corrected by the difference of the two forms.
+// Sources that are not far go through pair_drive_f32 with lanes = stages, as in lo_drive_kernel.  Out of the
+// rest state before t = 0, d'' comes up within the first segment: the samples have kinks at 0 and 1, which the
+// two charges' retarded times meet apart.  Where one of them is across a kink from the centre's by o samples,
+// the form's linear continuation is off by mu o times the second difference of g there, which is added (a
+// stage or none per pair and kink; moments stay within 8 c dt, so that four samples around it are enough).
+// The two forms' whole difference there had cost 1.25 blocks of pair_drive_f32 a pair, a third of 1000 steps
+// of 4096 oscillators.
 // A block whose reach holds a sample beyond the limits (a.nbad) goes through lo_drive_kernel's sources
 // altogether; the next far block then forms the carried sums itself.
-// Measured, 4096 oscillators in a 600 nm cube: 3.10 -> 0.55 ms a block of 16 steps, about 10 warp
-// instructions per pair and block against 179; bound by the gathers of the samples (the pair tables alone,
-// 20 B a pair, take 0.05 ms from HBM).  A ring of 256: 21 -> 11.6 us a block, launch included.
+// Measured, 4096 oscillators in a 600 nm cube: 3.10 -> 0.38 ms a block of 16 steps, about 11 warp
+// instructions per pair and block against 179; bound by the gathers of the samples from L2 (272 B a pair,
+// 12 TB/s; the pair tables, 20 B a pair, take 0.05 ms from HBM).
+// MID: where the cooperative loop below runs (smaller configurations, whose near pairs are a larger part: 12 %
+// in a ring of 256), mid pairs stay in the far form and add their cubic terms at the samples: 12.2 -> 9.5 us a
+// block there with the crossings above; for larger ones its registers cost more than it saves (4096: 0.55 ->
+// 0.70 ms a block).
 // ------------------------------------------------------------------------------------------------
 struct FarSums {
   float G, H0, H2, F;
 };
+// Mid pairs: the cubic terms at a sample (X, V, A), added to its g.  The slopes that they take, per sample,
+// are V and A themselves, and none for A: the differences are (w dt) and (w R/c)^3 of terms that are 1e-4 of g.
+struct MidPair {
+  float4 p;  // cos(rho, p_j), weights of Ca and D, 1 / R
+  float4 r;  // R, f, source and base sample (bits)
+};
+__device__ __forceinline__ MidPair mid_pair(const RunArgs &a, size_t bj, float4 geo, float f, int j, int kb) {
+  const float iR = __fdividef(1.f, geo.x), w = 0.25f * a.dipf[bj * kDipF + 11] * iR * iR;
+  return {make_float4(geo.y * iR, w * geo.z * iR, w * geo.w, iR),
+          make_float4(geo.x, f, __int_as_float(j), __int_as_float(kb))};
+}
+__device__ __forceinline__ float mid_terms(float4 p, float R, float4 h) {
+  const float al = h.z * R;
+  const Cubic q = cubic_terms(p.x, h.x * p.w, h.y, al, h.y, al, 0.f);
+  return fmaf(q.Ca, p.y, q.D * p.z);
+}
 // The far sources of slice z (table rows from tab), samples at positions 2 + m + shift (m = lane & 15) of
 // the block at n0: sums per position over the slice's sources, groups of 32 compensated.  A slice takes
 // every nsplit-th source, so that the near ones, neighbours in index as often as not, spread over them.
-template <bool RING>
+// mn, mw: lane c gets the near sources of group c (32 sources) as bits and those with a charge across sample 0
+// or 1 from its centre, for the first 32 groups.
+template <bool RING, bool MID, int U>
 __device__ __forceinline__ FarSums far_sources(const RunArgs &a, size_t b0, size_t tab, int z, int n0, int shift,
-                                               float4 *s_k, int2 *s_j) {
+                                               float4 *s_k, int2 *s_j, MidPair *s_m, size_t row, unsigned &mn,
+                                               unsigned &mw) {
   const int lane = threadIdx.x & 31, half = lane >> 4;
   const char *H = reinterpret_cast<const char *>(a.H32 + b0 * (size_t)a.hs);
   const unsigned hb = (unsigned)a.hs * 16u;  // a.hs < 2^27 (the host's condition)
   const int mask = RING ? (int)a.wm : -1;
   const int pos = 2 + (lane & 15) + shift;
   FarSums S = {0.f, 0.f, 0.f, 0.f}, C = {0.f, 0.f, 0.f, 0.f};
+  mn = mw = 0;
+  float4 pk = make_float4(0.f, 0.f, 0.f, 0.f);
+  int D = kFarNone;
+  if (lane < a.fcp) {
+    D = a.pfarD[tab + lane];
+    pk = a.pfar[tab + lane];
+  }
   for (int t0 = 0; t0 < a.fcp; t0 += 32) {
     const int t = t0 + lane;
-    float4 pk = make_float4(0.f, 0.f, 0.f, 0.f);
-    int D = kFarNone;
-    if (t < a.fcp) {
-      D = a.pfarD[tab + t];
-      pk = a.pfar[tab + t];
+    const bool far = D >= 0, mid = MID && far && (D & kFarMid);
+    if (mid) D -= kFarMid;
+    const unsigned mf = __ballot_sync(0xffffffffu, far), mm = MID ? __ballot_sync(0xffffffffu, mid) : 0u;
+    if (mid) {
+      const int sl = __popc(mm & ((1u << lane) - 1u)), j = z + a.nsplit * t;
+      s_m[sl] = mid_pair(a, b0 + j, a.pgeo[row + j], pk.w, j, n0 - D - 1);
     }
-    const bool far = D >= 0;
-    const unsigned mf = __ballot_sync(0xffffffffu, far);
+    {
+      // a charge across sample 0 or 1 from its centre at a stage of this block
+      bool wave = false;
+      if (far && n0 - D <= 6 && n0 - D + a.K + 5 >= 0) {
+        const float4 gg = a.pgeo[row + z + a.nsplit * t];
+        const float x0 = reinterpret_cast<const float4 *>(H + (size_t)(unsigned)(z + a.nsplit * t) * hb)->x;
+        const float c = (float)(n0 - D) - pk.w, hd = fabsf(__fdividef(x0 * gg.y, gg.x)) + 1e-4f;
+        const float s0 = fminf(fmaxf(rintf(-2.f * c), 1.f), 2.f * a.K), s1 = fminf(fmaxf(rintf(2.f - 2.f * c), 1.f), 2.f * a.K);
+        wave = fabsf(fmaf(0.5f, s0, c)) <= hd || fabsf(fmaf(0.5f, s1, c - 1.f)) <= hd;
+      }
+      const unsigned m1 = __ballot_sync(0xffffffffu, D == kFarNear), m2 = __ballot_sync(0xffffffffu, wave);
+      if (lane == (t0 >> 5)) {
+        mn = m1;
+        mw = m2;
+      }
+    }
     const int cnt = __popc(mf);
     __syncwarp();
     if (far) {
@@ -1397,8 +1467,14 @@ __device__ __forceinline__ FarSums far_sources(const RunArgs &a, size_t b0, size
       s_j[cnt] = make_int2(z, 0);
     }
     __syncwarp();
+    // the next group's entries come in while this one's samples do
+    D = kFarNone;
+    if (t + 32 < a.fcp) {
+      D = a.pfarD[tab + t + 32];
+      pk = a.pfar[tab + t + 32];
+    }
     FarSums g = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
+#pragma unroll U
     for (int e = half; e < cnt; e += 2) {
       const float4 k = s_k[e];
       const int2 r = s_j[e];
@@ -1409,6 +1485,17 @@ __device__ __forceinline__ FarSums far_sources(const RunArgs &a, size_t b0, size
       g.H0 = fmaf(__saturatef(k.w - 0.5f), v, g.H0);
       g.H2 = fmaf(__saturatef(0.5f - k.w), v, g.H2);
       g.F = fmaf(k.w, v, g.F);
+    }
+    const int cm = __popc(mm);
+    for (int e = half; e < cm; e += 2) {
+      const float4 p = s_m[e].p, r = s_m[e].r;
+      const unsigned n = (unsigned)(max(__float_as_int(r.w) + pos, 0) & mask);
+      const float4 h = *reinterpret_cast<const float4 *>(H + (size_t)__float_as_uint(r.z) * hb + 16u * n);
+      const float v = mid_terms(p, r.x, h);
+      g.G += v;
+      g.H0 = fmaf(__saturatef(r.y - 0.5f), v, g.H0);
+      g.H2 = fmaf(__saturatef(0.5f - r.y), v, g.H2);
+      g.F = fmaf(r.y, v, g.F);
     }
     auto add = [](float &s, float &c, float x) {
       const float y = x - c, t = s + y;
@@ -1428,33 +1515,20 @@ __device__ __forceinline__ FarSums far_sources(const RunArgs &a, size_t b0, size
   return S;
 }
 
-template <bool NEAR, bool RING>
-__global__ void __launch_bounds__(kRunWarps * 32) lo_far_drive_kernel(const __grid_constant__ RunArgs a, int64_t n0_, int ns_) {
-  __shared__ double sh[kRunWarps][32];
-  __shared__ float4 s_k[kRunWarps][34];
-  __shared__ int2 s_j[kRunWarps][34];
-  if (*((volatile int *)a.status)) return;  // an earlier block failed
-  int64_t n0l = n0_;
-  int ns = ns_;
-  if (ns < 0) {
-    n0l = a.blk[0];
-    if (n0l >= a.n_steps) return;
-    ns = 2 * (int)min((int64_t)a.K, a.n_steps - n0l);
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.y;
-  const int i = blockIdx.x * kRunWarps + warp;
-  if (i >= a.N) return;
-  const int z = blockIdx.z;
+// One warp's part of a block: receiver i, source slice z, stages into dst[1 .. ns]; s_k, s_j its staging
+// buffers, sh 32 doubles; nbad the last sample beyond the limits (before this block), or -1.
+template <bool NEAR, bool RING, bool MID, int U>
+__device__ __forceinline__ void far_block(const RunArgs &a, int b, int i, int z, int64_t n0l, int ns, int nbad, double *dst,
+                                          double *sh, float4 *s_k, int2 *s_j, MidPair *s_m) {
+  const int lane = threadIdx.x & 31;
   const size_t bi = bidx(a, b, i), b0 = bidx(a, b, 0);
-  double *dst = (a.nsplit > 1 ? a.Epart + (size_t)z * a.B * a.N * (2 * kMaxBlock + 1) : a.Es) + bi * (2 * kMaxBlock + 1);
   const int n0 = (int)n0l, K = a.K;
   int err = 0;
   // (the reach is the depth of a run state too, so that a resumed run decides as the uninterrupted one)
-  const int nbad = *((volatile int *)a.nbad), back = a.max_reach;
+  const int back = a.max_reach;
   if (nbad >= 0 && n0 - back <= nbad) {
     const int j_lo = min(a.N, z * a.fcp), j_hi = min(a.N, j_lo + a.fcp);
-    drive_phase<true, NEAR, RING, true, false>(a, b, i, n0l, ns, sh[warp], &err, j_lo, j_hi, dst);
+    drive_phase<true, NEAR, RING, true, false>(a, b, i, n0l, ns, sh, &err, j_lo, j_hi, dst);
     if (err) set_status(a.status, err);
     return;
   }
@@ -1463,15 +1537,16 @@ __global__ void __launch_bounds__(kRunWarps * 32) lo_far_drive_kernel(const __gr
   // went through the other form) as positions K and K + 1 of that block
   float4 *cw = a.carry + ((size_t)z * a.B + b) * (size_t)a.N + i;
   float4 c;
+  unsigned mnl, mwl;
   if (n0l == a.n_begin || (nbad >= 0 && n0 - K - back <= nbad)) {
-    const FarSums P = far_sources<RING>(a, b0, tab, z, n0, -K, s_k[warp], s_j[warp]);
+    const FarSums P = far_sources<RING, MID, U>(a, b0, tab, z, n0, -K, s_k, s_j, s_m, row, mnl, mwl);
     const float h1 = P.G - P.H0 - P.H2;
     c = make_float4(__shfl_sync(0xffffffffu, P.H0, K - 2), __shfl_sync(0xffffffffu, P.H0, K - 1),
                     __shfl_sync(0xffffffffu, h1, K - 1), __shfl_sync(0xffffffffu, P.F, K - 1));
   } else {
     c = *cw;
   }
-  const FarSums S = far_sources<RING>(a, b0, tab, z, n0, 0, s_k[warp], s_j[warp]);
+  const FarSums S = far_sources<RING, MID, U>(a, b0, tab, z, n0, 0, s_k, s_j, s_m, row, mnl, mwl);
   const float h1 = S.G - S.H0 - S.H2;
   {
     const float4 cn = make_float4(__shfl_sync(0xffffffffu, S.H0, K - 2), __shfl_sync(0xffffffffu, S.H0, K - 1),
@@ -1483,35 +1558,45 @@ __global__ void __launch_bounds__(kRunWarps * 32) lo_far_drive_kernel(const __gr
   double accd = 0.0;
   const float stage_f = 0.5f * (__int_as_float(0x4B000000 | (lane + 1)) - 8388608.f);
   for (int t0 = 0; t0 < a.fcp; t0 += 32) {
-    const int D = t0 + lane < a.fcp ? a.pfarD[tab + t0 + lane] : kFarNone;
-    const int kb = n0 - D - 1;
-    const bool near = D == kFarNear, wave = D >= 0 && kb <= 1 && kb + K + 2 >= 0;
-    const unsigned mn = __ballot_sync(0xffffffffu, near), mw = __ballot_sync(0xffffffffu, wave);
+    unsigned mn, mw;
+    if (t0 < 1024) {
+      mn = __shfl_sync(0xffffffffu, mnl, t0 >> 5);
+      mw = __shfl_sync(0xffffffffu, mwl, t0 >> 5);
+    } else {
+      const int D = t0 + lane < a.fcp ? a.pfarD[tab + t0 + lane] : kFarNone;
+      const int kb = n0 - (D & ~kFarMid) - 1;
+      mn = __ballot_sync(0xffffffffu, D == kFarNear);
+      mw = __ballot_sync(0xffffffffu, D >= 0 && kb <= 5 && kb + K + 6 >= 0);
+    }
+    if (!(mn | mw)) continue;
     float grp = 0.f;
-    for (unsigned m = mn | mw; m; m &= m - 1) {
+    for (unsigned m = mn; m; m &= m - 1) {
       const int l = __ffs((int)m) - 1, j = z + a.nsplit * (t0 + l);
       if (lane >= ns) continue;
       const int2 dl = a.delay[row + j];
       const float4 geo = a.pgeo[row + j];
       const float xs = stage_f - __int_as_float(dl.y);
       float flf;
-      const int fl = Num<float>::floor_int(xs, flf);
-      const int k = n0 - dl.x + fl;
-      const float th = xs - flf;
-      if (NEAR && geo.x < a.near_L) {
+      const int k = n0 - dl.x + Num<float>::floor_int(xs, flf);
+      if (NEAR && geo.x < a.near_L)
         accd += pair_drive_f64(a, b, i, j, (double)n0 + (double)stage_f, n0, k, &err, 0, 2);
-        if (!((mw >> l) & 1u)) continue;
-      } else {
-        grp += pair_drive_f32<RING>(a, b, i, j, k, th, geo, n0 + 1, &err);
-      }
-      if ((mw >> l) & 1u) {
-        const float4 *hj = a.H32 + (b0 + (size_t)j) * (size_t)a.hs;
-        const int mask = RING ? (int)a.wm : -1;
-        const float4 h0 = hj[max(k, 0) & mask], h1_ = hj[max(k + 1, 0) & mask], pk = a.pfar[tab + t0 + l];
-        const float v0 = fmaf(pk.z, h0.z, fmaf(pk.y, h0.y, pk.x * h0.x));
-        const float v1 = fmaf(pk.z, h1_.z, fmaf(pk.y, h1_.y, pk.x * h1_.x));
-        grp -= fmaf(th, v1 - v0, v0);
-      }
+      else
+        grp += pair_drive_f32<RING>(a, b, i, j, k, xs - flf, geo, n0 + 1, &err);
+    }
+    for (unsigned m = mw; m; m &= m - 1) {
+      const int l = __ffs((int)m) - 1, j = z + a.nsplit * (t0 + l);
+      const int2 dl = a.delay[row + j];
+      const float4 geo = a.pgeo[row + j], pk = a.pfar[tab + t0 + l];
+      const float4 cj = *reinterpret_cast<const float4 *>(a.dipf + (b0 + j) * kDipF + 8);  // (p_z, mu+, mu-, q/e)
+      const float4 *hj = a.H32 + (b0 + (size_t)j) * (size_t)a.hs;
+      const float4 h0 = hj[0], h1_ = hj[1], h2_ = hj[2];
+      // the charge whose offset points at the sample from the centre's retarded time passes it by o samples
+      const float xs = (float)(n0 - dl.x) + (stage_f - __int_as_float(dl.y)), sx = __fdividef(h0.x * geo.y, geo.x);
+      const float w0 = (xs < 0.f) == (sx > 0.f) ? cj.y : cj.z, w1 = (xs < 1.f) == (sx > 0.f) ? cj.y : cj.z;
+      const float o0 = fmaf(w0, fabsf(sx), -fabsf(xs)), o1 = fmaf(w1, fabsf(sx), -fabsf(xs - 1.f));
+      if (o0 > 0.f && n0 > 0) grp += w0 * o0 * fmaf(pk.z, h1_.z, fmaf(pk.y, h1_.y, pk.x * (h1_.x - h0.x)));
+      if (o1 > 0.f && n0 > 1)
+        grp += w1 * o1 * fmaf(pk.z, h2_.z - 2.f * h1_.z, fmaf(pk.y, h2_.y - 2.f * h1_.y, pk.x * ((h2_.x - h1_.x) - (h1_.x - h0.x))));
     }
     const float y = grp - comp;
     const float t = accf + y;
@@ -1534,6 +1619,29 @@ __global__ void __launch_bounds__(kRunWarps * 32) lo_far_drive_kernel(const __gr
   }
 }
 
+// the block at hand: the launch's, or with ns < 0 the device cursor's; false where there is none
+__device__ __forceinline__ bool block_at(const RunArgs &a, int64_t &n0, int &ns) {
+  if (*((volatile int *)a.status)) return false;  // an earlier block failed
+  if (ns < 0) {
+    n0 = a.blk[0];
+    if (n0 >= a.n_steps) return false;
+    ns = 2 * (int)min((int64_t)a.K, a.n_steps - n0);
+  }
+  return true;
+}
+template <bool NEAR, bool RING, bool MID>
+__global__ void __launch_bounds__(kRunWarps * 32) lo_far_drive_kernel(const __grid_constant__ RunArgs a, int64_t n0, int ns) {
+  __shared__ double sh[kRunWarps][32];
+  __shared__ float4 s_k[kRunWarps][34];
+  __shared__ int2 s_j[kRunWarps][34];
+  __shared__ MidPair s_m[MID ? kRunWarps : 1][32];
+  if (!block_at(a, n0, ns)) return;
+  const int warp = threadIdx.x >> 5, b = blockIdx.y, i = blockIdx.x * kRunWarps + warp, z = blockIdx.z;
+  if (i >= a.N) return;
+  double *dst = a.nsplit > 1 ? a.Epart + (size_t)z * a.B * a.N * (2 * kMaxBlock + 1) : a.Es;
+  far_block<NEAR, RING, MID, 4>(a, b, i, z, n0, ns, *((volatile int *)a.nbad), dst + bidx(a, b, i) * (2 * kMaxBlock + 1), sh[warp], s_k[warp], s_j[warp],
+                                s_m[MID ? warp : 0]);
+}
 
 // ------------------------------------------------------------------------------------------------
 // The same for the float64 drive, in the split form (pc_far_f32.cuh): the linear part as in
@@ -1601,32 +1709,16 @@ __device__ __forceinline__ void far_halves64(FarSums64 &S) {
 }
 
 template <bool RING>
-__global__ void __launch_bounds__(kRunWarps * 32)
-    lo_far64_drive_kernel(const __grid_constant__ RunArgs a, int64_t n0_, int ns_) {
-  __shared__ double sh[kRunWarps][32];
-  __shared__ FarEntry64 s_k[kRunWarps][34];
-  __shared__ int2 s_j[kRunWarps][34];
-  if (*((volatile int *)a.status)) return;  // an earlier block failed
-  int64_t n0l = n0_;
-  int ns = ns_;
-  if (ns < 0) {
-    n0l = a.blk[0];
-    if (n0l >= a.n_steps) return;
-    ns = 2 * (int)min((int64_t)a.K, a.n_steps - n0l);
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.y;
-  const int i = blockIdx.x * kRunWarps + warp;
-  if (i >= a.N) return;
-  const int z = blockIdx.z;
+__device__ __forceinline__ void far64_block(const RunArgs &a, int b, int i, int z, int64_t n0l, int ns, int nbad, double *dst,
+                                            double *sh, FarEntry64 *s_k, int2 *s_j) {
+  const int lane = threadIdx.x & 31;
   const size_t bi = bidx(a, b, i), b0 = bidx(a, b, 0);
-  double *dst = (a.nsplit > 1 ? a.Epart + (size_t)z * a.B * a.N * (2 * kMaxBlock + 1) : a.Es) + bi * (2 * kMaxBlock + 1);
   const int n0 = (int)n0l, K = a.K;
   int err = 0;
-  const int nbad = *((volatile int *)a.nbad), back = a.max_reach;
+  const int back = a.max_reach;
   if (nbad >= 0 && n0 - back <= nbad) {
     const int j_lo = min(a.N, z * a.fcp), j_hi = min(a.N, j_lo + a.fcp);
-    drive_phase<false>(a, b, i, n0l, ns, sh[warp], &err, j_lo, j_hi, dst);
+    drive_phase<false>(a, b, i, n0l, ns, sh, &err, j_lo, j_hi, dst);
     if (err) set_status(a.status, err);
     return;
   }
@@ -1638,8 +1730,8 @@ __global__ void __launch_bounds__(kRunWarps * 32)
     FarSums64 P = {0.0, 0.0, 0.0, 0.0};
     int D;
     for (int t0 = 0; t0 < a.fcp; t0 += 32) {
-      const int cnt = far_stage64(a, tab, z, t0, n0, s_k[warp], s_j[warp], D);
-      far_group64<RING>(a, b0, cnt, pos - K, s_k[warp], s_j[warp], P);
+      const int cnt = far_stage64(a, tab, z, t0, n0, s_k, s_j, D);
+      far_group64<RING>(a, b0, cnt, pos - K, s_k, s_j, P);
     }
     far_halves64(P);
     c0 = __shfl_sync(0xffffffffu, P.H0, K - 2);
@@ -1660,15 +1752,15 @@ __global__ void __launch_bounds__(kRunWarps * 32)
   const int mask = RING ? (int)a.wm : -1;
   for (int t0 = 0; t0 < a.fcp; t0 += 32) {
     int D;
-    const int cnt = far_stage64(a, tab, z, t0, n0, s_k[warp], s_j[warp], D);
-    far_group64<RING>(a, b0, cnt, pos, s_k[warp], s_j[warp], S);
+    const int cnt = far_stage64(a, tab, z, t0, n0, s_k, s_j, D);
+    far_group64<RING>(a, b0, cnt, pos, s_k, s_j, S);
     const int kb0 = n0 - D - 1;
     const bool near = D == kFarNear, wave = D >= 0 && kb0 <= 2 && kb0 + K + 3 >= 0;
     const unsigned mn = __ballot_sync(0xffffffffu, near), mw = __ballot_sync(0xffffffffu, wave);
     if (lane < ns) {
       float grp = 0.f;
       for (int e = 0; e < cnt; ++e) {
-        const int2 r = s_j[warp][e];
+        const int2 r = s_j[e];
         const int kb = r.y;
         if (kb <= 2 && kb + K + 3 >= 0) continue;  // crossing t = 0: below
         const size_t ij = row + (size_t)r.x;
@@ -1690,7 +1782,7 @@ __global__ void __launch_bounds__(kRunWarps * 32)
         const float hd = 0.5f * fabsf(X * mu);
         const float o = fmaxf(hd - th, 0.f), o1 = fmaxf(th + hd - 1.f, 0.f);
         if (o > 0.f || o1 > 0.f) {
-          const FarEntry64 &kk = s_k[warp][e];
+          const FarEntry64 &kk = s_k[e];
           const int m = o > 0.f ? k : k + 1;  // the sample between the two segments
           const size_t nm = hrow + (size_t)(max(m - 1, 0) & (int)mask), n_ = hrow + (size_t)(max(m, 0) & (int)mask),
                        np = hrow + (size_t)(max(m + 1, 0) & (int)mask);
@@ -1746,6 +1838,127 @@ __global__ void __launch_bounds__(kRunWarps * 32)
     dst[1 + 2 * t] = ((x0 + xm) + S.H2) + mh;
     dst[2 + 2 * t] = (fm + (S.G - S.F)) + mw_;
   }
+}
+
+template <bool RING>
+__global__ void __launch_bounds__(kRunWarps * 32)
+    lo_far64_drive_kernel(const __grid_constant__ RunArgs a, int64_t n0, int ns) {
+  __shared__ double sh[kRunWarps][32];
+  __shared__ FarEntry64 s_k[kRunWarps][34];
+  __shared__ int2 s_j[kRunWarps][34];
+  if (!block_at(a, n0, ns)) return;
+  const int warp = threadIdx.x >> 5, b = blockIdx.y, i = blockIdx.x * kRunWarps + warp, z = blockIdx.z;
+  if (i >= a.N) return;
+  double *dst = a.nsplit > 1 ? a.Epart + (size_t)z * a.B * a.N * (2 * kMaxBlock + 1) : a.Es;
+  far64_block<RING>(a, b, i, z, n0, ns, *((volatile int *)a.nbad), dst + bidx(a, b, i) * (2 * kMaxBlock + 1), sh[warp], s_k[warp], s_j[warp]);
+}
+
+// ------------------------------------------------------------------------------------------------
+// The grid path's whole block loop in one cooperative launch (a CTA per SM at most, all resident), for the
+// far and split drives of up to kCoopRecv receivers a CTA (2128 on 152 SMs; kCoopRecv64 in float64).  A CTA
+// owns its receivers: their (receiver, slice) parts go to its warps as they come free, the slices' sums and
+// the RK4 steps follow from shared memory, then one grid-wide barrier a block, after which the appended
+// samples are visible.  Same functions and orders as the per-block kernels, bitwise the same results.
+// A block of a few hundred receivers is bound by latency (the gathers, the pair's and RK4's dependent
+// chains, the barrier), to which three kernels and the loop's condition added as much again.
+// Measured, us a block of 16 steps, graph of kernels -> here (the ring's neighbours as mid pairs on both sides;
+// as near ones, as they are, the ring of 256 takes 9.5): ring of 66 12.7 -> 7.1, 256 14.9 -> 8.2, 700 32.4 ->
+// 28.2, 1216 50.9 -> 39.5, 2000 117 -> 107, cloud of 256 15.2 -> 8.6, of 1500 72 -> 66, of 2000 117 -> 121; float64
+// ring of 256 109 -> 102, clouds of 400 and more slower (215 -> 230): their near pairs' float64 work balances
+// better over the whole grid's warps.  16 warps with eight gathers in flight each: 20 and 24 warps of fewer
+// registers and four gathers were 0 to 20 % slower.
+// The barrier's wait is bounded: a CTA that gives up sets PC_ERR_TIMEOUT.  A CTA that sees an error leaves,
+// and the others do not wait for it.
+// ------------------------------------------------------------------------------------------------
+constexpr int kCoopWarps = 16, kCoopRecv = 14, kCoopRecv64 = 2;
+constexpr unsigned kCoopSpins = 1u << 24;  // polls, of half a microsecond or more
+struct CoopRecv {
+  double Es[2 * kMaxBlock + 1], ys[2], tab[kTab];
+  float fsc[3];
+};
+// MODE 0: mixed, 1: mixed with near float64 sources, 2: float64
+template <int MODE, bool RING>
+__global__ void __launch_bounds__(kCoopWarps * 32, 1) lo_coop_kernel(const __grid_constant__ RunArgs a, int recv) {
+  extern __shared__ double dyn[];
+  __shared__ double sh[kCoopWarps][32];
+  __shared__ typename std::conditional<MODE == 2, FarEntry64, float4>::type s_k[kCoopWarps][34];
+  __shared__ int2 s_j[kCoopWarps][34];
+  __shared__ MidPair s_m[MODE == 2 ? 1 : kCoopWarps][32];
+  __shared__ int s_stop, s_nbad, s_next;
+  CoopRecv *rc = reinterpret_cast<CoopRecv *>(dyn);
+  double *part = dyn + (sizeof(CoopRecv) * recv + 7) / 8;  // [recv][nsplit][2 kMaxBlock + 1]
+  constexpr int kRow = 2 * kMaxBlock + 1;
+  const int64_t nbn = (int64_t)a.B * a.N;
+  const int64_t c0 = (int64_t)blockIdx.x * recv;
+  const int nr = (int)max((int64_t)0, min((int64_t)recv, nbn - c0));
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int r = 0; r < nr; ++r) {
+    const size_t bi = (size_t)(c0 + r);
+    for (int t = threadIdx.x; t < kTab; t += blockDim.x) rc[r].tab[t] = a.rk4tab[bi * kTab + t];
+    if (threadIdx.x == 0) {
+      const size_t sl = bi * (size_t)a.hs + (a.n_begin & a.wm);
+      rc[r].ys[0] = a.d[sl];
+      rc[r].ys[1] = a.dd[sl];
+      rc[r].Es[0] = a.Es[bi * kRow];
+      for (int c = 0; c < 3; ++c) rc[r].fsc[c] = dbl2flt(a.rk4tab[bi * kTab + kTabC + 4 + c]);
+    }
+  }
+  if (threadIdx.x == 0) {
+    s_stop = *((volatile int *)a.status);
+    s_nbad = *((volatile int *)a.nbad);
+    s_next = kCoopWarps;
+  }
+  __syncthreads();
+  unsigned phase = 0;
+  for (int64_t n0 = a.n_begin; n0 < a.n_steps && !s_stop; n0 += a.K) {
+    const int kb = (int)min((int64_t)a.K, a.n_steps - n0);
+    // (a slice with near sources takes longer than the others: the warps take the parts as they come)
+    for (int t = warp; t < nr * a.nsplit;) {
+      const int r = t / a.nsplit, z = t % a.nsplit;
+      const int b = (int)((c0 + r) / a.N), i = (int)((c0 + r) % a.N);
+      double *dst = part + (size_t)t * kRow;
+      if constexpr (MODE == 2) far64_block<RING>(a, b, i, z, n0, 2 * kb, s_nbad, dst, sh[warp], s_k[warp], s_j[warp]);
+      else far_block<MODE == 1, RING, true, 8>(a, b, i, z, n0, 2 * kb, s_nbad, dst, sh[warp], s_k[warp], s_j[warp],
+                                           s_m[warp]);
+      if (lane == 0) t = atomicAdd(&s_next, 1);
+      t = __shfl_sync(0xffffffffu, t, 0);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_next = kCoopWarps;
+    for (int r = warp; r < nr; r += kCoopWarps) {
+      if (lane < 2 * kb) {
+        double t = 0.0;
+        for (int z = 0; z < a.nsplit; ++z) t += part[((size_t)r * a.nsplit + z) * kRow + 1 + lane];
+        rc[r].Es[1 + lane] = t;
+      }
+      __syncwarp();
+      int stop = 0;
+      rk4_block_warp<true>(a, (int)((c0 + r) / a.N), (int)((c0 + r) % a.N), n0, kb, &stop, rc[r].Es, rc[r].ys, rc[r].tab,
+                           rc[r].fsc, 1 - (int)(phase & 1));
+    }
+    // every thread's samples before the arrival, the others' after the wait
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const unsigned want = (phase + 1) * gridDim.x;
+      atomicAdd(a.bar, 1u);
+      for (unsigned seen, spins = 0;; ++spins) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.bar) : "memory");
+        // (a CTA that leaves on an error does not arrive again: the others must not wait for it)
+        if ((int)(seen - want) >= 0 || *((volatile int *)a.status)) break;
+        if (spins > kCoopSpins) set_status(a.status, PC_ERR_TIMEOUT);
+      }
+      __threadfence();
+      s_stop = *((volatile int *)a.status);
+      // a block's RK4 steps mark samples beyond the limits in the slot of its parity: this block's is not
+      // written again before the next but one, which waits for this CTA
+      s_nbad = max(s_nbad, *((volatile int *)a.nbad + (1 - (int)(phase & 1))));
+    }
+    ++phase;
+    __syncthreads();
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicMax(a.nbad, s_nbad);
+  for (int r = threadIdx.x; r < nr; r += blockDim.x) a.Es[(size_t)(c0 + r) * kRow] = rc[r].Es[0];
 }
 
 // Sum of the slices' partial stage fields (fixed order) into Es[lo..hi].
@@ -2345,9 +2558,47 @@ static void *block_drive_kernel_for(const RunArgs &a, bool mixed) {
   if (!a.pfarD) return drive_kernel_for(a, mixed);
   if (!mixed) return a.wm >= 0 ? (void *)lo_far64_drive_kernel<true> : (void *)lo_far64_drive_kernel<false>;
   const bool ring = a.wm >= 0;
+  if (a.near_L > 0.f && a.mid)
+    return ring ? (void *)lo_far_drive_kernel<true, true, true> : (void *)lo_far_drive_kernel<true, false, true>;
   if (a.near_L > 0.f)
-    return ring ? (void *)lo_far_drive_kernel<true, true> : (void *)lo_far_drive_kernel<true, false>;
-  return ring ? (void *)lo_far_drive_kernel<false, true> : (void *)lo_far_drive_kernel<false, false>;
+    return ring ? (void *)lo_far_drive_kernel<true, true, false> : (void *)lo_far_drive_kernel<true, false, false>;
+  if (a.mid) return ring ? (void *)lo_far_drive_kernel<false, true, true> : (void *)lo_far_drive_kernel<false, false, true>;
+  return ring ? (void *)lo_far_drive_kernel<false, true, false> : (void *)lo_far_drive_kernel<false, false, false>;
+}
+static void *coop_kernel_for(const RunArgs &a, bool mixed) {
+  const bool ring = a.wm >= 0;
+  if (!mixed) return ring ? (void *)lo_coop_kernel<2, true> : (void *)lo_coop_kernel<2, false>;
+  if (a.near_L > 0.f) return ring ? (void *)lo_coop_kernel<1, true> : (void *)lo_coop_kernel<1, false>;
+  return ring ? (void *)lo_coop_kernel<0, true> : (void *)lo_coop_kernel<0, false>;
+}
+// Receivers per CTA of the cooperative loop, 0 where the loop of graph nodes is faster
+static int coop_recv(const pc_ctx *ctx, size_t nbn, bool mixed) {
+  const size_t r = (nbn + ctx->num_sms - 1) / ctx->num_sms;
+  return r <= (size_t)(mixed ? kCoopRecv : kCoopRecv64) ? (int)r : 0;
+}
+static size_t coop_smem(int recv, int nsplit) {
+  return ((sizeof(CoopRecv) * recv + 7) / 8 + (size_t)recv * nsplit * (2 * kMaxBlock + 1)) * sizeof(double);
+}
+// The loop in one cooperative launch; a PC_ERR_CUDA, before anything ran, where it cannot be launched.
+static pc_status launch_coop_loop(pc_ctx *ctx, const RunArgs &a, bool mixed, cudaStream_t st) {
+  const int64_t nbn = (int64_t)a.B * a.N;
+  const int recv = coop_recv(ctx, (size_t)nbn, mixed);
+  const size_t smem = coop_smem(recv, a.nsplit);
+  if (!a.pfarD || recv == 0 || smem > 150 * 1024) return PC_ERR_CUDA;
+  void *fn = coop_kernel_for(a, mixed);
+  int coop = 0, occ = 0;
+  if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device) != cudaSuccess || !coop ||
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kCoopWarps * 32, smem) != cudaSuccess || occ < 1)
+    return PC_ERR_CUDA;
+  RunArgs aa = a;
+  int rr = recv;
+  void *args[] = {&aa, &rr};
+  if (cudaMemsetAsync(a.bar, 0, sizeof(unsigned), st) != cudaSuccess) return PC_ERR_CUDA;
+  return cudaLaunchCooperativeKernel(fn, dim3((unsigned)((nbn + recv - 1) / recv)), dim3(kCoopWarps * 32), args, smem, st) ==
+                 cudaSuccess
+             ? PC_OK
+             : PC_ERR_CUDA;
 }
 static void *run_kernel_for(const RunArgs &a, bool mixed) {
   if (!mixed) return (void *)lo_run_kernel<false>;
@@ -2536,8 +2787,11 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   // the far form's tables (mixed grid path with fixed origins); without the memory for them the run
   // takes the two-charge form throughout
   // eight source slices per receiver (4096 oscillators, 1000 steps: 49, 41, 37, 37, 39 and 44 ms with 2, 4,
-  // 8, 16, 32 and 64; 1024: 5.3, 5.0, 4.45, 4.5, 5.0 with 2, 4, 8, 16 and 32), or as set or tuned
-  const int far_split = std::min(kMaxSplit, std::min(ctx->run_slices > 0 ? ctx->run_slices : 8, std::max(1, dp->N / 8)));
+  // 8, 16, 32 and 64 before the crossings were cheap), or as set or tuned; in the cooperative loop so many
+  // that they fill its 16 warps evenly
+  const int recv = pc::coop_recv(ctx, nbn, mixed);
+  const int even = recv == 0 ? 8 : std::max(4, 16 / (recv & -recv));
+  const int far_split = std::min(kMaxSplit, std::min(ctx->run_slices > 0 ? ctx->run_slices : even, std::max(1, dp->N / 8)));
   const int far_cp = (dp->N + far_split - 1) / far_split;
   const size_t far_n = nbn * (size_t)far_split * far_cp;
   const size_t far_off = od_off + od_bytes, pf_bytes = al(far_n * (mixed ? sizeof(float4) : sizeof(FarK64)));
@@ -2599,9 +2853,11 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
     a.carry64 = (double *)a.carry;
     a.amax = (unsigned long long *)(f + pf_bytes + pd_bytes + cr_bytes);
     a.nbad = (int *)(f + pf_bytes + pd_bytes + cr_bytes + am_bytes);
+    a.bar = (unsigned *)(a.nbad + 16);
     if (!mixed) a.pgeo = (float4 *)(f + pf_bytes + pd_bytes + cr_bytes + am_bytes + 256);
     a.fcp = far_cp;
     a.nsplit = far_split;
+    a.mid = mixed && recv > 0;
     // entries past the last source stay kFarNone
     if (cudaMemsetAsync(a.pfarD, 0xff, far_n * sizeof(int), st) != cudaSuccess) return PC_ERR_CUDA;
   }
@@ -2772,8 +3028,14 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
       // descend into conditional graph nodes see every launch)
       // (and always when the launches are timed, pc_set_run_timing: an event pair around each)
       const char *hl = getenv("PYCHARGE_GB300_HOST_LOOP");
-      pc_status gs = (timed || (hl && hl[0] == '1')) ? PC_ERR_CUDA
-                                                     : pc::launch_block_loop(ctx, a, mixed, dgrid, rgrid, st);
+      pc_status gs = PC_ERR_CUDA;
+      if (!timed && !(hl && hl[0] == '1')) {
+        gs = pc::launch_coop_loop(ctx, a, mixed, st);
+        if (gs != PC_OK) {
+          cudaGetLastError();
+          gs = pc::launch_block_loop(ctx, a, mixed, dgrid, rgrid, st);
+        }
+      }
       if (gs != PC_OK) {
         cudaGetLastError();
         int nev = 0;

@@ -178,6 +178,73 @@ def test_far_drive_refuses_what_is_not_a_number(ctx):
         pc.pc_dipoles_run(ctx, pc.lo_config_to_device(cfg), cfg.dt, 400, precision=pc.PC_MIXED)
 
 
+@pytest.mark.parametrize("amp,near", [(1e-12, 0.0), (1.9e-11, 0.0), (2.8e-11, 0.0), (2.8e-11, 20e-9)])
+def test_mid_pairs_against_float64(ctx, amp, near):
+    # pairs from 20 samples (6 nm) on with charges up to 1.5 amp / 6 nm = 7e-3 of their distance apart, below
+    # where the cubic form ends (1e-2) and where charges are too fast (2.86e-11 m); the bounds above
+    cfg = _cloud(200, cell=10.2e-9, seed=7)
+    cfg.d0[:] = W.E_CHARGE * amp
+    cfg.m1[0, ::7] *= 1.5  # and sources that never are mid pairs
+    lod = pc.lo_config_to_device(cfg)
+    f = pc.pc_dipoles_run(ctx, lod, cfg.dt, 340, precision=pc.PC_F64, want_Ed=True)
+    m = pc.pc_dipoles_run(ctx, lod, cfg.dt, 340, precision=pc.PC_MIXED, near_f64=near, want_Ed=True)
+    assert _err(m["Ed"], f["Ed"]) < 3e-6
+    assert _err(m["d"], f["d"]) < 1e-9
+
+
+# ------------------------------------------------------------------------------------------------
+# the grid path's block loop in one cooperative launch
+# ------------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("N,B,precision,near,steps", [
+    (65, 1, "mixed", 0.0, 203), (153, 1, "mixed", 60e-9, 203), (90, 3, "mixed", 0.0, 333), (307, 1, "mixed", 0.0, 16),
+    (2128, 1, "mixed", 0.0, 40), (65, 1, "f64", 0.0, 203), (304, 1, "f64", 0.0, 50), (90, 2, "f64", 0.0, 333)])
+def test_cooperative_loop_is_the_loop_of_launches(ctx, monkeypatch, N, B, precision, near, steps):
+    # one, two and up to fourteen receivers a CTA, a last CTA with fewer, receivers of two configurations in a
+    # CTA, a single block, a partial last one; both stores; resumed from a state with samples beyond the
+    # limits, which the blocks must notice at the same ones
+    cfg = _cloud(N, B=B, seed=N)
+    lod = pc.lo_config_to_device(cfg)
+    kw = dict(precision=pc.PC_MIXED if precision == "mixed" else pc.PC_F64, near_f64=near)
+    state = torch.zeros(pc.pc_dipoles_state_size(ctx, lod, cfg.dt), dtype=torch.float64, device="cuda")
+
+    def runs():
+        full = pc.pc_dipoles_run(ctx, lod, cfg.dt, steps, want_Ed=True, **kw)
+        ring = pc.pc_dipoles_run(ctx, lod, cfg.dt, steps, want_history=False, state_out=state, **kw)
+        D = int(state[2])
+        state[4 + B * N:].view(B * N, D + 1, 3)[:3, -5:-3] *= 4.0
+        back = pc.pc_dipoles_run(ctx, lod, cfg.dt, steps, state_in=state, want_Ed=True, **kw)
+        return [r[k].clone() for r in (full, ring, back) for k in sorted(r) if torch.is_tensor(r[k])] + [state.clone()]
+
+    got = runs()
+    monkeypatch.setenv("PYCHARGE_GB300_HOST_LOOP", "1")
+    for g, h in zip(got, runs()):
+        assert torch.equal(g, h)
+
+
+def test_cooperative_runs_on_two_streams(ctx):
+    # two threads with a context and a stream each, at the same time
+    import threading
+
+    cfgs = [_cloud(180, seed=1), _cloud(250, seed=2)]
+    lods = [pc.lo_config_to_device(c) for c in cfgs]
+    ref = [pc.pc_dipoles_run(ctx, lo, 1e-18, 400, precision=pc.PC_MIXED)["d"].clone() for lo in lods]
+    torch.cuda.synchronize()
+    out = [None, None]
+
+    def work(k):
+        c, st = pc.Context(0), torch.cuda.Stream()
+        with torch.cuda.stream(st):
+            for _ in range(5):
+                out[k] = pc.pc_dipoles_run(c, lods[k], 1e-18, 400, precision=pc.PC_MIXED, stream=st)["d"]
+        st.synchronize()
+        c.close()
+
+    t = [threading.Thread(target=work, args=(k,)) for k in (0, 1)]
+    [x.start() for x in t]
+    [x.join() for x in t]
+    assert all(torch.equal(o, r) for o, r in zip(out, ref))
+
+
 # ------------------------------------------------------------------------------------------------
 # the oscillator run's split drive (grid path, float64)
 # ------------------------------------------------------------------------------------------------

@@ -1268,7 +1268,7 @@ __global__ void __launch_bounds__(256) lo_pairs_kernel(const RunArgs a) {
         if (a.pfar64) {
           // p_i . E of the split form's linear part, with the charge's unit and the samples' scales:
           // k1 d + k2 d' + k3 d'' is the field in V/m
-          const bool far = i != j && fl >= kFarDelay && a.m1[bj] == a.m2[bj] && xd <= kSplitX * x &&
+          const bool far = i != j && fl >= kFarDelay && a.m1[bj] == a.m2[bj] && xd <= kSplitX * x && xd <= 8.0 &&
                            xd * __longlong_as_double((long long)a.amax[2 * b + 1]) * a.dt <= kSplitV;
           const double ir = 1.0 / r, c1 = (dx * pj_[0] + dy * pj_[1] + dz * pj_[2]) * ir,
                        c2 = (dx * pi_[0] + dy * pi_[1] + dz * pi_[2]) * ir,
@@ -1648,13 +1648,14 @@ __global__ void __launch_bounds__(kRunWarps * 32) lo_far_drive_kernel(const __gr
 // lo_far_drive_kernel in float64 on the float64 history, and the cubic terms, smaller by (X/R)^2, in
 // float32 with lanes = stages on the history's float32 mirror.  Where a charge's own retarded time falls
 // just outside the segment of the centre's (by o samples, at most half its offset), its state differs from
-// that segment's extension by o times the second difference of the samples: that term in float64.  Sources
-// crossing t = 0, where the second difference is not small, are corrected by the difference of
-// pair_drive_f64 and the linear part instead.
-// Measured: a cloud of 1000 oscillators, 320 steps 316 -> 12.7 ms, a ring of 256, 1000 steps 63.4 -> 7.0 ms.  A
+// that segment's extension by o times the second difference of the samples: that term in float64.  At the
+// kinks at samples 0 and 1, where the second difference is not small, a source that may have a charge across
+// one at a stage of the block (far_crosses64) is corrected by the difference of pair_drive_f64 and the linear
+// part instead.  (All sources within a block of t = 0 had been: 1.3 blocks a pair, a fifth of 1000 steps.)
+// Measured: a cloud of 1000 oscillators, 320 steps 316 -> 12.7 ms, a ring of 256, 1000 steps 63.4 -> 5.1 ms.  A
 // far pair costs 7 float64 instructions per two of them and 16 positions and about 170 float32 ones per 32
 // stages, a near one about 280 float64 ones per 32 stages: the ring is bound by its 10 near pairs a
-// receiver.  E_d against binary128 on a cloud of 400: 1.4e-12 rms (3.9e-12 with two charges throughout).
+// receiver.  E_d against binary128 on a cloud of 400: 4.6e-13 rms (3.9e-12 with two charges throughout).
 // ------------------------------------------------------------------------------------------------
 struct FarSums64 {
   double G, H0, H2, F;
@@ -1701,6 +1702,15 @@ __device__ __forceinline__ int far_stage64(const RunArgs &a, size_t tab, int z, 
   __syncwarp();
   return cnt;
 }
+// Whether at a stage of the block at n0 a charge of a far source may be across sample 0 or 1 from its centre
+// (kinks of the history, see above): x0 its first sample's X, geo the pair's geometry with rho.p_j in rp.
+__device__ __forceinline__ bool far_crosses64(float x0, float R, float rp, int nD, float f) {
+  const float c = (float)nD - f, iR = __fdividef(1.f, R);
+  const float hd = fabsf(0.5f * x0 * rp * iR) + x0 * x0 * iR + 1e-3f;
+  const float s0 = fminf(fmaxf(rintf(-2.f * c), 1.f), 2.f * kMaxBlock), s1 = fminf(fmaxf(rintf(2.f - 2.f * c), 1.f), 2.f * kMaxBlock);
+  return fabsf(fmaf(0.5f, s0, c)) <= hd || fabsf(fmaf(0.5f, s1, c - 1.f)) <= hd;
+}
+__device__ __forceinline__ bool far_reaches_start(int nD) { return nD <= 6 && nD + kMaxBlock + 5 >= 0; }
 __device__ __forceinline__ void far_halves64(FarSums64 &S) {
   S.G += __shfl_xor_sync(0xffffffffu, S.G, 16);
   S.H0 += __shfl_xor_sync(0xffffffffu, S.H0, 16);
@@ -1754,15 +1764,22 @@ __device__ __forceinline__ void far64_block(const RunArgs &a, int b, int i, int 
     int D;
     const int cnt = far_stage64(a, tab, z, t0, n0, s_k, s_j, D);
     far_group64<RING>(a, b0, cnt, pos, s_k, s_j, S);
-    const int kb0 = n0 - D - 1;
-    const bool near = D == kFarNear, wave = D >= 0 && kb0 <= 2 && kb0 + K + 3 >= 0;
-    const unsigned mn = __ballot_sync(0xffffffffu, near), mw = __ballot_sync(0xffffffffu, wave);
+    bool wave = false;
+    if (D >= 0 && far_reaches_start(n0 - D)) {
+      const size_t j = (size_t)z + (size_t)a.nsplit * (t0 + lane);
+      const float4 g = a.pgeo[row + j];
+      wave = far_crosses64(a.H32[(b0 + j) * (size_t)a.hs].x, g.x, g.y, n0 - D, __int_as_float(a.delay[row + j].y));
+    }
+    const unsigned mn = __ballot_sync(0xffffffffu, D == kFarNear), mw = __ballot_sync(0xffffffffu, wave);
+    // the same as bits of the staged entries
+    const unsigned mf = __ballot_sync(0xffffffffu, D >= 0);
+    const unsigned ew = __reduce_or_sync(0xffffffffu, wave ? 1u << __popc(mf & ((1u << lane) - 1u)) : 0u);
     if (lane < ns) {
       float grp = 0.f;
       for (int e = 0; e < cnt; ++e) {
         const int2 r = s_j[e];
         const int kb = r.y;
-        if (kb <= 2 && kb + K + 3 >= 0) continue;  // crossing t = 0: below
+        if ((ew >> e) & 1u) continue;  // crossing t = 0: below
         const size_t ij = row + (size_t)r.x;
         const float4 geo = a.pgeo[ij];
         const float xs = stage_f - __int_as_float(a.delay[ij].y);
@@ -3246,38 +3263,31 @@ struct AdjArgs {
   int64_t margin;      // samples of slack around the retarded window (charge offsets)
 };
 
+// One warp per receiver (its scan over the sources by one thread took 265 us with 256 of them).
 __global__ void adj_init_kernel(const AdjArgs A) {
   const RunArgs &a = A.f;
   const double L = kC * a.dt;
-  for (int64_t bi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; bi < (int64_t)a.B * a.N;
-       bi += (int64_t)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t bi = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; bi < (int64_t)a.B * a.N;
+       bi += ((int64_t)gridDim.x * blockDim.x) >> 5) {
     const int b = (int)(bi / a.N), i = (int)(bi % a.N);
     const double m1 = a.m1[bi], m2 = a.m2[bi], q = a.q[bi], w0 = a.omega0[bi];
     const double m = m1 * m2 / (m1 + m2);
     const size_t sN = (size_t)bi * a.hs + (a.n_steps & a.wm);
     const double dN = a.d[sN], vN = a.dd[sN];
     const double w = A.wE ? A.wE[bi] : 0.0;
-    A.wts[2 * bi] = m2 / (m1 + m2) / q;
-    A.wts[2 * bi + 1] = -m1 / (m1 + m2) / q;
     double dmax = 0.0;
     if (a.org_pos) {
       const int64_t H = 2 * a.n_steps + 1;
       const double *P0 = a.org_pos + bi * H * 3;
-      for (int64_t h = 1; h < H; ++h) {
+      for (int64_t h = 1 + lane; h < H; h += 32) {
         const double *Ph = P0 + 3 * h;
         const double ex = Ph[0] - P0[0], ey = Ph[1] - P0[1], ez = Ph[2] - P0[2];
         dmax = fmax(dmax, sqrt(ex * ex + ey * ey + ez * ez));
       }
     }
-    A.disp[bi] = dmax / L;
-    // E = m (w0^2 d^2 + d'^2) / (2 q^2)
-    A.lam[2 * bi] = w * m * w0 * w0 * dN / (q * q);
-    A.lam[2 * bi + 1] = w * m * vN / (q * q);
-    A.w0bar[bi] = w * m * w0 * dN * dN / (q * q);
-    A.carry[bi] = 0.0;
-    for (int c = 0; c < 3; ++c) A.g_origin[3 * bi + c] = 0.0;
     double tmin = 1e300, tmax = 0.0;
-    for (int jj = 0; jj < a.N; ++jj) {
+    for (int jj = lane; jj < a.N; jj += 32) {
       if (jj == i) continue;
       const size_t bj = bidx(a, b, jj);
       const double dx = a.origin[3 * bi] - a.origin[3 * bj], dy = a.origin[3 * bi + 1] - a.origin[3 * bj + 1],
@@ -3286,6 +3296,21 @@ __global__ void adj_init_kernel(const AdjArgs A) {
       tmin = fmin(tmin, t);
       tmax = fmax(tmax, t);
     }
+    for (int o = 16; o > 0; o >>= 1) {
+      dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+      tmin = fmin(tmin, __shfl_xor_sync(0xffffffffu, tmin, o));
+      tmax = fmax(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+    }
+    if (lane) continue;
+    A.wts[2 * bi] = m2 / (m1 + m2) / q;
+    A.wts[2 * bi + 1] = -m1 / (m1 + m2) / q;
+    A.disp[bi] = dmax / L;
+    // E = m (w0^2 d^2 + d'^2) / (2 q^2)
+    A.lam[2 * bi] = w * m * w0 * w0 * dN / (q * q);
+    A.lam[2 * bi + 1] = w * m * vN / (q * q);
+    A.w0bar[bi] = w * m * w0 * dN * dN / (q * q);
+    A.carry[bi] = 0.0;
+    for (int c = 0; c < 3; ++c) A.g_origin[3 * bi + c] = 0.0;
     A.tau[2 * bi] = tmin;
     A.tau[2 * bi + 1] = tmax;
   }
@@ -3293,104 +3318,119 @@ __global__ void adj_init_kernel(const AdjArgs A) {
 
 // (1) reverse RK4 of steps n0 + kb - 1 .. n0 for one receiver; writes the stage-field adjoints of
 // the block to Ebar[1 .. 2 kb] (stage s at time n0 + s/2).
+// One warp per receiver, one lane per step: the step is linear in the state, y_{n+1} = M y_n + ..., so the
+// state's adjoint after step k, L_k = s_k + M^T L_{k+1} with s_k from the history sample's, is a scan over the
+// lanes with the powers of M that the forward run tabulates; all else is a step's own.  (One thread per
+// receiver, bound by the kb dependent steps: 61 us a block of 16 of 256 receivers.)
 __global__ void adj_rk4_kernel(const AdjArgs A, int64_t n0, int kb) {
   const RunArgs &a = A.f;
-  const int64_t bi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t bi = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (bi >= (int64_t)a.B * a.N) return;
+  const bool on = lane < kb;
+  const int k = min(lane, kb - 1);
   const int64_t So = a.n_steps - a.n_begin + 1;
   const size_t row = (size_t)bi * a.hs;
-  const double m1 = a.m1[bi], m2 = a.m2[bi], q = a.q[bi], w0 = a.omega0[bi];
-  const double m = m1 * m2 / (m1 + m2);
-  const double g0 = q * q * w0 * w0 / (6.0 * kPi * kEps0 * kC * kC * kC * m);
-  const double qm = q * q / m;
+  const double *T = a.rk4tab + bi * kTab;
+  const double w0 = a.omega0[bi], g0 = T[kTabC], w2 = T[kTabC + 1], qm = T[kTabC + 2];
   const double dt = a.dt, h = 0.5 * dt;
-  double l0 = A.lam[2 * bi], l1 = A.lam[2 * bi + 1];
-  double carry = A.carry[bi];
-  double w0b = 0.0;
+  const int64_t n = n0 + k;
+  // history sample n+1 = (d, d', d'') with d'' = qm E(n+1) - g0 d' - w0^2 d; its adjoint is
+  // complete (only later blocks read the sample) and is consumed here, its slot cleared for reuse
+  double *mu1 = A.mu + (row + ((n + 1) & a.wm)) * 3;
+  const double m0 = mu1[0], m2v = mu1[2];
+  double m1v = mu1[1];
+  if (A.dseed && n + 1 >= A.seed_first && n + 1 < A.seed_first + A.seed_len)
+    m1v += A.dseed[(size_t)bi * A.seed_len + (size_t)(n + 1 - A.seed_first)];
+  __syncwarp();
+  if (on) mu1[0] = mu1[1] = mu1[2] = 0.0;
+  double l0 = on ? m0 - w2 * m2v : 0.0, l1 = on ? m1v - g0 * m2v : 0.0;
+  if (lane == kb - 1) {
+    l0 += A.lam[2 * bi];
+    l1 += A.lam[2 * bi + 1];
+  }
+  for (int off = 1; off < kb; off <<= 1) {
+    const double ox = __shfl_down_sync(0xffffffffu, l0, off), oy = __shfl_down_sync(0xffffffffu, l1, off);
+    if (lane + off < kb) {
+      const double *P = T + 4 * (off - 1);  // M^off
+      l0 = fma(P[2], oy, fma(P[0], ox, l0));
+      l1 = fma(P[3], oy, fma(P[1], ox, l1));
+    }
+  }
+  const size_t sN = row + ((n + 1) & a.wm), s0 = row + (n & a.wm);
+  const double yN0 = a.d[sN], yN1 = a.dd[sN];
+  double e4b = qm * m2v;
+  double g0b = -yN1 * m2v, w2b = -yN0 * m2v;
+  // forward stages of step n
+  const double y0 = a.d[s0], y1 = a.dd[s0];
+  const double e1 = a.Ed[(size_t)bi * So + (size_t)(n - a.n_begin)],
+               e2 = a.Ehalf[(size_t)bi * (So - 1) + (size_t)(n - a.n_begin)];
+  const double k1a = y1, k1b = -g0 * y1 - w2 * y0 + qm * e1;
+  const double y0b = y0 + h * k1a, y1b = y1 + h * k1b;
+  const double k2a = y1b, k2b = -g0 * y1b - w2 * y0b + qm * e2;
+  const double y0c = y0 + h * k2a, y1c = y1 + h * k2b;
+  const double k3a = y1c, k3b = -g0 * y1c - w2 * y0c + qm * e2;
+  const double y0d = y0 + dt * k3a, y1d = y1 + dt * k3b;
+  // reverse of y_{n+1} = y_n + dt/6 (k1 + 2 k2 + 2 k3 + k4)
+  const double dt6 = dt / 6.0, dt3 = dt / 3.0;
+  double y0bar = l0, y1bar = l1;
+  double k1ab = dt6 * l0, k2ab = dt3 * l0, k3ab = dt3 * l0;
+  const double k4ab = dt6 * l0, k4bb = dt6 * l1;
+  double k1bb = dt6 * l1, k2bb = dt3 * l1, k3bb = dt3 * l1;
+  double e2b = 0.0, e1b = 0.0;
+  // k4 = f(y_d, e4)
+  const double y1db = k4ab - g0 * k4bb, y0db = -w2 * k4bb;
+  e4b += qm * k4bb;
+  g0b += -y1d * k4bb;
+  w2b += -y0d * k4bb;
+  y0bar += y0db;
+  k3ab += dt * y0db;
+  y1bar += y1db;
+  k3bb += dt * y1db;
+  // k3 = f(y_c, e2)
+  const double y1cb = k3ab - g0 * k3bb, y0cb = -w2 * k3bb;
+  e2b += qm * k3bb;
+  g0b += -y1c * k3bb;
+  w2b += -y0c * k3bb;
+  y0bar += y0cb;
+  k2ab += h * y0cb;
+  y1bar += y1cb;
+  k2bb += h * y1cb;
+  // k2 = f(y_b, e2)
+  const double y1bb = k2ab - g0 * k2bb, y0bb = -w2 * k2bb;
+  e2b += qm * k2bb;
+  g0b += -y1b * k2bb;
+  w2b += -y0b * k2bb;
+  y0bar += y0bb;
+  k1ab += h * y0bb;
+  y1bar += y1bb;
+  k1bb += h * y1bb;
+  // k1 = f(y_n, e1)
+  y1bar += k1ab - g0 * k1bb;
+  y0bar += -w2 * k1bb;
+  e1b += qm * k1bb;
+  g0b += -y1 * k1bb;
+  w2b += -y0 * k1bb;
+  // E(n+1) is step n's last stage and step n+1's first
+  const double next = __shfl_down_sync(0xffffffffu, e1b, 1);
+  e4b += lane == kb - 1 ? A.carry[bi] : next;
   double *Eb = A.Ebar + bi * (2 * kMaxBlock + 1);
-  for (int k = kb - 1; k >= 0; --k) {
-    const int64_t n = n0 + k;
-    // history sample n+1 = (d, d', d'') with d'' = qm E(n+1) - g0 d' - w0^2 d; its adjoint is
-    // complete (only later blocks read the sample) and is consumed here, its slot cleared for reuse
-    double *mu1 = A.mu + (row + ((n + 1) & a.wm)) * 3;
-    const double m0 = mu1[0], m2v = mu1[2];
-    double m1v = mu1[1];
-    if (A.dseed && n + 1 >= A.seed_first && n + 1 < A.seed_first + A.seed_len)
-      m1v += A.dseed[(size_t)bi * A.seed_len + (size_t)(n + 1 - A.seed_first)];
-    mu1[0] = 0.0;
-    mu1[1] = 0.0;
-    mu1[2] = 0.0;
-    const size_t sN = row + ((n + 1) & a.wm), s0 = row + (n & a.wm);
-    const double yN0 = a.d[sN], yN1 = a.dd[sN];
-    l0 += m0 - w0 * w0 * m2v;
-    l1 += m1v - g0 * m2v;
-    double e4b = carry + qm * m2v;
-    double g0b = -yN1 * m2v, w2b = -yN0 * m2v;
-    // forward stages of step n
-    const double y0 = a.d[s0], y1 = a.dd[s0];
-    const size_t o = (size_t)bi * So + (size_t)(n - a.n_begin);
-    const double e1 = a.Ed[o], e2 = a.Ehalf[(size_t)bi * (So - 1) + (size_t)(n - a.n_begin)], e4 = a.Ed[o + 1];
-    const double k1a = y1, k1b = -g0 * y1 - w0 * w0 * y0 + qm * e1;
-    const double y0b = y0 + h * k1a, y1b = y1 + h * k1b;
-    const double k2a = y1b, k2b = -g0 * y1b - w0 * w0 * y0b + qm * e2;
-    const double y0c = y0 + h * k2a, y1c = y1 + h * k2b;
-    const double k3a = y1c, k3b = -g0 * y1c - w0 * w0 * y0c + qm * e2;
-    const double y0d = y0 + dt * k3a, y1d = y1 + dt * k3b;
-    (void)e4;
-    // reverse of y_{n+1} = y_n + dt/6 (k1 + 2 k2 + 2 k3 + k4)
-    double y0bar = l0, y1bar = l1;
-    double k1ab = dt / 6.0 * l0, k2ab = dt / 3.0 * l0, k3ab = dt / 3.0 * l0, k4ab = dt / 6.0 * l0;
-    double k1bb = dt / 6.0 * l1, k2bb = dt / 3.0 * l1, k3bb = dt / 3.0 * l1, k4bb = dt / 6.0 * l1;
-    double e2b = 0.0, e1b = 0.0;
-    // k4 = f(y_d, e4)
-    double y1db = k4ab - g0 * k4bb, y0db = -w0 * w0 * k4bb;
-    e4b += qm * k4bb;
-    g0b += -y1d * k4bb;
-    w2b += -y0d * k4bb;
-    y0bar += y0db;
-    k3ab += dt * y0db;
-    y1bar += y1db;
-    k3bb += dt * y1db;
-    // k3 = f(y_c, e2)
-    double y1cb = k3ab - g0 * k3bb, y0cb = -w0 * w0 * k3bb;
-    e2b += qm * k3bb;
-    g0b += -y1c * k3bb;
-    w2b += -y0c * k3bb;
-    y0bar += y0cb;
-    k2ab += h * y0cb;
-    y1bar += y1cb;
-    k2bb += h * y1cb;
-    // k2 = f(y_b, e2)
-    double y1bb = k2ab - g0 * k2bb, y0bb = -w0 * w0 * k2bb;
-    e2b += qm * k2bb;
-    g0b += -y1b * k2bb;
-    w2b += -y0b * k2bb;
-    y0bar += y0bb;
-    k1ab += h * y0bb;
-    y1bar += y1bb;
-    k1bb += h * y1bb;
-    // k1 = f(y_n, e1)
-    y1bar += k1ab - g0 * k1bb;
-    y0bar += -w0 * w0 * k1bb;
-    e1b += qm * k1bb;
-    g0b += -y1 * k1bb;
-    w2b += -y0 * k1bb;
-    // g0 = q^2 w0^2 / (6 pi eps0 c^3 m), w2 = w0^2
-    w0b += g0b * 2.0 * g0 / w0 + w2b * 2.0 * w0;
+  if (on) {
     Eb[2 * k + 2] = e4b;
     Eb[2 * k + 1] = e2b;
-    carry = e1b;
-    l0 = y0bar;
-    l1 = y1bar;
   }
-  A.lam[2 * bi] = l0;
-  A.lam[2 * bi + 1] = l1;
-  A.carry[bi] = carry;
-  A.w0bar[bi] += w0b;
-  if (A.ebmax) {
-    double m = 0.0;
-    for (int k = 1; k <= 2 * kb; ++k) m = fmax(m, fabs(Eb[k]));
-    atomicMax(A.ebmax, (unsigned long long)__double_as_longlong(m));
+  // g0 = q^2 w0^2 / (6 pi eps0 c^3 m), w2 = w0^2
+  double w0b = on ? g0b * (2.0 * g0 / w0) + w2b * (2.0 * w0) : 0.0, m = on ? fmax(fabs(e4b), fabs(e2b)) : 0.0;
+  for (int o = 16; o > 0; o >>= 1) {
+    w0b += __shfl_xor_sync(0xffffffffu, w0b, o);
+    m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  }
+  if (lane == 0) {
+    A.lam[2 * bi] = y0bar;
+    A.lam[2 * bi + 1] = y1bar;
+    A.carry[bi] = e1b;
+    A.w0bar[bi] += w0b;
+    if (A.ebmax) atomicMax(A.ebmax, (unsigned long long)__double_as_longlong(m));
   }
 }
 
@@ -3719,10 +3759,11 @@ __global__ void __launch_bounds__(128, 4) adj_field_kernel(const AdjArgs A, int6
 // g = k1 d + k2 d' + k3 d'': lanes = positions.  The cubic terms go through their reverse in float32, lanes =
 // stages, their adjoints of the samples gathered by the positions.  Where a charge is off its centre's
 // segment by o samples the term o/2 (k . second difference) is reversed in float64.  The geometry's gradient
-// is formed at the end of a batch, lanes = receivers.  Near sources, those crossing t = 0 and blocks that may
-// hold a sample beyond the limits go through pair_rev_f64, lanes = stages.  All history adjoints go to A.mu
-// by atomics that return nothing (a shared-memory window's float64 ones are compare-and-swap loops: 1.25 ms a
-// block of the ring of 256 against 0.42; 2.7 with two charges throughout).  The float64 unit is busy 82 %.
+// is formed at the end of a batch, lanes = receivers.  Near sources, those with a charge across sample 0 or 1 (far_crosses64)
+// and blocks that may hold a sample beyond the limits go through pair_rev_f64, lanes = stages.  All history
+// adjoints go to A.mu by atomics that return nothing (a shared-memory window's float64 ones are
+// compare-and-swap loops: 1.25 ms a block of the ring of 256 against 0.42, 0.37 since fewer pairs cross t = 0;
+// 2.7 with two charges throughout).  Bound by the float64 unit (82 % busy).
 constexpr int kRevWarps = 4;
 struct RevShared {
   double s[8 * 4][19];       // partial sums of 8 pairs, rows = (pair, S1 .. S4), columns = positions, the last: crossings
@@ -3767,8 +3808,14 @@ __global__ void __launch_bounds__(kRevWarps * 32, 3) adj_split_kernel(const __gr
     int D;
     const int cnt = far_stage64(a, tab, z, t0, n0i, sh.k, sh.j, D);
     const bool valid = D != kFarNone;
-    const int kb0 = n0i - D - 1;
-    const bool wave = D >= 0 && kb0 <= 2 && kb0 + kMaxBlock + 3 >= 0;
+    bool wave = false;
+    if (D >= 0 && far_reaches_start(n0i - D)) {
+      const size_t ji = bj * (size_t)a.N + (size_t)(z + a.nsplit * (t0 + lane));
+      const float4 g = a.pgeo[ji];  // with the roles exchanged
+      wave = far_crosses64(hj[0].x, g.x, g.z, n0i - D, __int_as_float(A.delay[ji].y));
+    }
+    const unsigned mf = __ballot_sync(0xffffffffu, D >= 0);
+    const unsigned ew = __reduce_or_sync(0xffffffffu, wave ? 1u << __popc(mf & ((1u << lane) - 1u)) : 0u);  // staged entries
     const unsigned mnear = __ballot_sync(0xffffffffu, valid && (D < 0 || wave || all_near));
     // ---- far receivers, eight at a time ----
     if (!all_near)
@@ -3777,7 +3824,7 @@ __global__ void __launch_bounds__(kRevWarps * 32, 3) adj_split_kernel(const __gr
         for (int e = e0; e < e1; ++e) {
           const int2 r = sh.j[e];
           const int i = r.x, kb = r.y;
-          const bool skip = kb <= 2 && kb + kMaxBlock + 3 >= 0;  // crossing t = 0: among the near ones
+          const bool skip = (ew >> e) & 1u;  // crossing t = 0: among the near ones
           const size_t bi = b0 + (size_t)i;
           const int row = 4 * (e - e0);
           __syncwarp();
@@ -3802,11 +3849,9 @@ __global__ void __launch_bounds__(kRevWarps * 32, 3) adj_split_kernel(const __gr
             const double thd = half ? (qh ? 0.5 : 1.5) - k.f : 1.0 - k.f;
             const float th = (float)thd;
             const int64_t sk0 = (int64_t)max(kk, 0) & wm, sk1 = (int64_t)max(kk + 1, 0) & wm;
-            const float4 h0 = hj[sk0];
+            const float4 h0 = hj[sk0], h1 = hj[sk1];
             const float R = geo.x, iR = __fdividef(1.f, R);
-            // (slopes from the float64 samples)
-            const float dX = (float)((dj[sk1] - dj[sk0]) * msx), dV = (float)((ddj[sk1] - ddj[sk0]) * msv),
-                        dA = (float)((dddj[sk1] - dddj[sk0]) * msa);
+            const float dX = h1.x - h0.x, dV = h1.y - h0.y, dA = h1.z - h0.z;
             const float X = fmaf(th, dX, h0.x), V = fmaf(th, dV, h0.y), Ac = fmaf(th, dA, h0.z);
             // rho points from j to i here: geo's from i to j (row j: rho . p_i, rho . p_j with the other sign)
             const float mu = -geo.z * iR, nu = -geo.y * iR;
@@ -3919,8 +3964,8 @@ __global__ void __launch_bounds__(kRevWarps * 32, 3) adj_split_kernel(const __gr
       }
     // ---- the far receivers' geometry, lanes = receivers ----
     if (!all_near && lane < cnt) {
-      const int i = sh.j[lane].x, kb = sh.j[lane].y;
-      if (!(kb <= 2 && kb + kMaxBlock + 3 >= 0)) {
+      const int i = sh.j[lane].x;
+      if (!((ew >> lane) & 1u)) {
         const size_t bi = b0 + (size_t)i;
         const double *pi = a.axis + 3 * bi, *Ri = a.origin + 3 * bi;
         const double rho[3] = {Ri[0] - Rj[0], Ri[1] - Rj[1], Ri[2] - Rj[2]};
@@ -4352,7 +4397,7 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
     if (omega_out && cudaMemcpyAsync(omega_out, fw_, nbn * sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
       return PC_ERR_CUDA;
   }
-  const unsigned rgrid = (unsigned)((nbn + 127) / 128);
+  const unsigned rgrid = (unsigned)((nbn + 127) / 128), wgrid = (unsigned)((nbn * 32 + 127) / 128);  // per thread, per warp
   // the forward run's split form (float64 forward on the grid path): its tables and mirror for the reverse
   auto use_tables = [&]() {
     a.pfar64 = run.pfar64;
@@ -4399,7 +4444,7 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
     pc_status rs = recompute(nseg - 1);
     if (rs != PC_OK) return rs;
   }
-  adj_init_kernel<<<rgrid, 128, 0, st>>>(A);
+  adj_init_kernel<<<wgrid, 128, 0, st>>>(A);
   // margin for charge offsets: three times the largest initial |r_dip|, in samples, plus one
   std::vector<double> hq(nbn), hd0(nbn), htau(2 * nbn), hdisp(nbn);
   if (cudaMemcpyAsync(hq.data(), dp->q, nbn * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -4458,7 +4503,7 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
     for (int64_t bk = nblocks - 1; bk >= 0; --bk) {
       const int64_t n0 = s0 + bk * K;
       const int kb = (int)std::min((int64_t)K, s1 - n0);
-      adj_rk4_kernel<<<rgrid, 128, 0, st>>>(A, n0, kb);
+      adj_rk4_kernel<<<wgrid, 128, 0, st>>>(A, n0, kb);
       if (mov) adj_field_kernel<true><<<fgrid, 128, smem, st>>>(A, n0, 2 * kb, wmax);
       else if (split) adj_split_kernel<<<sgrid, kRevWarps * 32, smem_split, st>>>(A, n0, 2 * kb);
       else adj_field_kernel<false><<<fgrid, 128, smem, st>>>(A, n0, 2 * kb, wmax);

@@ -416,6 +416,40 @@ __device__ __forceinline__ ff ff_sqrt(ff a) {
   float r = fmaf(-s0, s0, a.hi) + a.lo;  // a - s0^2
   return ff_two_sum(s0, r / (2.f * s0));
 }
+// The delay of a list point: rho = anchor's rho (g, gl) + offset (dr, drl), |rho| and the retarded sample
+// fa - (|rho| - |g|) as kb + xc with 0 <= xc < 1.  Unevaluated high and low parts throughout, renormalised
+// nowhere (their low parts stay within a few of the high parts' last places): 1e-11 of a sample at 1e4, in
+// half the operations of the ff_ functions.
+struct ListDelay {
+  float rx, ry, rz, rho2, i, rn, xc;
+  int kb;
+};
+__device__ __forceinline__ ListDelay list_delay(float4 g, float4 gl, float drx, float dry, float drz, float drlx, float drly,
+                                                float drlz, float fa, int kb) {
+  const ff px = ff_two_sum(g.x, drx), py = ff_two_sum(g.y, dry), pz = ff_two_sum(g.z, drz);
+  const float lx = px.lo + (gl.x + drlx), ly = py.lo + (gl.y + drly), lz = pz.lo + (gl.z + drlz);
+  const float xx = px.hi * px.hi, yy = py.hi * py.hi, zz = pz.hi * pz.hi;
+  const float ex = fmaf(2.f * px.hi, lx, fmaf(px.hi, px.hi, -xx)), ey = fmaf(2.f * py.hi, ly, fmaf(py.hi, py.hi, -yy)),
+              ez = fmaf(2.f * pz.hi, lz, fmaf(pz.hi, pz.hi, -zz));
+  const ff a = ff_two_sum(xx, yy), b = ff_two_sum(a.hi, zz);
+  const float lo = (ex + ey) + (ez + (a.lo + b.lo));
+  ListDelay o;
+  o.rx = px.hi;
+  o.ry = py.hi;
+  o.rz = pz.hi;
+  o.rho2 = b.hi;
+  o.i = b.hi > 1e-30f ? rsqrt_fast(b.hi) : 0.f;
+  const float s0 = b.hi * o.i;
+  o.rn = s0;
+  const ff d = ff_two_sum(s0, -g.w);  // |rho| = s0 + (rho^2 - s0^2) / (2 s0)
+  const float dl = d.lo + (0.5f * o.i * (fmaf(-s0, s0, b.hi) + lo) - gl.w);
+  const ff x = ff_two_sum(fa, -d.hi);
+  float flf;
+  const int fl = Num<float>::floor_int(x.hi, flf);
+  o.kb = kb + fl;
+  o.xc = (x.hi - flf) + (x.lo - dl);
+  return o;
+}
 __device__ __forceinline__ ff ff_from_double(double x) {
   float hi = (float)x;
   return {hi, (float)(x - (double)hi)};
@@ -638,7 +672,12 @@ __device__ __forceinline__ int64_t tile_point(const Launch &L, int64_t tiles_v, 
   return (iu < L.pts.nu && iv < L.pts.nv) ? iu * L.pts.nv + iv : L.pts.P;
 }
 
-template <int KIND, bool LIST, int CH>
+// FAR (large lists): a pair beyond its source's L.rfar takes the first-order dipole form (pc_far_f32.cuh), a
+// third of the two-charge form's operations.  Points of a list are anywhere, so each pair is asked by itself;
+// in a micrometre cube one warp in five has a near lane for a source.  Measured, 64 dipoles at 100 003 points in
+// two frames: 347 -> 311 us a call with list_delay, 259 of them here; bound by latency (24 warps an SM, the
+// second wave of CTAs a quarter full) and by the float64 unit in near pairs that cancel (40 % busy).
+template <int KIND, bool LIST, int CH, bool FAR = false>
 __global__ void __launch_bounds__(kMixThreads, 4) fields_mixed_kernel(const Launch L, int64_t tiles_v) {
   __shared__ double s_anchor[3];
   __shared__ float s_anc_hi[3], s_anc_lo[3];  // the anchor / (c dt) of the dipoles as float-float
@@ -649,6 +688,7 @@ __global__ void __launch_bounds__(kMixThreads, 4) fields_mixed_kernel(const Laun
   __shared__ float4 s_mix[CH];   // m2/(m1+m2), m1/(m1+m2), fraction and integer part of the
                                      // retarded sample of the anchor (integer as bits)
   __shared__ const float4 *s_hist[CH];
+  __shared__ float s_rfar[FAR ? CH : 1];
 
   const int tid = threadIdx.x;
   const int f = blockIdx.y;
@@ -736,6 +776,7 @@ __global__ void __launch_bounds__(kMixThreads, 4) fields_mixed_kernel(const Laun
         const float4 mm = L.srcf[4 * j + 1];
         s_mix[tid] = make_float4(mm.x, mm.y, (x.hi - kaf) + x.lo, __int_as_float(kai));
         s_hist[tid] = L.Hd + (size_t)j * s.Sd;
+        if (FAR) s_rfar[tid] = L.rfar[j];
       }
       __syncthreads();
       if (!active || err) continue;
@@ -753,30 +794,25 @@ __global__ void __launch_bounds__(kMixThreads, 4) fields_mixed_kernel(const Laun
         const float4 mx = s_mix[jj];
         const float2 mu = make_float2(mx.x, mx.y);
         const float fa = mx.z;
-        const float rx = g.x + drx, ry = g.y + dry, rz = g.z + drz;
-        const float rho2 = rx * rx + ry * ry + rz * rz;
-        // rho2 == 0 makes rn NaN, which sends the pair to the slow path through the tests below
-        const float rn = rho2 * rsqrtf(rho2);
+        float rx, ry, rz, rn, irn = 0.f;
         // retarded time of the dipole centre, in samples: kb + xc with |xc| small
         int kb = __float_as_int(mx.w);
         float xc;
-        if (!LIST) {
+        if constexpr (!LIST) {
+          rx = g.x + drx, ry = g.y + dry, rz = g.z + drz;
+          const float rho2 = rx * rx + ry * ry + rz * rz;
+          // rho2 == 0 makes rn NaN, which sends the pair to the slow path through the tests below
+          rn = rho2 * rsqrtf(rho2);
           // compact tile: |rho| - |rho_a| from the tile offset without cancellation
           const float corr = __fdividef(2.f * (g.x * drx + g.y * dry + g.z * drz) + dr2, rn + g.w);
           xc = fa - corr;
         } else {
-          // points of a list tile may lie far apart: |rho| - |rho_a| in float-float, integer part
+          // points of a list tile may lie far apart: |rho| - |rho_a| in two parts, integer part
           // moved into kb so that the fraction keeps its precision
-          const float4 gl = s_geo_lo[jj];
-          const ff px = ff_add({g.x, gl.x}, {drx, drlx}), py = ff_add({g.y, gl.y}, {dry, drly}),
-                   pz = ff_add({g.z, gl.z}, {drz, drlz});
-          const ff n2 = ff_add(ff_add(ff_mul(px, px), ff_mul(py, py)), ff_mul(pz, pz));
-          const ff dn = ff_add(ff_sqrt(n2), {-g.w, -gl.w});
-          const ff x = ff_add({fa, 0.f}, {-dn.hi, -dn.lo});
-          float flf;
-          const int fl = Num<float>::floor_int(x.hi, flf);
-          kb += fl;
-          xc = (x.hi - flf) + x.lo;
+          const ListDelay t = list_delay(g, s_geo_lo[jj], drx, dry, drz, drlx, drly, drlz, fa, kb);
+          rx = t.rx, ry = t.ry, rz = t.rz, rn = t.rn, irn = t.i;
+          xc = t.xc;
+          kb = t.kb;
         }
         const float rp = rx * ax.x + ry * ax.y + rz * ax.z;
         // fast path: both charges on the interior segment of their centre's retarded time, the point
@@ -795,6 +831,39 @@ __global__ void __launch_bounds__(kMixThreads, 4) fields_mixed_kernel(const Laun
             float x0, v0, a0, x1, v1, a1;
             H.get_in(j, x0, v0, a0);
             H.get_in(j + 1, x1, v1, a1);
+            // (not on the first two segments: the rest state before the history makes a kink there)
+            if (FAR && rn >= s_rfar[jj] && j > 1) {
+              const float th = xc - fl, i2 = irn * irn, rpi2 = rp * i2, m = rpi2 * irn;
+              const float X1 = ax.w * fmaf(th, x1 - x0, x0), V1 = ax.w * fmaf(th, v1 - v0, v0);
+              const float A1 = KIND == PC_COULOMB ? 0.f : ax.w * fmaf(th, a1 - a0, a0);
+              const float t1 = fmaf(irn, X1, V1);
+              float cE, cP, cB;
+              if (KIND == PC_COULOMB) {
+                cE = m * (3.f * irn) * t1;
+                cP = -(i2 * t1);
+                cB = i2 * irn * V1;
+              } else if (KIND == PC_RADIATION) {
+                cE = m * A1;
+                cP = -(irn * A1);
+                cB = i2 * A1;
+              } else {
+                cE = m * fmaf(3.f * irn, t1, A1);
+                cP = -(irn * fmaf(irn, t1, A1));
+                cB = i2 * fmaf(irn, V1, A1);
+              }
+              const float vi = V1 * irn;
+              P[0].x = fmaf(cP, ax.x, fmaf(cE, rx, P[0].x));
+              P[0].y = fmaf(cP, ax.y, fmaf(cE, ry, P[0].y));
+              P[3].x = fmaf(cP, ax.z, fmaf(cE, rz, P[3].x));
+              P[1].x = fmaf(cB, fmaf(ax.y, rz, -(ax.z * ry)), P[1].x);
+              P[1].y = fmaf(cB, fmaf(ax.z, rx, -(ax.x * rz)), P[1].y);
+              P[3].y = fmaf(cB, fmaf(ax.x, ry, -(ax.y * rx)), P[3].y);
+              P[2].x = fmaf(vi, ax.x, P[2].x);
+              P[2].y = fmaf(vi, ax.y, P[2].y);
+              P[4].x = fmaf(vi, ax.z, P[4].x);
+              P[4].y = fmaf(rpi2, t1, P[4].y);
+              continue;
+            }
             fast = dip_pair_states_fast(x0, v0, a0, x1, v1, a1, xc - fl, rn, rp, mu.x, mu.y, X, V, Ac, dl);
           }
         }
@@ -824,25 +893,19 @@ __global__ void __launch_bounds__(kMixThreads, 4) fields_mixed_kernel(const Laun
         const float4 g = s_geo[jj];
         const float4 ax = s_ax[jj];
         const float4 mx = s_mix[jj];
-        const float rx = g.x + drx, ry = g.y + dry, rz = g.z + drz;
-        const float rho2 = rx * rx + ry * ry + rz * rz;
-        const float rn = rho2 > 0.f ? rho2 * rsqrtf(rho2) : 0.f;
+        float rx, ry, rz, rn, xc;
         int kb = __float_as_int(mx.w);
-        float xc;
-        if (!LIST) {
+        if constexpr (!LIST) {
+          rx = g.x + drx, ry = g.y + dry, rz = g.z + drz;
+          const float rho2 = rx * rx + ry * ry + rz * rz;
+          rn = rho2 > 0.f ? rho2 * rsqrtf(rho2) : 0.f;
           const float corr = __fdividef(2.f * (g.x * drx + g.y * dry + g.z * drz) + dr2, rn + g.w);
           xc = mx.z - corr;
         } else {
-          const float4 gl = s_geo_lo[jj];
-          const ff px = ff_add({g.x, gl.x}, {drx, drlx}), py = ff_add({g.y, gl.y}, {dry, drly}),
-                   pz = ff_add({g.z, gl.z}, {drz, drlz});
-          const ff n2 = ff_add(ff_add(ff_mul(px, px), ff_mul(py, py)), ff_mul(pz, pz));
-          const ff dn = ff_add(ff_sqrt(n2), {-g.w, -gl.w});
-          const ff x = ff_add({mx.z, 0.f}, {-dn.hi, -dn.lo});
-          float flf;
-          const int fl = Num<float>::floor_int(x.hi, flf);
-          kb += fl;
-          xc = (x.hi - flf) + x.lo;
+          const ListDelay t = list_delay(g, s_geo_lo[jj], drx, dry, drz, drlx, drly, drlz, mx.z, kb);
+          rx = t.rx, ry = t.ry, rz = t.rz, rn = t.rn;
+          xc = t.xc;
+          kb = t.kb;
         }
         double rp64[3];
         point_at(L.pts, tile_point(L, tiles_v, tid), rp64);
@@ -1685,6 +1748,12 @@ static void launch_mixed_plane(const Launch &L, dim3 grid, int64_t tiles_v, bool
   }
 }
 static void launch_mixed_list(const Launch &L, dim3 grid, int kind, cudaStream_t st) {
+  if (L.rfar) {
+    if (kind == PC_TOTAL) fields_mixed_kernel<PC_TOTAL, true, kChunk, true><<<grid, kMixThreads, 0, st>>>(L, 1);
+    else if (kind == PC_COULOMB) fields_mixed_kernel<PC_COULOMB, true, kChunk, true><<<grid, kMixThreads, 0, st>>>(L, 1);
+    else fields_mixed_kernel<PC_RADIATION, true, kChunk, true><<<grid, kMixThreads, 0, st>>>(L, 1);
+    return;
+  }
   if (kind == PC_TOTAL) fields_mixed_kernel<PC_TOTAL, true, kChunk><<<grid, kMixThreads, 0, st>>>(L, 1);
   else if (kind == PC_COULOMB) fields_mixed_kernel<PC_COULOMB, true, kChunk><<<grid, kMixThreads, 0, st>>>(L, 1);
   else fields_mixed_kernel<PC_RADIATION, true, kChunk><<<grid, kMixThreads, 0, st>>>(L, 1);
@@ -1737,6 +1806,8 @@ static cudaError_t launch_far(const pc_ctx *ctx, const Launch &L, int kind, cuda
 // asking the device (one read-back, about 10 us).  Sets L.tile_r, the largest distance of a tile's point
 // from its anchor (c dt).
 constexpr double kFarWork = 8e6;  // fields_mixed_kernel: about 30 us
+// lists: (point, dipole, frame) triples from which the far distances (a memset and a small kernel, 5 us) pay
+constexpr double kFarListWork = 2e6;
 static bool far_candidate(Launch &L, bool plane_of_dipoles, int32_t T) {
   if (!plane_of_dipoles || (double)L.src.N * (double)L.pts.P * (double)T < kFarWork) return false;
   double r2 = 0.0;
@@ -1918,12 +1989,13 @@ static pc_status fields_impl(pc_ctx *ctx, const pc_charges *ch, const pc_dipole_
       L.ev_L[i] = (float)(L.pts.ev[i] * L.iLd);
     }
     far_try = far_candidate(L, !list && has_dp && !has_ch, T);
+    const bool far_lim = far_try || (list && has_dp && (double)s.N * (double)P * (double)T >= kFarListWork);
     unsigned *xvmax = (unsigned *)(Hc + nc + ns);
-    if (far_try && cudaMemsetAsync(xvmax, 0, 2 * (size_t)s.N * sizeof(unsigned), st) != cudaSuccess) return PC_ERR_CUDA;
+    if (far_lim && cudaMemsetAsync(xvmax, 0, 2 * (size_t)s.N * sizeof(unsigned), st) != cudaSuccess) return PC_ERR_CUDA;
     if (has_dp) {
-      launch_prep_dipoles(s, Hd, Hc + nc, far_try ? xvmax : nullptr, L.status, st);
+      launch_prep_dipoles(s, Hd, Hc + nc, far_lim ? xvmax : nullptr, L.status, st);
     }
-    if (far_try) {
+    if (far_lim) {
       float *rfar = (float *)(xvmax + 2 * (size_t)s.N);
       far_limit_kernel<<<(unsigned)((s.N + 127) / 128), 128, 0, st>>>(s.N, xvmax, L.srcf, L.rex_fast, rfar);
       L.rfar = rfar;

@@ -95,6 +95,30 @@ def test_coarse_grid_tiles_are_never_wholly_far(ctx):
     _check(ctx, _sources(64), 401, 403, [11.4e-15], step=4e-8)
 
 
+@pytest.mark.parametrize("kind", [pc.PC_TOTAL, pc.PC_COULOMB, pc.PC_RADIATION])
+@pytest.mark.parametrize("case", ["cube", "amplitude", "masses", "wide"])
+def test_large_lists_take_the_far_form_by_pair(ctx, case, kind):
+    # 28 801 points (a last CTA of one) around 70 sources (a partial group and chunk), two frames: points among
+    # the sources and, "wide", micrometres away, where the anchor's and a point's delays differ by 10 000
+    # samples; charges as fast as the limit; sources that are never far
+    dp = _sources(70, amp=2.8e-11 if case == "amplitude" else 1e-11)
+    if case == "masses":
+        dp.m1[::3] = 1836.0 * W.M_E
+    rng = np.random.default_rng(12)
+    pts = rng.uniform(0.0, 1e-6, (28801, 3))
+    if case == "wide":
+        pts[::2] += rng.uniform(-1.5e-6, 1.5e-6, pts[::2].shape)
+    times = [11.3e-15, 13.05e-15]
+    out = pc.pc_fields(ctx, dipoles=pc.dipoles_to_device(dp), points=torch.as_tensor(pts, device="cuda"), times=times,
+                       kind=kind, precision=pc.PC_MIXED)
+    p = np.unique(np.r_[0, 28800, rng.integers(0, 28801, 200)])
+    ref = oracle.fields(pts[p], times, dipoles=dp, kind=kind)
+    assert ref["status"] == oracle.OK
+    sub = {k: v[:, torch.as_tensor(p, device="cuda")].cpu() for k, v in out.items()}
+    sub = {k: v if k == "mask" else v.numpy() for k, v in sub.items()}
+    compare(sub, ref, pc.PC_MIXED)
+
+
 # ------------------------------------------------------------------------------------------------
 # the oscillator run's far drive (grid path, mixed)
 # ------------------------------------------------------------------------------------------------

@@ -1384,7 +1384,7 @@ __global__ void __launch_bounds__(kRunWarps * 32) lo_drive_kernel(const RunArgs 
 // Measured, 4096 oscillators in a 600 nm cube: 3.10 -> 0.38 ms a block of 16 steps, about 11 warp
 // instructions per pair and block against 179; bound by the gathers of the samples from L2 (272 B a pair,
 // 12 TB/s; the pair tables, 20 B a pair, take 0.05 ms from HBM).
-// MID: where the cooperative loop below runs (smaller configurations, whose near pairs are a larger part: 12 %
+// MID: where the cooperative loop below runs (smaller configurations, whose near pairs are a larger part: 8 %
 // in a ring of 256), mid pairs stay in the far form and add their cubic terms at the samples: 12.2 -> 9.5 us a
 // block there with the crossings above; for larger ones its registers cost more than it saves (4096: 0.55 ->
 // 0.70 ms a block).
@@ -2726,6 +2726,7 @@ struct RunPlan {
   const pc_dipole_motion *motion = nullptr;
   const int2 **delay_out = nullptr;         // the pair delay table (valid until the context's next run)
   const double **rk4tab_out = nullptr;      // the per-dipole tables (idem)
+  bool two_charge = false;                  // no far or split form
   // a history store supplied by the caller of run_impl, [B][N][shs] with sample n at slot n & swm
   // (null: the caller's full outputs, or a ring of the context)
   double *sd = nullptr, *sdd = nullptr, *sddd = nullptr;
@@ -2816,7 +2817,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   const size_t cr_bytes = al((size_t)far_split * nbn * (mixed ? sizeof(float4) : 4 * sizeof(double)));
   const size_t fg_bytes = mixed ? 0 : al(nbn * dp->N * sizeof(float4));  // the float64 drive's pair geometry
   const size_t far_bytes = pf_bytes + pd_bytes + cr_bytes + am_bytes + fg_bytes + 256;
-  bool far = grid && !motion && !pl.tables_only && n_end < ((int64_t)1 << 30);
+  bool far = grid && !motion && !pl.tables_only && !pl.two_charge && n_end < ((int64_t)1 << 30);
   if (far && far_bytes > ((size_t)1 << 30) && far_off + far_bytes > ctx->run_scratch.bytes) {
     size_t mfree = 0, mall = 0;  // at most half of what is left
     if (cudaMemGetInfo(&mfree, &mall) != cudaSuccess || far_bytes > mfree / 2) far = false;
@@ -4216,6 +4217,9 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
   pc_run_opts fo = *opts;
   fo.fit = 0;
   fo.checkpoint_every = 0;
+  // a mixed forward takes the two-charge form throughout: the gradients amplify the rounding in which the
+  // forms differ (1.1e-9 of them at a ring of 151), and the float64 reverse leaves it a few percent of the time
+  const bool two_charge = fo.precision == PC_MIXED;
   const int64_t first = rates ? opts->first_index : 0;
   const int64_t flen = S - first;  // the fit window's samples
   // ---- geometry: causal block length K and state depth D (tables only) ----
@@ -4225,6 +4229,7 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
     pc_run_out none;
     memset(&none, 0, sizeof(none));
     RunPlan pl;
+    pl.two_charge = two_charge;
     pl.k_out = &K;
     pl.reach_out = &D;
     pl.tables_only = true;
@@ -4274,6 +4279,7 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
     fw.d_ddot = ddd;
     fw.Ed = Ed;
     RunPlan pl;
+    pl.two_charge = two_charge;
     pl.Ehalf = Eh;
     pl.motion = motion;
     pl.delay_out = &delay;
@@ -4298,6 +4304,7 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
       pc_run_out none;
       memset(&none, 0, sizeof(none));
       RunPlan pl;
+      pl.two_charge = two_charge;
       if (rates) {
         pl.ke = ke;
         pl.kdd = kdd;
@@ -4422,6 +4429,7 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
     memset(&ro, 0, sizeof(ro));
     ro.Ed = Ed;
     RunPlan pl;
+    pl.two_charge = two_charge;
     pl.Ehalf = Eh;
     pl.sd = d;
     pl.sdd = dd;

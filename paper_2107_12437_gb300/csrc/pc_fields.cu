@@ -1802,10 +1802,11 @@ static cudaError_t launch_far(const pc_ctx *ctx, const Launch &L, int kind, cuda
 }
 
 // Whether a mixed call of T frames may take fields_far_kernel (then far_chosen decides): plane grids
-// of dipoles alone.  Below kFarWork (point, dipole, frame) triples the whole sum takes about as long as
-// asking the device (one read-back, about 10 us).  Sets L.tile_r, the largest distance of a tile's point
+// of dipoles alone.  Asking the device (three launches and a read-back) takes 28 us, which a call whose
+// sources turn out near pays for nothing: below kFarWork (point, dipole, frame) triples that is more than a
+// few percent of it.  Sets L.tile_r, the largest distance of a tile's point
 // from its anchor (c dt).
-constexpr double kFarWork = 8e6;  // fields_mixed_kernel: about 30 us
+constexpr double kFarWork = 1e8;  // fields_mixed_kernel: about 700 us, fields_far_kernel 250
 // lists: (point, dipole, frame) triples from which the far distances (a memset and a small kernel, 5 us) pay
 constexpr double kFarListWork = 2e6;
 static bool far_candidate(Launch &L, bool plane_of_dipoles, int32_t T) {

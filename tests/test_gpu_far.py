@@ -31,9 +31,13 @@ def _sources(N, seed=5, amp=1e-11, t_end=15e-15):
 
 def _check(ctx, dp, nu, nv, times, kind=pc.PC_TOTAL, r_excl=0.0, step=0.5e-9, z=0.4e-6, origin=(0.1e-6, 0.2e-6),
            per_frame=150, nonempty_mask=False):
+    # the frames an odd number of times over, so that the call is large enough (1e8 triples) for the far kernel
+    times = list(times)
+    reps = int(1e8 / (dp.origin.shape[0] * nu * nv * len(times))) + 1
     out = pc.pc_fields_plane(ctx, dipoles=pc.dipoles_to_device(dp), origin=(*origin, z), eu=(step, 0, 0),
-                             ev=(0, step, 0), nu=nu, nv=nv, times=list(times), kind=kind, precision=pc.PC_MIXED,
-                             r_excl=r_excl)
+                             ev=(0, step, 0), nu=nu, nv=nv, times=times * (reps | 1), kind=kind,
+                             precision=pc.PC_MIXED, r_excl=r_excl)
+    out = {k: v[:len(times)] for k, v in out.items()}
     rng = np.random.default_rng(3)
     # scattered points, the grid's corners among them
     p = np.unique(np.r_[0, nv - 1, (nu - 1) * nv, nu * nv - 1, rng.integers(0, nu * nv, per_frame)])
@@ -204,7 +208,7 @@ def test_far_drive_refuses_what_is_not_a_number(ctx):
 
 @pytest.mark.parametrize("amp,near", [(1e-12, 0.0), (1.9e-11, 0.0), (2.8e-11, 0.0), (2.8e-11, 20e-9)])
 def test_mid_pairs_against_float64(ctx, amp, near):
-    # pairs from 20 samples (6 nm) on with charges up to 1.5 amp / 6 nm = 7e-3 of their distance apart, below
+    # pairs from 20 samples (6 nm) on with charges up to amp / 6 nm = 5e-3 of their distance apart, below
     # where the cubic form ends (1e-2) and where charges are too fast (2.86e-11 m); the bounds above
     cfg = _cloud(200, cell=10.2e-9, seed=7)
     cfg.d0[:] = W.E_CHARGE * amp

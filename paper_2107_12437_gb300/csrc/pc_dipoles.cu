@@ -1652,7 +1652,7 @@ __global__ void __launch_bounds__(kRunWarps * 32) lo_far_drive_kernel(const __gr
 // kinks at samples 0 and 1, where the second difference is not small, a source that may have a charge across
 // one at a stage of the block (far_crosses64) is corrected by the difference of pair_drive_f64 and the linear
 // part instead.  (All sources within a block of t = 0 had been: 1.3 blocks a pair, a fifth of 1000 steps.)
-// Measured: a cloud of 1000 oscillators, 320 steps 316 -> 12.7 ms, a ring of 256, 1000 steps 63.4 -> 5.1 ms.  A
+// Measured: a cloud of 1000 oscillators, 320 steps 316 -> 10.9 ms, a ring of 256, 1000 steps 63.4 -> 5.1 ms.  A
 // far pair costs 7 float64 instructions per two of them and 16 positions and about 170 float32 ones per 32
 // stages, a near one about 280 float64 ones per 32 stages: the ring is bound by its 10 near pairs a
 // receiver.  E_d against binary128 on a cloud of 400: 4.6e-13 rms (3.9e-12 with two charges throughout).

@@ -1435,10 +1435,6 @@ __device__ __forceinline__ FarSums far_sources(const RunArgs &a, size_t b0, size
     const bool far = D >= 0, mid = MID && far && (D & kFarMid);
     if (mid) D -= kFarMid;
     const unsigned mf = __ballot_sync(0xffffffffu, far), mm = MID ? __ballot_sync(0xffffffffu, mid) : 0u;
-    if (mid) {
-      const int sl = __popc(mm & ((1u << lane) - 1u)), j = z + a.nsplit * t;
-      s_m[sl] = mid_pair(a, b0 + j, a.pgeo[row + j], pk.w, j, n0 - D - 1);
-    }
     {
       // a charge across sample 0 or 1 from its centre at a stage of this block
       bool wave = false;
@@ -1456,7 +1452,13 @@ __device__ __forceinline__ FarSums far_sources(const RunArgs &a, size_t b0, size
       }
     }
     const int cnt = __popc(mf);
+    // the other lanes' reads of the staged entries of the group before (or of the call before) come first:
+    // the ballots above order no memory accesses
     __syncwarp();
+    if (mid) {
+      const int sl = __popc(mm & ((1u << lane) - 1u)), j = z + a.nsplit * t;
+      s_m[sl] = mid_pair(a, b0 + j, a.pgeo[row + j], pk.w, j, n0 - D - 1);
+    }
     if (far) {
       const int sl = __popc(mf & ((1u << lane) - 1u));
       s_k[sl] = pk;

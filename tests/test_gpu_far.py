@@ -220,6 +220,28 @@ def test_mid_pairs_against_float64(ctx, amp, near):
     assert _err(m["d"], f["d"]) < 1e-9
 
 
+def test_mid_pairs_of_several_groups_of_a_slice(ctx):
+    # one slice of 300 sources, staged 32 at a time, mid pairs in every group: each group's staged entries
+    # have to be read before the next group's take their place, in both passes of a run's first block (the
+    # resumed run starts with two).  The same run in slices of 25 differs by the order of its sums alone
+    cfg = _cloud(300, cell=10.2e-9, seed=13)
+    lod = pc.lo_config_to_device(cfg)
+    state = torch.zeros(pc.pc_dipoles_state_size(ctx, lod, cfg.dt), dtype=torch.float64, device="cuda")
+    f = pc.pc_dipoles_run(ctx, lod, cfg.dt, 203, precision=pc.PC_F64, state_out=state, want_Ed=True)
+    g = pc.pc_dipoles_run(ctx, lod, cfg.dt, 100, precision=pc.PC_F64, state_in=state, want_Ed=True)
+    try:
+        for slices in (1, 12):
+            pc.pc_set_run_tiling(ctx, slices)
+            m = pc.pc_dipoles_run(ctx, lod, cfg.dt, 203, precision=pc.PC_MIXED, want_Ed=True)
+            again = pc.pc_dipoles_run(ctx, lod, cfg.dt, 203, precision=pc.PC_MIXED, want_Ed=True)
+            assert torch.equal(m["Ed"], again["Ed"])
+            assert _err(m["Ed"], f["Ed"]) < 3e-6
+            m = pc.pc_dipoles_run(ctx, lod, cfg.dt, 100, precision=pc.PC_MIXED, state_in=state, want_Ed=True)
+            assert _err(m["Ed"], g["Ed"]) < 3e-6
+    finally:
+        pc.pc_set_run_tiling(ctx, 0)
+
+
 # ------------------------------------------------------------------------------------------------
 # the grid path's block loop in one cooperative launch
 # ------------------------------------------------------------------------------------------------

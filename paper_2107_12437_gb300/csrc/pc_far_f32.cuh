@@ -206,12 +206,20 @@ __device__ __forceinline__ void add_quad_slope(Cubic &c, float sign, float mu, f
 constexpr double kSplitX = 4e-4, kSplitV = 2e-4;
 
 
+// The split form continues the centre's history segment to both charges and adds, for one that has left it,
+// its overshoot times the second difference of the samples at that end: exact on piecewise linear histories
+// only while at most one charge is off the segment, and less than a segment off it.  Seen from any point the
+// charges' retarded samples lie up to |X| (1 + kSplitV) apart, so |X| has to stay below one sample.  (With 2
+// samples the field was 5e-9 off, with 6.7 1e-8; and a charge that far from its centre can be past the end of
+// the history or within an exclusion radius where the centre is not.)
+constexpr float kSplitSamples = 0.95f;
+
 // One dipole's field at a point in the split form, for the float64 field sum and for near fields that
 // cancel in float32: r the separation from its centre (c dt), p its axis, qs = q / e, u the time in samples,
 // d / dd / ddd its float64 history with the scales (1/(qL), 1/(qc), dt/(qc)) and H the float32 mirror.
 // Adds the linear part to lin[10] (float64) and the cubic terms to cub[10] (float32), both as (E, B, phi, A)
 // in the units of dipole_pair.  False, adding nothing, where the two-charge form has to decide: off the
-// interior of the history, within rmin of the centre, or X/R or V beyond the limits at the samples.  Equal
+// interior of the history, within rmin of the centre, or X, X/R or V beyond the limits at the samples.  Equal
 // masses only (the caller's condition).
 // 1/R comes from float32's by one third-order step y (1 + e/2 + 3 e^2/8), e = 1 - R^2 y^2 (its error 5 e^3/16
 // is below 1e-19), the sample index by adding 1.5 * 2^52 with rounding down: about 66 instructions on the
@@ -241,7 +249,8 @@ __device__ __forceinline__ bool split_dipole(double rx, double ry, double rz, do
   const int k = __double2loint(m);
   const double th = (u - (m - magic)) - R;  // (u less a whole number of samples is exact)
   const float4 h0 = __ldg(H + k), h1 = __ldg(H + k + 1);
-  if (!(fmaxf(fabsf(h0.x), fabsf(h1.x)) <= lim.x * Rf && fmaxf(fabsf(h0.y), fabsf(h1.y)) <= lim.v)) return false;
+  if (!(fmaxf(fabsf(h0.x), fabsf(h1.x)) <= fminf(lim.x * Rf, kSplitSamples) && fmaxf(fabsf(h0.y), fabsf(h1.y)) <= lim.v))
+    return false;
   const double d0 = d[k], v0 = dd[k], a0 = ddd[k];
   const double Dd = d[k + 1] - d0, Dv = dd[k + 1] - v0, Da = ddd[k + 1] - a0;
   double X = fma(th, Dd, d0), V = fma(th, Dv, v0), A = fma(th, Da, a0);

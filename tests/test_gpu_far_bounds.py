@@ -1,0 +1,117 @@
+"""Where the far and split forms end (csrc/pc_far_f32.cuh): separations of a dipole's charges of more than one
+sample c dt, planes whose tiles are wide against the distance of their sources, moments that grow during a run,
+and devices without the memory for the forms' tables.  References: binary128 and the FP64 oracle."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2107_12437_gb300 as pc
+import workloads as W
+from test_gpu_far import OMEGA0, _cloud, _ed_binary128
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = pc.Context(0)
+    yield c
+    c.close()
+
+
+def _norm(v):
+    return np.abs(v) if v.ndim == 2 else np.linalg.norm(v, axis=-1)
+
+
+# ------------------------------------------------------------------------------------------------
+# separations of more than one sample: the float64 field sum
+# ------------------------------------------------------------------------------------------------
+# dt, separation of the charges, distance, extent of the sources, histories' end, frames: the separations are
+# 0.33, 0.95, 1.05, 2, 6.7 and 3.3 samples; the last one's charges are slow enough only near their turning
+# points, at which the frames look (sources within 20 nm, retarded by 17.5 um, and the quarter period)
+_SPREAD = {
+    "10 pm": (1e-19, 1e-11, 1.2e-6, 2e-7, 8e-15, (6.6e-15, 7.3e-15)),
+    "28.4 pm": (1e-19, 2.84e-11, 1.2e-6, 2e-7, 8e-15, (6.6e-15, 7.3e-15)),
+    "31.6 pm": (1e-19, 3.16e-11, 1.2e-6, 2e-7, 8e-15, (6.6e-15, 7.3e-15)),
+    "60 pm": (1e-19, 6e-11, 1.2e-6, 2e-7, 8e-15, (6.6e-15, 7.3e-15)),
+    "200 pm": (1e-19, 2e-10, 4.1e-6, 2e-8, 20e-15, tuple(4.09e-6 / W.C + (k + 0.5) * 2.5e-15 for k in (0, 1))),
+    "1 nm": (1e-18, 1e-9, 17.5e-6, 2e-8, 80e-15, tuple(17.49e-6 / W.C + (k + 0.5) * 2.5e-15 for k in (2, 5))),
+}
+
+
+@pytest.mark.parametrize("kind", [pc.PC_TOTAL, pc.PC_COULOMB, pc.PC_RADIATION])
+@pytest.mark.parametrize("case", sorted(_SPREAD))
+def test_float64_fields_of_wide_dipoles(ctx, case, kind):
+    # the bound of tests/test_gpu_far.py::test_split_fields_against_binary128, five sources at random places
+    dt, amp, z, ext, t_end, times = _SPREAD[case]
+    rng = np.random.default_rng(31)
+    dp = W.sinusoidal_dipoles(rng.uniform(0.0, ext, (5, 3)), W.unit_vectors(rng, 5), OMEGA0, amp, dt, t_end)
+    P = 11003
+    pts = np.concatenate([rng.uniform(0.0, ext, (P, 2)), np.full((P, 1), z)], axis=1)
+    out = pc.pc_fields(ctx, dipoles=pc.dipoles_to_device(dp), points=torch.as_tensor(pts, device="cuda"),
+                       times=list(times), kind=kind)
+    p = np.r_[0, P - 1, rng.integers(0, P, 60)]
+    ref = oracle.fields_x(pts[p], times, dipoles=dp, kind=kind)
+    scale = oracle.fields(pts[p], times, dipoles=dp, kind=kind)["scale_source"]
+    assert ref["status"] == oracle.OK and not out["mask"].any()
+    worst = {}
+    for k in ("E", "B", "phi", "A"):
+        g = out[k][:, torch.as_tensor(p, device="cuda")].cpu().numpy()
+        sc = scale["E"] / W.C if k == "B" else scale[k]
+        worst[k] = float(np.max(_norm(g - ref[k]) / np.maximum(_norm(ref[k]), 1e-3 * sc)))
+    assert max(worst.values()) <= 1e-10, worst
+
+
+# 600 pm at 0.1 as: 20 samples, so that a charge lies up to 10 from its centre; 12 um away, where every form's
+# condition on separation over distance holds.  The moment rests, and all points are the same one.
+_WIDE = dict(dt=1e-19, amp=6e-10, S=3001, R=12e-6)
+
+
+def _resting(N):
+    d = W.E_CHARGE * _WIDE["amp"] * np.ones((N, _WIDE["S"]))
+    z = np.zeros((N, _WIDE["S"]))
+    one = np.ones(N)
+    axis = np.tile([0.0, 0.0, 1.0], (N, 1))
+    return W.Dipoles(origin=np.zeros((N, 3)), axis=axis, q=W.E_CHARGE * one, m1=W.M_E * one, m2=W.M_E * one, d=d, d_dot=z,
+                     d_ddot=z.copy(), t0=0.0, dt=_WIDE["dt"])
+
+
+def _wide_call(ctx, form, time, r_excl=0.0):
+    # enough (point, dipole) pairs for the form to be taken: 1e5, 2e6 and 1e8
+    N, nu, nv = {"float64": (4, 160, 160), "list": (4, 710, 710), "plane": (64, 1300, 1300)}[form]
+    dp = pc.dipoles_to_device(_resting(N))
+    kw = dict(dipoles=dp, times=[time], r_excl=r_excl, precision=pc.PC_F64 if form == "float64" else pc.PC_MIXED)
+    if form == "plane":
+        return pc.pc_fields_plane(ctx, origin=(0.0, 0.0, _WIDE["R"]), eu=(1e-18, 0, 0), ev=(0, 1e-18, 0), nu=nu, nv=nv, **kw)
+    pts = torch.zeros((nu * nv, 3), dtype=torch.float64, device="cuda")
+    pts[:, 2] = _WIDE["R"]
+    return pc.pc_fields(ctx, points=pts, **kw)
+
+
+@pytest.mark.parametrize("form", ["float64"])
+def test_charge_beyond_the_end_of_its_history(ctx, form):
+    # the centre's retarded time 9.5 samples inside the history, the nearer charge's half a sample past it
+    pt = np.array([[0.0, 0.0, _WIDE["R"]]])
+    for inside, status in ((9.5, oracle.ERR_HISTORY), (10.5, oracle.OK)):
+        time = _WIDE["R"] / W.C + (_WIDE["S"] - 1 - inside) * _WIDE["dt"]
+        assert oracle.fields(pt, [time], dipoles=_resting(1))["status"] == status
+        if status == oracle.OK:
+            assert not _wide_call(ctx, form, time)["mask"].any()
+        else:
+            with pytest.raises(pc.PcError, match="PC_ERR_HISTORY"):
+                _wide_call(ctx, form, time)
+
+
+@pytest.mark.parametrize("form", ["float64"])
+def test_charge_within_the_exclusion_radius(ctx, form):
+    # the centre 9.5 samples outside r_excl, the nearer charge half a sample inside
+    pt = np.array([[0.0, 0.0, _WIDE["R"]]])
+    time = _WIDE["R"] / W.C + 1000 * _WIDE["dt"]
+    for outside, masked in ((9.5, True), (10.5, False)):
+        r_excl = _WIDE["R"] - outside * _WIDE["dt"] * W.C
+        assert bool(oracle.fields(pt, [time], dipoles=_resting(1), r_excl=r_excl)["mask"].all()) == masked
+        m = _wide_call(ctx, form, time, r_excl)["mask"]
+        assert bool(m.all()) == masked and bool(m.any()) == masked

@@ -219,8 +219,8 @@ constexpr float kSplitSamples = 0.95f;
 // d / dd / ddd its float64 history with the scales (1/(qL), 1/(qc), dt/(qc)) and H the float32 mirror.
 // Adds the linear part to lin[10] (float64) and the cubic terms to cub[10] (float32), both as (E, B, phi, A)
 // in the units of dipole_pair.  False, adding nothing, where the two-charge form has to decide: off the
-// interior of the history, within rmin of the centre, or X, X/R or V beyond the limits at the samples.  Equal
-// masses only (the caller's condition).
+// interior of the history, within rmin of the centre, X, X/R or V beyond the limits at the samples, or
+// samples that are not those of a smooth motion.  Equal masses only (the caller's condition).
 // 1/R comes from float32's by one third-order step y (1 + e/2 + 3 e^2/8), e = 1 - R^2 y^2 (its error 5 e^3/16
 // is below 1e-19), the sample index by adding 1.5 * 2^52 with rounding down: about 66 instructions on the
 // float64 unit a pair, where the two charges' roots and difference form take 280.
@@ -259,6 +259,8 @@ __device__ __forceinline__ bool split_dipole(double rx, double ry, double rz, do
   // (the slopes from the float64 samples: a difference of float32 ones is good to 5e-5 only, which put
   // 1e-14 instead of 1e-15 into the fields of 10 pm dipoles)
   const float dX = (float)(Dd * sx), dV = (float)(Dv * sv), dA = (float)(Da * sa);
+  // (the slope of X enters as a speed does; samples of d need not follow those of d')
+  if (!(fabsf(dX) <= lim.v)) return false;
   const float Xf = fmaf(thf, dX, h0.x);
   // a charge whose own retarded time lies off the centre's segment: its state differs from the segment's
   // extension by the overshoot times the second difference of the samples.  The charges' delays are off the
@@ -283,6 +285,12 @@ __device__ __forceinline__ bool split_dipole(double rx, double ry, double rz, do
       ex = (float)(eX * sx) * iRf;
       ev = (float)(eV * sv);
       ea = (float)(eA * sa) * Rf;
+      // what is left out, of the order of the change e times the change of X's slope there or the square of
+      // (X/R, V), stays below 1e-11 of the pair's field for every history that its samples resolve (140 a
+      // period); others (noise, jumps) take the two charges here
+      const float kink = fabsf((float)(((d[n + 1] - d[n]) - (d[n] - d[n - 1])) * sx)) + 3e-8f;
+      if (!(kink * (fabsf(ex) + fabsf(ev) + fabsf(ea)) <= 1e-11f * (fabsf(Xf) * iRf + fabsf(h0.y) + fabsf(h0.z) * Rf)))
+        return false;
     }
   }
   X *= sx;

@@ -115,3 +115,43 @@ def test_charge_within_the_exclusion_radius(ctx, form):
         assert bool(oracle.fields(pt, [time], dipoles=_resting(1), r_excl=r_excl)["mask"].all()) == masked
         m = _wide_call(ctx, form, time, r_excl)["mask"]
         assert bool(m.all()) == masked and bool(m.any()) == masked
+
+
+# ------------------------------------------------------------------------------------------------
+# histories that are not smooth: the float64 field sum
+# ------------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("kind", [pc.PC_TOTAL, pc.PC_COULOMB, pc.PC_RADIATION])
+@pytest.mark.parametrize("case", ["d", "d_ddot", "all", "step", "mixture"])
+def test_float64_fields_of_rough_histories(ctx, case, kind):
+    # the fields are those of the piecewise linear samples, whatever these are: noise of a tenth of the moment
+    # from sample to sample, one step of it, or noise in one dipole of five; bound as above
+    rng = np.random.default_rng(17)
+    dp = W.sinusoidal_dipoles(rng.uniform(0.0, 2e-7, (5, 3)), W.unit_vectors(rng, 5), OMEGA0, 1e-11, 1e-18, 9e-15)
+    noise = rng.uniform(-0.1, 0.1, (3,) + dp.d.shape)
+    if case == "mixture":
+        noise[:, 1:] = 0.0
+    if case in ("d", "all", "mixture"):
+        dp.d += W.E_CHARGE * 1e-11 * noise[0]
+    if case in ("all", "mixture"):
+        dp.d_dot += W.E_CHARGE * 1e-11 * OMEGA0 * noise[1]
+    if case in ("d_ddot", "all", "mixture"):
+        dp.d_ddot += W.E_CHARGE * 1e-11 * OMEGA0 ** 2 * noise[2]
+    if case == "step":
+        dp.d[:, 6000:] += W.E_CHARGE * 1e-12
+    times = [7.5e-15, 8.9e-15]
+    P = 11003
+    pts = np.concatenate([rng.uniform(0.0, 2e-7, (P, 2)), np.full((P, 1), 4.5e-7)], axis=1)
+    out = pc.pc_fields(ctx, dipoles=pc.dipoles_to_device(dp), points=torch.as_tensor(pts, device="cuda"),
+                       times=times, kind=kind)
+    # points whose retarded samples of the first source lie around the step, and others
+    late = np.linalg.norm(pts - dp.origin[0], axis=1) / (W.C * 1e-18)
+    p = np.r_[np.argsort(np.abs(late - 1500.0))[:40], rng.integers(0, P, 160)]
+    ref = oracle.fields_x(pts[p], times, dipoles=dp, kind=kind)
+    scale = oracle.fields(pts[p], times, dipoles=dp, kind=kind)["scale_source"]
+    assert ref["status"] == oracle.OK and not out["mask"].any()
+    worst = {}
+    for k in ("E", "B", "phi", "A"):
+        g = out[k][:, torch.as_tensor(p, device="cuda")].cpu().numpy()
+        sc = scale["E"] / W.C if k == "B" else scale[k]
+        worst[k] = float(np.max(_norm(g - ref[k]) / np.maximum(_norm(ref[k]), 1e-3 * sc)))
+    assert max(worst.values()) <= 1e-10, worst

@@ -249,7 +249,9 @@ __device__ __forceinline__ bool split_dipole(double rx, double ry, double rz, do
   const int k = __double2loint(m);
   const double th = (u - (m - magic)) - R;  // (u less a whole number of samples is exact)
   const float4 h0 = __ldg(H + k), h1 = __ldg(H + k + 1);
-  if (!(fmaxf(fabsf(h0.x), fabsf(h1.x)) <= fminf(lim.x * Rf, kSplitSamples) && fmaxf(fabsf(h0.y), fabsf(h1.y)) <= lim.v))
+  // (the slope of X enters as a speed does; samples of d need not follow those of d')
+  if (!(fmaxf(fabsf(h0.x), fabsf(h1.x)) <= fminf(lim.x * Rf, kSplitSamples) &&
+        fmaxf(fmaxf(fabsf(h0.y), fabsf(h1.y)), fabsf(h1.x - h0.x)) <= lim.v))
     return false;
   const double d0 = d[k], v0 = dd[k], a0 = ddd[k];
   const double Dd = d[k + 1] - d0, Dv = dd[k + 1] - v0, Da = ddd[k + 1] - a0;
@@ -259,8 +261,6 @@ __device__ __forceinline__ bool split_dipole(double rx, double ry, double rz, do
   // (the slopes from the float64 samples: a difference of float32 ones is good to 5e-5 only, which put
   // 1e-14 instead of 1e-15 into the fields of 10 pm dipoles)
   const float dX = (float)(Dd * sx), dV = (float)(Dv * sv), dA = (float)(Da * sa);
-  // (the slope of X enters as a speed does; samples of d need not follow those of d')
-  if (!(fabsf(dX) <= lim.v)) return false;
   const float Xf = fmaf(thf, dX, h0.x);
   // a charge whose own retarded time lies off the centre's segment: its state differs from the segment's
   // extension by the overshoot times the second difference of the samples.  The charges' delays are off the
@@ -288,8 +288,9 @@ __device__ __forceinline__ bool split_dipole(double rx, double ry, double rz, do
       // what is left out, of the order of the change e times the change of X's slope there or the square of
       // (X/R, V), stays below 1e-11 of the pair's field for every history that its samples resolve (140 a
       // period); others (noise, jumps) take the two charges here
-      const float kink = fabsf((float)(((d[n + 1] - d[n]) - (d[n] - d[n - 1])) * sx)) + 3e-8f;
-      if (!(kink * (fabsf(ex) + fabsf(ev) + fabsf(ea)) <= 1e-11f * (fabsf(Xf) * iRf + fabsf(h0.y) + fabsf(h0.z) * Rf)))
+      const float of = (float)o;
+      if (!(fmaf(fabsf(ex), Rf, 3e-8f * of) * (fabsf(ex) + fabsf(ev) + fabsf(ea)) <=
+            1e-11f * of * (fabsf(Xf) * iRf + fabsf(h0.y) + fabsf(h0.z) * Rf)))
         return false;
     }
   }

@@ -250,8 +250,10 @@ __device__ __forceinline__ bool split_dipole(double rx, double ry, double rz, do
   const double th = (u - (m - magic)) - R;  // (u less a whole number of samples is exact)
   const float4 h0 = __ldg(H + k), h1 = __ldg(H + k + 1);
   // (the slope of X enters as a speed does; samples of d need not follow those of d')
-  if (!(fmaxf(fabsf(h0.x), fabsf(h1.x)) <= fminf(lim.x * Rf, kSplitSamples) &&
-        fmaxf(fmaxf(fabsf(h0.y), fabsf(h1.y)), fabsf(h1.x - h0.x)) <= lim.v))
+  // (each by itself: a maximum would pass over a NaN, which the two-charge form refuses in d)
+  const float xl = fminf(lim.x * Rf, kSplitSamples);
+  if (!(fabsf(h0.x) <= xl && fabsf(h1.x) <= xl && fabsf(h0.y) <= lim.v && fabsf(h1.y) <= lim.v &&
+        fabsf(h1.x - h0.x) <= lim.v))
     return false;
   const double d0 = d[k], v0 = dd[k], a0 = ddd[k];
   const double Dd = d[k + 1] - d0, Dv = dd[k + 1] - v0, Da = ddd[k + 1] - a0;

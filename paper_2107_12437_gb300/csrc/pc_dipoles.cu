@@ -1268,7 +1268,10 @@ __global__ void __launch_bounds__(256) lo_pairs_kernel(const RunArgs a) {
         if (a.pfar64) {
           // p_i . E of the split form's linear part, with the charge's unit and the samples' scales:
           // k1 d + k2 d' + k3 d'' is the field in V/m
-          const bool far = i != j && fl >= kFarDelay && a.m1[bj] == a.m2[bj] && xd <= kSplitX * x && xd <= 8.0 &&
+          // (kSplitSamples: the drive and its reverse, too, take one second difference for a charge off its
+          // centre's segment)
+          const bool far = i != j && fl >= kFarDelay && a.m1[bj] == a.m2[bj] && xd <= kSplitX * x &&
+                           xd * kFarGrow <= (double)kSplitSamples &&
                            xd * __longlong_as_double((long long)a.amax[2 * b + 1]) * a.dt <= kSplitV;
           const double ir = 1.0 / r, c1 = (dx * pj_[0] + dy * pj_[1] + dz * pj_[2]) * ir,
                        c2 = (dx * pi_[0] + dy * pi_[1] + dz * pi_[2]) * ir,

@@ -181,3 +181,42 @@ def test_float64_fields_of_a_sample_that_is_no_number(ctx, which, side):
     small = call(500)
     assert small == call(40001)
     assert small == pc.capi.PC_ERR_NOCONV if which == "d" else True in small.values()
+
+
+# ------------------------------------------------------------------------------------------------
+# separations of more than one sample: the float64 run and its gradients
+# ------------------------------------------------------------------------------------------------
+def _wide_cloud(amp, dt, N=70, cell=1.6e-7, steps=9000):
+    """_cloud() with steps of dt and charges amp apart; pairs from 1.1e-7 m on, most of them past one light
+    crossing within the steps."""
+    cfg = _cloud(N, cell=cell, seed=41)
+    cfg.dt = dt
+    cfg.d0[:] = W.E_CHARGE * amp
+    cfg.n_steps = steps
+    return cfg
+
+
+@pytest.mark.parametrize("amp,dt,steps", [(1.8e-11, 1e-19, 9000), (4.5e-11, 1e-19, 9000), (4.5e-11, 2e-20, 45000)])
+def test_float64_drive_of_wide_dipoles(ctx, amp, dt, steps):
+    # 0.6, 1.5 and 7.5 samples: E_d on the run's own history within the float64 path's 1e-10 of its largest value
+    cfg = _wide_cloud(amp, dt)
+    f = pc.pc_dipoles_run(ctx, pc.lo_config_to_device(cfg), dt, steps, precision=pc.PC_F64, want_Ed=True)
+    at = np.linspace(steps // 2, steps, 29).astype(int) - np.arange(29) % 7
+    recv = [0, 33, 69]
+    h = [f[k][0].cpu().numpy() for k in ("d", "d_dot", "d_ddot")]
+    ref = _ed_binary128(cfg, h, 0.0, at * dt, recv)
+    err = [float(np.max(np.abs(f["Ed"][0, i].cpu().numpy()[at] - e)) / np.max(np.abs(e))) for e, i in zip(ref, recv)]
+    assert max(err) < 1e-10, err
+
+
+@pytest.mark.parametrize("amp,dt,steps", [(1.8e-11, 1e-19, 9000), (4.5e-11, 1e-19, 9000)])
+def test_float64_gradients_of_wide_dipoles(ctx, amp, dt, steps):
+    # as tests/test_gpu_far.py::test_split_reverse_against_the_two_charge_form: masses one rounding apart keep
+    # every pair in the two-charge form (a cloud of 0.15 um: its delays have to lie within some 9000 samples)
+    cfg = _wide_cloud(amp, dt, cell=3e-8)
+    w = torch.linspace(0.5, 1.5, cfg.N, dtype=torch.float64, device="cuda").view(1, cfg.N)
+    got = pc.pc_dipoles_adjoint(ctx, pc.lo_config_to_device(cfg), dt, steps, w)
+    cfg.m1 = np.nextafter(cfg.m1, np.inf)
+    ref = pc.pc_dipoles_adjoint(ctx, pc.lo_config_to_device(cfg), dt, steps, w)
+    err = [float((g - r).abs().max() / r.abs().max()) for g, r in zip(got, ref)]
+    assert max(err) < 1e-10, err

@@ -1722,10 +1722,12 @@ __global__ void far_limit_kernel(int N, const unsigned *xvmax, const float4 *src
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= N) return;
   const float4 mu = srcf[4 * j + 1];
-  // not below kNearL (nearer pairs are tested for a near field that cancels), nor where a charge may
-  // lie within r_excl
-  rfar[j] = fmaxf(fmaxf(kNearL, rex_fast),
-                  far_limit(__uint_as_float(xvmax[2 * j]), __uint_as_float(xvmax[2 * j + 1]), mu.x, mu.y));
+  const float x = __uint_as_float(xvmax[2 * j]);
+  // not below kNearL (nearer pairs are tested for a near field that cancels), nor where a charge may lie within
+  // r_excl; nowhere for charges that may be a sample or more from their centre, as the margins kept at the
+  // history's ends and about r_excl are for less
+  rfar[j] = x <= kSplitSamples ? fmaxf(fmaxf(kNearL, rex_fast), far_limit(x, __uint_as_float(xvmax[2 * j + 1]), mu.x, mu.y))
+                               : __int_as_float(0x7f800000);
 }
 
 // ================================================================================================

@@ -91,7 +91,7 @@ def _wide_call(ctx, form, time, r_excl=0.0):
     return pc.pc_fields(ctx, points=pts, **kw)
 
 
-@pytest.mark.parametrize("form", ["float64"])
+@pytest.mark.parametrize("form", ["float64", "list", "plane"])
 def test_charge_beyond_the_end_of_its_history(ctx, form):
     # the centre's retarded time 9.5 samples inside the history, the nearer charge's half a sample past it
     pt = np.array([[0.0, 0.0, _WIDE["R"]]])
@@ -105,7 +105,7 @@ def test_charge_beyond_the_end_of_its_history(ctx, form):
                 _wide_call(ctx, form, time)
 
 
-@pytest.mark.parametrize("form", ["float64"])
+@pytest.mark.parametrize("form", ["float64", "list", "plane"])
 def test_charge_within_the_exclusion_radius(ctx, form):
     # the centre 9.5 samples outside r_excl, the nearer charge half a sample inside
     pt = np.array([[0.0, 0.0, _WIDE["R"]]])

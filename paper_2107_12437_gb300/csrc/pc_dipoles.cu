@@ -1379,7 +1379,8 @@ __global__ void __launch_bounds__(kRunWarps * 32) lo_drive_kernel(const RunArgs 
 // rest state before t = 0, d'' comes up within the first segment: the samples have kinks at 0 and 1, which the
 // two charges' retarded times meet apart.  Where one of them is across a kink from the centre's by o samples,
 // the form's linear continuation is off by mu o times the second difference of g there, which is added (a
-// stage or none per pair and kink; moments stay within 8 c dt, so that four samples around it are enough).
+// stage or none per pair and kink); moments that are wide against the distance take pair_drive_f32 at these
+// stages (far_wide).
 // The two forms' whole difference there had cost 1.25 blocks of pair_drive_f32 a pair, a third of 1000 steps
 // of 4096 oscillators.
 // A block whose reach holds a sample beyond the limits (a.nbad) goes through lo_drive_kernel's sources
@@ -1411,6 +1412,11 @@ __device__ __forceinline__ float mid_terms(float4 p, float R, float4 h) {
   const Cubic q = cubic_terms(p.x, h.x * p.w, h.y, al, h.y, al, 0.f);
   return fmaf(q.Ca, p.y, q.D * p.z);
 }
+// Whether a source's kinks take the two charges' whole field (x0 its moment while at rest): where only one charge
+// has met a kink the terms of second order in X/R do not cancel between them, X (X/R) of the step that the
+// field makes there.  Up to 8e-6 (every far pair of 10 pm charges at steps of 1 as) that is left out; with 3 to 7
+// samples between the charges it was 1e-4 of the step, 5e-5 of E_d.
+__device__ __forceinline__ bool far_wide(float x0, float R) { return x0 * x0 > 8e-6f * R; }
 // The far sources of slice z (table rows from tab), samples at positions 2 + m + shift (m = lane & 15) of
 // the block at n0: sums per position over the slice's sources, groups of 32 compensated.  A slice takes
 // every nsplit-th source, so that the near ones, neighbours in index as often as not, spread over them.
@@ -1445,8 +1451,10 @@ __device__ __forceinline__ FarSums far_sources(const RunArgs &a, size_t b0, size
         const float4 gg = a.pgeo[row + z + a.nsplit * t];
         const float x0 = reinterpret_cast<const float4 *>(H + (size_t)(unsigned)(z + a.nsplit * t) * hb)->x;
         const float c = (float)(n0 - D) - pk.w, hd = fabsf(__fdividef(x0 * gg.y, gg.x)) + 1e-4f;
+        const bool wide = far_wide(x0, gg.x);
         const float s0 = fminf(fmaxf(rintf(-2.f * c), 1.f), 2.f * a.K), s1 = fminf(fmaxf(rintf(2.f - 2.f * c), 1.f), 2.f * a.K);
-        wave = fabsf(fmaf(0.5f, s0, c)) <= hd || fabsf(fmaf(0.5f, s1, c - 1.f)) <= hd;
+        wave = fabsf(fmaf(0.5f, s0, c)) <= hd || fabsf(fmaf(0.5f, s1, c - 1.f)) <= hd ||
+               (wide && c + 0.5f <= 1.f + hd && c + (float)a.K >= -hd);
       }
       const unsigned m1 = __ballot_sync(0xffffffffu, D == kFarNear), m2 = __ballot_sync(0xffffffffu, wave);
       if (lane == (t0 >> 5)) {
@@ -1520,6 +1528,28 @@ __device__ __forceinline__ FarSums far_sources(const RunArgs &a, size_t b0, size
   return S;
 }
 
+// A far pair's field at a stage from both charges, less its far form's (table entry e): zero where neither is
+// between the kinks.  Out of line: it runs for a few stages of a pair's first block only.
+template <bool RING, bool MID>
+__device__ __noinline__ float wide_crossing(const RunArgs &a, int b, int i, int j, size_t e, int n0, float stage_f, int *err) {
+  const size_t ij = bidx(a, b, i) * (size_t)a.N + j, bj = bidx(a, b, j);
+  const int2 dl = a.delay[ij];
+  const float4 geo = a.pgeo[ij], pk = a.pfar[e];
+  const float4 *hj = a.H32 + bj * (size_t)a.hs;
+  const int mask = RING ? (int)a.wm : -1;
+  const float xs = stage_f - __int_as_float(dl.y);
+  if (fabsf((float)(n0 - dl.x) + xs - 0.5f) > 0.5f + fabsf(__fdividef(hj[0].x * geo.y, geo.x)) + 1e-3f) return 0.f;
+  float flf;
+  const int k = n0 - dl.x + Num<float>::floor_int(xs, flf);
+  const float4 h0 = hj[max(k, 0) & mask], h1 = hj[max(k + 1, 0) & mask];
+  float g0 = fmaf(pk.z, h0.z, fmaf(pk.y, h0.y, pk.x * h0.x)), g1 = fmaf(pk.z, h1.z, fmaf(pk.y, h1.y, pk.x * h1.x));
+  if (MID && (a.pfarD[e] & kFarMid)) {
+    const MidPair q = mid_pair(a, bj, geo, 0.f, j, 0);
+    g0 += mid_terms(q.p, geo.x, h0);
+    g1 += mid_terms(q.p, geo.x, h1);
+  }
+  return pair_drive_f32<RING>(a, b, i, j, k, xs - flf, geo, n0 + 1, err) - fmaf(xs - flf, g1 - g0, g0);
+}
 // One warp's part of a block: receiver i, source slice z, stages into dst[1 .. ns]; s_k, s_j its staging
 // buffers, sh 32 doubles; nbad the last sample beyond the limits (before this block), or -1.
 template <bool NEAR, bool RING, bool MID, int U>
@@ -1595,6 +1625,10 @@ __device__ __forceinline__ void far_block(const RunArgs &a, int b, int i, int z,
       const float4 cj = *reinterpret_cast<const float4 *>(a.dipf + (b0 + j) * kDipF + 8);  // (p_z, mu+, mu-, q/e)
       const float4 *hj = a.H32 + (b0 + (size_t)j) * (size_t)a.hs;
       const float4 h0 = hj[0], h1_ = hj[1], h2_ = hj[2];
+      if (far_wide(h0.x, geo.x)) {
+        if (lane < ns) grp += wide_crossing<RING, MID>(a, b, i, j, tab + t0 + l, n0, stage_f, &err);
+        continue;
+      }
       // the charge whose offset points at the sample from the centre's retarded time passes it by o samples
       const float xs = (float)(n0 - dl.x) + (stage_f - __int_as_float(dl.y)), sx = __fdividef(h0.x * geo.y, geo.x);
       const float w0 = (xs < 0.f) == (sx > 0.f) ? cj.y : cj.z, w1 = (xs < 1.f) == (sx > 0.f) ? cj.y : cj.z;
@@ -1634,8 +1668,11 @@ __device__ __forceinline__ bool block_at(const RunArgs &a, int64_t &n0, int &ns)
   }
   return true;
 }
+// (three CTAs per SM keep enough gathers in flight: with 102 registers and two, 1000 steps of 4096 oscillators
+// took 34.3 ms instead of 27.8)
 template <bool NEAR, bool RING, bool MID>
-__global__ void __launch_bounds__(kRunWarps * 32) lo_far_drive_kernel(const __grid_constant__ RunArgs a, int64_t n0, int ns) {
+__global__ void __launch_bounds__(kRunWarps * 32, NEAR ? 2 : 3)
+    lo_far_drive_kernel(const __grid_constant__ RunArgs a, int64_t n0, int ns) {
   __shared__ double sh[kRunWarps][32];
   __shared__ float4 s_k[kRunWarps][34];
   __shared__ int2 s_j[kRunWarps][34];

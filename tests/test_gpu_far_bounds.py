@@ -220,3 +220,17 @@ def test_float64_gradients_of_wide_dipoles(ctx, amp, dt, steps):
     ref = pc.pc_dipoles_adjoint(ctx, pc.lo_config_to_device(cfg), dt, steps, w)
     err = [float((g - r).abs().max() / r.abs().max()) for g, r in zip(got, ref)]
     assert max(err) < 1e-10, err
+
+
+@pytest.mark.parametrize("amp,dt,steps,cell", [(1.8e-11, 1e-19, 9000, 1.6e-7), (2.8e-11, 3e-20, 20000, 4e-8),
+                                               (2e-11, 1e-20, 60000, 1e-7)])
+def test_mixed_drive_of_wide_dipoles(ctx, amp, dt, steps, cell):
+    # 0.6, 3.1 and 6.7 samples: E_d within 1e-5 of its largest value, the bound of
+    # tests/test_gpu_far.py::test_far_drive_against_oracle, also in the steps in which the field of a source sets
+    # in, its two charges' one after the other
+    cfg = _wide_cloud(amp, dt, cell=cell)
+    lod = pc.lo_config_to_device(cfg)
+    f = pc.pc_dipoles_run(ctx, lod, dt, steps, precision=pc.PC_F64, want_Ed=True)
+    m = pc.pc_dipoles_run(ctx, lod, dt, steps, precision=pc.PC_MIXED, want_Ed=True)
+    e = float(((m["Ed"] - f["Ed"]).abs().amax(-1) / f["Ed"].abs().amax(-1)).max())
+    assert e < 1e-5, e

@@ -1395,7 +1395,7 @@ __device__ __forceinline__ AnchorGeo anchor_geo(const Launch &L, const float *hi
 // whether a source is far for every point within L.tile_r of the anchor, all their retarded samples
 // (and, a sample further, the charges') on interior segments of the history
 __device__ __forceinline__ bool tile_far(const Launch &L, const AnchorGeo &g, int j) {
-  const float rt = L.tile_r;  // below 1e5 (the host's condition for this kernel)
+  const float rt = L.tile_r;  // at most kFarTile
   const int ir = (int)rt + 2;
   // (anchor samples from 2^22 on are beyond the float floor's range)
   return g.n.hi - rt >= L.rfar[j] && g.k >= ir + 2 && g.k < (1 << 22) && g.k + ir <= (int)L.src.Sd - 5;
@@ -1511,7 +1511,11 @@ __device__ __forceinline__ int near_sources_far(const Launch &L, int f, int n, i
   return err;
 }
 
-template <int KIND, int NF>
+// FINE: |rho|^2 as |g|^2 and its difference.  That cancels where a point is much nearer to the source than the
+// tile's anchor (with steps of 40 nm the field was 1e-5 off there), so it serves tiles that are small against every
+// far distance (far_fine: then |g| <= 1.25 |rho|, and it rounds like the other sum); wider ones add up the squares
+// of the components.  (That for all: 10.0 -> 10.25 ms on the field grid.)
+template <int KIND, int NF, bool FINE>
 __global__ void __launch_bounds__(kMixThreads, 2)
     fields_far_kernel(const __grid_constant__ Launch L, int64_t tiles_v, int reps) {
   __shared__ float s_anc_hi[3], s_anc_lo[3];
@@ -1590,7 +1594,8 @@ __global__ void __launch_bounds__(kMixThreads, 2)
           // |rho|^2 - |g|^2 = 2 g.dr + dr^2, 1/|rho|, |rho| - |g| = (|rho|^2 - |g|^2) / (|rho| + |g|)
           const V2 gx(a.x), gy(a.y), gz(a.z), px(b.x), py(b.y), pz(b.z);
           const V2 num = fma2(gx, Dx, fma2(gy, Dy, fma2(gz, Dz, dr2)));
-          const V2 rho2 = num + V2(b.w);
+          const V2 rx = fma2(half, Dx, gx), ry = fma2(half, Dy, gy), rz = fma2(half, Dz, gz);
+          const V2 rho2 = FINE ? num + V2(b.w) : fma2(rz, rz, fma2(ry, ry, rx * rx));
           const V2 i(rsqrt_fast(rho2.v.x), rsqrt_fast(rho2.v.y));
           const V2 den = fma2(rho2, i, V2(a.w));
           const V2 corr = num * V2(rcp_fast(den.v.x), rcp_fast(den.v.y));
@@ -1611,7 +1616,6 @@ __global__ void __launch_bounds__(kMixThreads, 2)
             h[n][2] = __ldg(hB);
             h[n][3] = __ldg(hB + 1);
           }
-          const V2 rx = fma2(half, Dx, gx), ry = fma2(half, Dy, gy), rz = fma2(half, Dz, gz);
           const V2 rp = fma2(rz, pz, fma2(ry, py, rx * px));
           const V2 cx = fma2(py, rz, -(pz * ry)), cy = fma2(pz, rx, -(px * rz)), cz = fma2(px, ry, -(py * rx));
           const V2 i2 = i * i, rpi2 = rp * i2, m = rpi2 * i, i3_ = V2(3.f) * i;
@@ -1764,10 +1768,10 @@ static void launch_mixed_list(const Launch &L, dim3 grid, int kind, cudaStream_t
 // Frames in twos, a last odd one by itself; each CTA walks as many of them as leave the grid kFarWaves
 // waves of two CTAs per SM.
 constexpr int kFarWaves = 8;
-template <int KIND, int NF>
+template <int KIND, int NF, bool FINE>
 static cudaError_t launch_far_nf(const pc_ctx *ctx, const Launch &L, int64_t tiles, int64_t tiles_v, cudaStream_t st) {
   const size_t smem = sizeof(KahanFar<NF>);
-  auto *fn = fields_far_kernel<KIND, NF>;
+  auto *fn = fields_far_kernel<KIND, NF, FINE>;
   const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int64_t groups = (L.T + NF - 1) / NF, want = (int64_t)kFarWaves * 2 * ctx->num_sms;
@@ -1775,12 +1779,15 @@ static cudaError_t launch_far_nf(const pc_ctx *ctx, const Launch &L, int64_t til
   fn<<<dim3((unsigned)tiles, (unsigned)((groups + reps - 1) / reps)), kMixThreads, smem, st>>>(L, tiles_v, reps);
   return cudaSuccess;
 }
+// (no source is far within kNearL, far_limit_kernel)
+static bool far_fine(const Launch &L) { return 4.f * L.tile_r <= kNearL; }
 template <int KIND>
 static cudaError_t launch_far_kind(const pc_ctx *ctx, const Launch &L, int64_t tiles, int64_t tiles_v, cudaStream_t st) {
   Launch M = L;
   M.T = L.T & ~1;
   if (M.T) {
-    const cudaError_t e = launch_far_nf<KIND, 2>(ctx, M, tiles, tiles_v, st);
+    const cudaError_t e = far_fine(L) ? launch_far_nf<KIND, 2, true>(ctx, M, tiles, tiles_v, st)
+                                      : launch_far_nf<KIND, 2, false>(ctx, M, tiles, tiles_v, st);
     if (e != cudaSuccess) return e;
   }
   if (L.T & 1) {
@@ -1791,7 +1798,8 @@ static cudaError_t launch_far_kind(const pc_ctx *ctx, const Launch &L, int64_t t
     M.uf[0] = L.uf[k];
     M.uf_hi[0] = L.uf_hi[k];
     M.uf_lo[0] = L.uf_lo[k];
-    return launch_far_nf<KIND, 1>(ctx, M, tiles, tiles_v, st);
+    return far_fine(L) ? launch_far_nf<KIND, 1, true>(ctx, M, tiles, tiles_v, st)
+                       : launch_far_nf<KIND, 1, false>(ctx, M, tiles, tiles_v, st);
   }
   return cudaSuccess;
 }
@@ -1811,6 +1819,11 @@ static cudaError_t launch_far(const pc_ctx *ctx, const Launch &L, int kind, cuda
 constexpr double kFarWork = 1e8;  // fields_mixed_kernel: about 700 us, fields_far_kernel 250
 // lists: (point, dipole, frame) triples from which the far distances (a memset and a small kernel, 5 us) pay
 constexpr double kFarListWork = 2e6;
+// the largest tile (radius, c dt): a tile's float32 offsets from its anchor round at 6e-8 of that, which counts
+// where a source is nearer than the anchor.  Against the 16 x 16 tiles of fields_mixed_kernel, on points 405 c dt
+// from a source beyond a corner: within 1e-6 of the source scale in both up to 1200 (steps of 20 nm at 1 as), from
+// 4 (100 nm) to 2 times its error above
+constexpr double kFarTile = 1200.0;
 static bool far_candidate(Launch &L, bool plane_of_dipoles, int32_t T) {
   if (!plane_of_dipoles || (double)L.src.N * (double)L.pts.P * (double)T < kFarWork) return false;
   double r2 = 0.0;
@@ -1823,7 +1836,7 @@ static bool far_candidate(Launch &L, bool plane_of_dipoles, int32_t T) {
     r2 = std::max(r2, q);
   }
   const double r = sqrt(r2) * (1.0 + 1e-6) + 1e-3;
-  if (!(r < 1e5)) return false;
+  if (!(r <= kFarTile)) return false;
   L.tile_r = (float)r;
   return true;
 }

@@ -234,3 +234,49 @@ def test_mixed_drive_of_wide_dipoles(ctx, amp, dt, steps, cell):
     m = pc.pc_dipoles_run(ctx, lod, dt, steps, precision=pc.PC_MIXED, want_Ed=True)
     e = float(((m["Ed"] - f["Ed"]).abs().amax(-1) / f["Ed"].abs().amax(-1)).max())
     assert e < 1e-5, e
+
+
+# ------------------------------------------------------------------------------------------------
+# planes whose tiles are wide against the distance of their sources
+# ------------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("kind", [pc.PC_TOTAL, pc.PC_COULOMB, pc.PC_RADIATION])
+@pytest.mark.parametrize("step", [1.6e-9, 1.9e-9, 1e-8, 2e-8, 2.2e-8, 4e-8, 1e-7, 3e-7, 1e-6])
+def test_points_much_nearer_than_the_anchor_of_their_tile(ctx, step, kind):
+    # sources straight beyond a corner of a tile (32 x 16 points), as near to it as the far form allows (400 c dt
+    # and the tile's radius from the anchor); steps on both sides of far_fine's (5.8 c dt) and of kFarTile's (70).
+    # The same frames in a call too small for the far kernel are fields_mixed_kernel's: the fields at those corners
+    # are no further from the oracle than twice its (its tiles of 16 x 16 are 1.6 times smaller) and a few
+    # float32 roundings of the source scale.
+    dt, nu, nv, N = 1e-18, 160, 144, 12
+    cdt = W.C * dt
+    rng = np.random.default_rng(59)
+    org = np.zeros((N, 3))
+    for j in range(N):
+        tu, tv = j % 5, (2 * j) % 9  # a tile of the 5 x 9, and a corner of it
+        corner = step * np.array([tu * 32 + 31 * (j & 1), tv * 16 + 15 * (j >> 1 & 1)])
+        out = corner - step * np.array([tu * 32 + 15.5, tv * 16 + 7.5])
+        org[j, :2] = corner + out / np.linalg.norm(out) * (405.0 * cdt)
+    S = int(math.hypot(nu, nv) * step / cdt) + 7000
+    dp = W.sinusoidal_dipoles(org, W.unit_vectors(rng, N), OMEGA0, 1e-11, dt, (S - 1) * dt)
+    times = [(S - 1900) * dt, (S - 1000.5) * dt]
+    reps = int(1e8 / (N * nu * nv * len(times))) + 1
+    iu, iv = np.meshgrid(np.arange(nu), np.arange(nv), indexing="ij")
+    pts = np.stack([iu.ravel() * step, iv.ravel() * step, np.zeros(nu * nv)], axis=1)
+    # of the points beyond 400 c dt of every source, the 12 nearest to each, and scattered ones
+    r = np.linalg.norm(pts[:, None] - org[None], axis=2) / cdt
+    r[r.min(axis=1) <= 400.0] = np.inf
+    p = np.unique(np.concatenate([np.argsort(r[:, j])[:12] for j in range(N)] + [rng.integers(0, nu * nv, 60)]))
+    p = p[np.isfinite(r[p, 0])]
+    ref = oracle.fields(pts[p], times, dipoles=dp, kind=kind)
+    assert ref["status"] == oracle.OK
+    dev = pc.dipoles_to_device(dp)
+    err = []
+    for frames in (times * reps, times):
+        out = pc.pc_fields_plane(ctx, dipoles=dev, origin=(0.0, 0.0, 0.0), eu=(step, 0, 0), ev=(0, step, 0), nu=nu, nv=nv,
+                                 times=frames, kind=kind, precision=pc.PC_MIXED)
+        err.append({})
+        for k in ("E", "B", "phi", "A"):
+            g = out[k][:len(times), torch.as_tensor(p, device="cuda")].cpu().numpy().astype(np.float64)
+            sc = ref["scale_source"]["E"] / W.C if k == "B" else ref["scale_source"][k]
+            err[-1][k] = float(np.max(_norm(g - ref[k]) / sc))
+    assert all(err[0][k] <= 2.0 * err[1][k] + 3e-7 for k in err[0]), err

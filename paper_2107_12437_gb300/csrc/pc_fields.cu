@@ -1973,12 +1973,12 @@ static pc_status fields_impl(pc_ctx *ctx, const pc_charges *ch, const pc_dipole_
   // dipole sample indices are 32-bit integers in both paths (the difference form's solves)
   if (has_dp && s.Sd > (int64_t)1 << 30) return PC_ERR_ARG;
   // the float64 sum of dipoles alone in the split form, where the pairs outweigh writing the float32 mirror
-  // (about 0.01 ns a sample against 0.4 ns a pair saved)
+  // (about 0.01 ns a sample against 0.4 ns a pair saved), and there is the memory for it
+  const size_t mirror = ((size_t)s.N * (size_t)s.Sd + 4 * (size_t)s.N) * sizeof(float4);
   const bool split = precision == PC_F64 && has_dp && !has_ch && (double)P * (double)T * s.N >= 1e5 &&
-                     (double)P * (double)T >= (double)s.Sd / 16.0;
+                     (double)P * (double)T >= (double)s.Sd / 16.0 && reserve_optional(ctx->hist_f32, mirror, mirror);
   if (split) {
     const size_t nd = (size_t)s.N * s.Sd;
-    if (ctx->hist_f32.reserve((nd + 4 * (size_t)s.N) * sizeof(float4)) != cudaSuccess) return PC_ERR_CUDA;
     float4 *Hd = (float4 *)ctx->hist_f32.ptr;
     L.Hd = Hd;
     launch_prep_dipoles(s, Hd, Hd + nd, nullptr, L.status, st);

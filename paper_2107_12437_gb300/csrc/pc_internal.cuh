@@ -43,6 +43,20 @@ struct Buf {
   }
 };
 
+// Room for a form that is faster but that the call can do without: b of n bytes, `extra` of them for that form
+// (more than 1 GB: at most half of the memory that is left).  False, with no error pending, where it cannot be had.
+inline bool reserve_optional(Buf &b, size_t n, size_t extra) {
+  if (n <= b.bytes) return true;
+  size_t left = 0, all = 0;
+  if (extra > ((size_t)1 << 30) && (cudaMemGetInfo(&left, &all) != cudaSuccess || extra > left / 2)) {
+    cudaGetLastError();
+    return false;
+  }
+  if (b.reserve(n) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
+}
+
 }  // namespace pc
 
 struct pc_ctx {

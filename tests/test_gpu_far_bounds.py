@@ -280,3 +280,36 @@ def test_points_much_nearer_than_the_anchor_of_their_tile(ctx, step, kind):
             sc = ref["scale_source"]["E"] / W.C if k == "B" else ref["scale_source"][k]
             err[-1][k] = float(np.max(_norm(g - ref[k]) / sc))
     assert all(err[0][k] <= 2.0 * err[1][k] + 3e-7 for k in err[0]), err
+
+
+# ------------------------------------------------------------------------------------------------
+# devices without the memory for a form's tables
+# ------------------------------------------------------------------------------------------------
+def _fill(leave):
+    """All of the device's free memory but `leave` bytes, as one tensor."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.empty(torch.cuda.mem_get_info()[0] - leave, dtype=torch.uint8, device="cuda")
+
+
+def test_float64_fields_without_memory_for_the_mirror():
+    # 64 histories of 10^6 samples: the split form's float32 mirror takes 1.07 GB, of which 0.6 are left
+    N, S, P = 64, 1 << 20, 70000
+    rng = np.random.default_rng(3)
+    dp = W.sinusoidal_dipoles(rng.uniform(0.0, 1e-6, (N, 3)), W.unit_vectors(rng, N), OMEGA0, 1e-11, 1e-18, (S - 1) * 1e-18)
+    dev = pc.dipoles_to_device(dp)
+    pts = torch.as_tensor(np.concatenate([rng.uniform(0.0, 1e-6, (P, 2)), np.full((P, 1), 1.3e-6)], axis=1), device="cuda")
+    c = pc.Context(0)
+    ref = {k: v.clone() for k, v in pc.pc_fields(c, dipoles=dev, points=pts, times=[1e-12]).items()}
+    c.close()
+    c = pc.Context(0)
+    pc.pc_fields(c, dipoles=dev, points=pts[:100], times=[1e-12])  # the two-charge form, loaded
+    hold = _fill(600 << 20)
+    try:
+        out = pc.pc_fields(c, dipoles=dev, points=pts, times=[1e-12])
+    finally:
+        del hold
+        c.close()
+        torch.cuda.empty_cache()
+    for k in ("E", "B", "phi", "A"):
+        assert float((out[k] - ref[k]).abs().max() / ref[k].abs().max()) < 1e-10, k

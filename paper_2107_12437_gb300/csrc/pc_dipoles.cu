@@ -2860,14 +2860,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   const size_t fg_bytes = mixed ? 0 : al(nbn * dp->N * sizeof(float4));  // the float64 drive's pair geometry
   const size_t far_bytes = pf_bytes + pd_bytes + cr_bytes + am_bytes + fg_bytes + 256;
   bool far = grid && !motion && !pl.tables_only && !pl.two_charge && n_end < ((int64_t)1 << 30);
-  if (far && far_bytes > ((size_t)1 << 30) && far_off + far_bytes > ctx->run_scratch.bytes) {
-    size_t mfree = 0, mall = 0;  // at most half of what is left
-    if (cudaMemGetInfo(&mfree, &mall) != cudaSuccess || far_bytes > mfree / 2) far = false;
-  }
-  if (far && ctx->run_scratch.reserve(far_off + far_bytes) != cudaSuccess) {
-    cudaGetLastError();
-    far = false;
-  }
+  far = far && pc::reserve_optional(ctx->run_scratch, far_off + far_bytes, far_bytes);
   if (!far && ctx->run_scratch.reserve(far_off) != cudaSuccess) return PC_ERR_CUDA;
   char *scr = (char *)ctx->run_scratch.ptr;
   pc::RunArgs a;
@@ -2969,22 +2962,26 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
     hs = W;
     wm = W - 1;
   }
-  if (K < 2 || hs >= ((int64_t)1 << 27)) {  // (the carried sums sit in lanes K - 2 and K - 1)
-    far = false;
-    a.pfar = nullptr;
-    a.pfar64 = nullptr;
-    a.pfarD = nullptr;
-    a.nbad = nullptr;
-  }
-  const bool mirror = mixed || far;  // the history's float32 mirror
   const bool own_ring = !full_store && !pl.sd;
   const size_t ring_b = own_ring ? al(nbn * (size_t)hs * sizeof(double)) : 0;
-  const size_t h_bytes = mirror ? al(nbn * (size_t)hs * sizeof(float4)) : 0;
+  const size_t mirror_b = al(nbn * (size_t)hs * sizeof(float4));
   // the fit's kinetic energies: after the run from the full store, or per step into their own rows
   const int64_t first = opts->fit ? opts->first_index : 0;
   const size_t ke_b = opts->fit ? al(nbn * (size_t)(full_store ? So : So - first) * sizeof(double)) : 0;
   // moving origins in the mixed drive: their float32 mirror (three float4 per half-step sample)
   const size_t om_b = (motion && mixed) ? al(nbn * (size_t)(2 * n_end + 1) * 3 * sizeof(float4)) : 0;
+  // (the carried sums sit in lanes K - 2 and K - 1; the float64 run can do without the mirror)
+  if (far && (K < 2 || hs >= ((int64_t)1 << 27) ||
+              (!mixed && !pc::reserve_optional(ctx->run_store, 3 * ring_b + mirror_b + ke_b + om_b, mirror_b)))) {
+    far = false;
+    a.pfar = nullptr;
+    a.pfar64 = nullptr;
+    a.pfarD = nullptr;
+    a.nbad = nullptr;
+    if (!mixed) a.pgeo = nullptr;
+  }
+  const bool mirror = mixed || far;  // the history's float32 mirror
+  const size_t h_bytes = mirror ? mirror_b : 0;
   if (ctx->run_store.reserve(3 * ring_b + h_bytes + ke_b + om_b) != cudaSuccess) return PC_ERR_CUDA;
   char *sto = (char *)ctx->run_store.ptr;
   a.hs = hs;
@@ -4529,24 +4526,25 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
     fields_adj_kernel<<<dim3((unsigned)dp->N, (unsigned)fseed->T, (unsigned)dp->B), 128, fsm, st>>>(A, *fseed, fw);
   }
   const dim3 fgrid((unsigned)dp->N, (unsigned)dp->B);
-  // the split reverse, where the run has its tables; a source's receivers over as many CTAs as have a group
-  // of 32 for each warp, up to four waves of three CTAs per SM
+  // the split reverse, where the segment's run has its tables (it goes without them where there is no memory for
+  // them); a source's receivers over as many CTAs as have a group of 32 for each warp, up to four waves of three
+  // CTAs per SM
   const size_t smem_split = sizeof(RevShared) * kRevWarps;
-  const bool split = a.pfar64 != nullptr && !mov;
-  if (split && cudaFuncSetAttribute(adj_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_split) !=
-                   cudaSuccess)
+  if (!mov && cudaFuncSetAttribute(adj_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_split) !=
+                  cudaSuccess)
     return PC_ERR_CUDA;
-  dim3 sgrid = fgrid;
-  if (split) {
-    const int64_t groups = (int64_t)((a.fcp + 31) / 32) * a.nsplit, most = (int64_t)ctx->num_sms * 12;
-    sgrid.z = (unsigned)std::max<int64_t>(1, std::min<int64_t>((groups + kRevWarps - 1) / kRevWarps,
-                                                              most / std::max<int64_t>(1, (int64_t)nbn)));
-  }
   // reverse sweep over the causal blocks, last first (segment by segment when checkpointing)
   for (int64_t c = nseg - 1; c >= 0; --c) {
     if (Cask > 0 && c < nseg - 1) {
       pc_status rs = recompute(c);
       if (rs != PC_OK) return rs;
+    }
+    const bool split = a.pfar64 != nullptr && !mov;
+    dim3 sgrid = fgrid;
+    if (split) {
+      const int64_t groups = (int64_t)((a.fcp + 31) / 32) * a.nsplit, most = (int64_t)ctx->num_sms * 12;
+      sgrid.z = (unsigned)std::max<int64_t>(1, std::min<int64_t>((groups + kRevWarps - 1) / kRevWarps,
+                                                                most / std::max<int64_t>(1, (int64_t)nbn)));
     }
     const int64_t s0 = c * C, s1 = std::min(n_steps, s0 + C);
     const int64_t nblocks = (s1 - s0 + K - 1) / K;

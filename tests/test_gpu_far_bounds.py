@@ -313,3 +313,61 @@ def test_float64_fields_without_memory_for_the_mirror():
         torch.cuda.empty_cache()
     for k in ("E", "B", "phi", "A"):
         assert float((out[k] - ref[k]).abs().max() / ref[k].abs().max()) < 1e-10, k
+
+
+def test_float64_run_without_memory_for_the_mirror():
+    # 66 oscillators, 400 000 steps: a mirror of 422 MB next to outputs of 211 MB each; 250 MB are left for it
+    steps = 400000
+    lod = pc.lo_config_to_device(_cloud(66))
+    c = pc.Context(0)
+    ref = pc.pc_dipoles_run(c, lod, 1e-18, steps, precision=pc.PC_F64)
+    c.close()
+    size = sum(v.numel() * v.element_size() for v in ref.values() if torch.is_tensor(v))
+    ref = ref["d"].cpu()
+    c = pc.Context(0)
+    pc.pc_dipoles_run(c, lod, 1e-18, 100, precision=pc.PC_MIXED)  # (the kernels loaded, and scratch for 100 steps)
+    hold = _fill(size + (250 << 20))
+    try:
+        out = pc.pc_dipoles_run(c, lod, 1e-18, steps, precision=pc.PC_F64)
+    finally:
+        del hold
+        c.close()
+        torch.cuda.empty_cache()
+    d = out["d"].cpu()
+    # (both forms' E_d are within 1e-10, which 400 000 steps may add up)
+    assert float((d - ref).abs().max() / ref.abs().max()) < 1e-7
+
+
+@pytest.mark.parametrize("checkpoint", [0, 16000])
+def test_float64_gradients_without_memory_for_the_mirror(checkpoint):
+    # the whole adjoint's memory but half of its mirror's 42 MB (checkpointed: of a segment's 35)
+    steps = 40000
+    lod = pc.lo_config_to_device(_cloud(66))
+    w = torch.linspace(0.5, 1.5, 66, dtype=torch.float64, device="cuda").view(1, 66)
+
+    def run(c, n=steps):
+        return pc.pc_dipoles_adjoint(c, lod, 1e-18, n, w, checkpoint_every=min(checkpoint, n // 2))
+
+    c = pc.Context(0)
+    run(c, 100)
+    c.close()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    c = pc.Context(0)
+    ref = [g.clone() for g in run(c)]
+    torch.cuda.synchronize()
+    used = before - torch.cuda.mem_get_info()[0]
+    c.close()
+    mirror = 66 * (32768 if checkpoint else steps + 1) * 16  # (a segment's store: 16000 steps and the depth, a power of 2)
+    c = pc.Context(0)
+    hold = _fill(used - mirror // 2)
+    try:
+        got = run(c)
+    finally:
+        del hold
+        c.close()
+        torch.cuda.empty_cache()
+    # both forms' gradients agree to 1e-10 over 417 steps (tests/test_gpu_far.py)
+    for g, r in zip(got, ref):
+        assert float((g - r).abs().max() / r.abs().max()) < 1e-10 * steps / 417

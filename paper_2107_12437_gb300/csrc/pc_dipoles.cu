@@ -131,9 +131,14 @@ constexpr int kTabC = 4 * 16 + 6;
 // and the moment and its rate up to which the far form's limits hold
 constexpr int kTab = kTabC + 13;
 
-// The far form's limits are set for moments up to kFarGrow times the largest initial one of the
-// configuration (and rates up to that times its omega0): a pair is far from d_max / (q kFarX) on.  A run
-// whose moments grow beyond takes the two-charge form for as long as a block can reach such a sample.
+// Which pairs are far is decided by the largest initial moment of the configuration, d_max / q, and rate (that
+// times the largest omega0) against the limits of pc_far_f32.cuh, and a run stays in the form while its moments and
+// rates stay within kFarGrow times these: X/R and V reach 1.5 times the limits.  What the form drops is then up to
+// 2.25 times what is stated there (mixed: 1.7e-7 of a pair's terms; the split form's fifth order 1.5e-13), which
+// leaves it no further off than two charges.  Resumed runs with moments 1.45 times the declared ones, rms error of
+// E_d in the far form and with two charges: mixed 8.4e-7 and 1.9e-6 (clouds of 100, 10 pm), 2.20e-6 and 2.15e-6
+// (2200); float64, against binary128, 4e-12 to 6e-12 and 7e-12 to 6e-11 (10 to 28 pm).  A run whose moments grow
+// beyond takes the two-charge form for as long as a block can reach such a sample.
 constexpr double kFarGrow = 1.5;
 constexpr int kFarNone = -1, kFarNear = -2;
 constexpr double kFarDelay = 16 + 4;  // samples: a block of kMaxBlock steps reads well behind the newest one

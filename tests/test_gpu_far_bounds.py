@@ -371,3 +371,36 @@ def test_float64_gradients_without_memory_for_the_mirror(checkpoint):
     # both forms' gradients agree to 1e-10 over 417 steps (tests/test_gpu_far.py)
     for g, r in zip(got, ref):
         assert float((g - r).abs().max() / r.abs().max()) < 1e-10 * steps / 417
+
+
+# ------------------------------------------------------------------------------------------------
+# moments that have grown
+# ------------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("amp,cell,first", [(1e-11, 3.75e-8, 1600), (1.9e-11, 6e-8, 3200), (2.85e-11, 1e-7, 4800)])
+def test_drive_of_grown_moments(ctx, amp, cell, first):
+    # a run resumed with declared moments 1.45 times smaller than its samples' (the forms stay to 1.5), pairs around
+    # both forms' least distance for these: E_d no further off than in the two-charge form, which declared moments
+    # of a hundredth force, by the rms of the same samples (a fifth for their scatter)
+    N, dt, n = 100, 1e-18, 400
+    cfg = _cloud(N, cell=cell, seed=5)
+    cfg.d0[:] = W.E_CHARGE * amp
+    lod = pc.lo_config_to_device(cfg)
+    state = torch.zeros(pc.pc_dipoles_state_size(ctx, lod, dt), dtype=torch.float64, device="cuda")
+    pc.pc_dipoles_run(ctx, lod, dt, first, precision=pc.PC_F64, state_out=state)
+    D = int(state[2])
+    smp = state[4 + N:].view(N, D + 1, 3).cpu().numpy()
+    at, recv = np.linspace(1, n, 40).astype(int), [0, 50, 99]
+    rms = {}
+    for precision in (pc.PC_F64, pc.PC_MIXED):
+        for scale in (1 / 1.45, 0.01):
+            decl = pc.lo_config_to_device(cfg)
+            decl.d0 *= scale
+            f = pc.pc_dipoles_run(ctx, decl, dt, n, precision=precision, state_in=state, want_Ed=True)
+            # on the run's own samples
+            hist = [np.concatenate([smp[:, :, c], f[k][0, :, 1:].cpu().numpy()], axis=1)
+                    for c, k in enumerate(("d", "d_dot", "d_ddot"))]
+            ref = _ed_binary128(cfg, hist, (first - D) * dt, (first + at) * dt, recv)
+            rms[precision, scale] = float(np.sqrt(np.mean([((f["Ed"][0, i].cpu().numpy()[at] - e) / np.max(np.abs(e))) ** 2
+                                                           for e, i in zip(ref, recv)])))
+    assert rms[pc.PC_F64, 1 / 1.45] <= 1.2 * rms[pc.PC_F64, 0.01], rms
+    assert rms[pc.PC_MIXED, 1 / 1.45] <= 1.2 * rms[pc.PC_MIXED, 0.01], rms

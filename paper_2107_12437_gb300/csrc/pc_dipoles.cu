@@ -3304,7 +3304,7 @@ struct AdjArgs {
   double *gpos, *gvel, *gacc;
   double *disp;
   double *g_origin, *g_omega0, *g_d0;
-  unsigned long long *ebmax;  // the largest |Ebar| so far (bits), or null
+  unsigned long long *ebmax;  // per configuration the largest |Ebar| so far (bits), or null
   int64_t margin;      // samples of slack around the retarded window (charge offsets)
 };
 
@@ -3475,7 +3475,7 @@ __global__ void adj_rk4_kernel(const AdjArgs A, int64_t n0, int kb) {
     A.lam[2 * bi + 1] = y1bar;
     A.carry[bi] = e1b;
     A.w0bar[bi] += w0b;
-    if (A.ebmax) atomicMax(A.ebmax, (unsigned long long)__double_as_longlong(m));
+    if (A.ebmax) atomicMax(A.ebmax + bi / a.N, (unsigned long long)__double_as_longlong(m));
   }
 }
 
@@ -3831,8 +3831,8 @@ __global__ void __launch_bounds__(kRevWarps * 32, 3) adj_split_kernel(const __gr
   const int nbad = *((volatile int *)a.nbad);
   const bool all_near = nbad >= 0 && n0 - a.max_reach <= nbad;
   const int kb_steps = ns / 2, n0i = (int)n0;
-  // the float32 part runs on stage adjoints over their largest so far, in units of k_e e / (c dt)^2
-  const double emax = __longlong_as_double((long long)*A.ebmax), iemax = emax > 0.0 ? 1.0 / emax : 0.0;
+  // the float32 part runs on stage adjoints over the configuration's largest so far, in units of k_e e / (c dt)^2
+  const double emax = __longlong_as_double((long long)A.ebmax[b]), iemax = emax > 0.0 ? 1.0 / emax : 0.0;
   const double unit = emax * a.e_unit;
   const double iL = 1.0 / (kC * a.dt), L = kC * a.dt;
   const double Rj[3] = {a.origin[3 * bj], a.origin[3 * bj + 1], a.origin[3 * bj + 2]};
@@ -4293,7 +4293,7 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
   const size_t edb = al(nbn * (size_t)Sg * sizeof(double));
   const size_t half = al(nbn * (size_t)(Sg - 1) * sizeof(double));
   const size_t mu_b = al(nbn * (size_t)Wg * 3 * sizeof(double));
-  const size_t small = al((nbn * (2 + 1 + (2 * kMaxBlock + 1) + 1 + 2 + 2 + 1) + 1) * sizeof(double));
+  const size_t small = al((nbn * (2 + 1 + (2 * kMaxBlock + 1) + 1 + 2 + 2 + 1) + dp->B) * sizeof(double));
   const size_t fit_b = rates ? 3 * al(nbn * (size_t)flen * sizeof(double)) + al(4 * nbn * sizeof(double)) : 0;
   const size_t ck_b = Cask > 0 ? al((size_t)std::max<int64_t>(nseg - 1, 0) * st_len * sizeof(double)) : 0;
   if (ctx->adj_scratch.reserve(3 * hist + edb + half + mu_b + small + fit_b + ck_b) != cudaSuccess) return PC_ERR_CUDA;
@@ -4398,7 +4398,7 @@ static pc_status adjoint_core(pc_ctx *ctx, const pc_dipoles *dp, double dt, int6
   A.wts = A.tau + 2 * nbn;
   A.disp = A.wts + 2 * nbn;
   A.ebmax = (unsigned long long *)(A.disp + nbn);
-  if (cudaMemsetAsync(A.ebmax, 0, sizeof(double), st) != cudaSuccess) return PC_ERR_CUDA;
+  if (cudaMemsetAsync(A.ebmax, 0, dp->B * sizeof(double), st) != cudaSuccess) return PC_ERR_CUDA;
   A.delay = delay;
   if (motion) {
     a.org_pos = motion->pos;

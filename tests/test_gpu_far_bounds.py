@@ -404,3 +404,17 @@ def test_drive_of_grown_moments(ctx, amp, cell, first):
                                                            for e, i in zip(ref, recv)])))
     assert rms[pc.PC_F64, 1 / 1.45] <= 1.2 * rms[pc.PC_F64, 0.01], rms
     assert rms[pc.PC_MIXED, 1 / 1.45] <= 1.2 * rms[pc.PC_MIXED, 0.01], rms
+
+
+def test_gradients_of_configurations_of_very_unequal_weights(ctx):
+    # each configuration's gradients are its own weights' alone, however small these are beside another's: the
+    # split reverse's float32 terms (1e-7 of a gradient) keep their scale.  Scaling rounds at 1e-13 or so.
+    cfg = _cloud(90, B=2, seed=90)
+    w = torch.linspace(0.5, 1.5, 180, dtype=torch.float64, device="cuda").view(2, 90)
+    ref = pc.pc_dipoles_adjoint(ctx, pc.lo_config_to_device(cfg), cfg.dt, 300, w)
+    v = w.clone()
+    v[1] *= 1e-40
+    got = pc.pc_dipoles_adjoint(ctx, pc.lo_config_to_device(cfg), cfg.dt, 300, v)
+    for g, r in zip(got, ref):
+        assert float((g[0] - r[0]).abs().max() / r[0].abs().max()) < 1e-12
+        assert float((g[1] / 1e-40 - r[1]).abs().max() / r[1].abs().max()) < 1e-12

@@ -1480,10 +1480,6 @@ __device__ __forceinline__ FarSums far_sources(const RunArgs &a, size_t b0, size
       s_k[sl] = pk;
       s_j[sl] = make_int2(z + a.nsplit * t, n0 - D - 1);
     }
-    if ((cnt & 1) && lane == 31) {  // an even count: a source of no weight
-      s_k[cnt] = make_float4(0.f, 0.f, 0.f, 0.f);
-      s_j[cnt] = make_int2(z, 0);
-    }
     __syncwarp();
     // the next group's entries come in while this one's samples do
     D = kFarNone;
@@ -1679,8 +1675,8 @@ template <bool NEAR, bool RING, bool MID>
 __global__ void __launch_bounds__(kRunWarps * 32, NEAR ? 2 : 3)
     lo_far_drive_kernel(const __grid_constant__ RunArgs a, int64_t n0, int ns) {
   __shared__ double sh[kRunWarps][32];
-  __shared__ float4 s_k[kRunWarps][34];
-  __shared__ int2 s_j[kRunWarps][34];
+  __shared__ float4 s_k[kRunWarps][32];
+  __shared__ int2 s_j[kRunWarps][32];
   __shared__ MidPair s_m[MID ? kRunWarps : 1][32];
   if (!block_at(a, n0, ns)) return;
   const int warp = threadIdx.x >> 5, b = blockIdx.y, i = blockIdx.x * kRunWarps + warp, z = blockIdx.z;
@@ -1741,10 +1737,6 @@ __device__ __forceinline__ int far_stage64(const RunArgs &a, size_t tab, int z, 
     const int sl = __popc(mf & ((1u << lane) - 1u));
     s_k[sl] = {p.x, p.y, p.z, p.w, fmax(p.w - 0.5, 0.0), fmax(0.5 - p.w, 0.0)};
     s_j[sl] = make_int2(z + a.nsplit * t, n0 - D - 1);
-  }
-  if ((cnt & 1) && lane == 31) {
-    s_k[cnt] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    s_j[cnt] = make_int2(z, 0);
   }
   __syncwarp();
   return cnt;
@@ -1908,8 +1900,8 @@ template <bool RING>
 __global__ void __launch_bounds__(kRunWarps * 32)
     lo_far64_drive_kernel(const __grid_constant__ RunArgs a, int64_t n0, int ns) {
   __shared__ double sh[kRunWarps][32];
-  __shared__ FarEntry64 s_k[kRunWarps][34];
-  __shared__ int2 s_j[kRunWarps][34];
+  __shared__ FarEntry64 s_k[kRunWarps][32];
+  __shared__ int2 s_j[kRunWarps][32];
   if (!block_at(a, n0, ns)) return;
   const int warp = threadIdx.x >> 5, b = blockIdx.y, i = blockIdx.x * kRunWarps + warp, z = blockIdx.z;
   if (i >= a.N) return;
@@ -1945,8 +1937,8 @@ template <int MODE, bool RING>
 __global__ void __launch_bounds__(kCoopWarps * 32, 1) lo_coop_kernel(const __grid_constant__ RunArgs a, int recv) {
   extern __shared__ double dyn[];
   __shared__ double sh[kCoopWarps][32];
-  __shared__ typename std::conditional<MODE == 2, FarEntry64, float4>::type s_k[kCoopWarps][34];
-  __shared__ int2 s_j[kCoopWarps][34];
+  __shared__ typename std::conditional<MODE == 2, FarEntry64, float4>::type s_k[kCoopWarps][32];
+  __shared__ int2 s_j[kCoopWarps][32];
   __shared__ MidPair s_m[MODE == 2 ? 1 : kCoopWarps][32];
   __shared__ int s_stop, s_nbad, s_next;
   CoopRecv *rc = reinterpret_cast<CoopRecv *>(dyn);
@@ -3817,8 +3809,8 @@ struct RevShared {
   float T[32][4];
   float h[6][33];            // adjoints of the two samples of a stage's segment (X, V, A each), columns = stages
   double eb[40];             // the stage adjoints of a receiver, stage s at eb[3 + s], zeros around
-  FarEntry64 k[34];
-  int2 j[34];
+  FarEntry64 k[32];
+  int2 j[32];
 };
 __global__ void __launch_bounds__(kRevWarps * 32, 3) adj_split_kernel(const __grid_constant__ AdjArgs A, int64_t n0, int ns) {
   extern __shared__ double dyn[];

@@ -108,6 +108,7 @@ struct RunArgs {
   double *carry64;    // the float64 drive's, four each
   int *nbad;
   unsigned *bar;      // the cooperative loop's barrier
+  unsigned long long *npair;  // [3]: pairs that are near, mid and far
   int mid;            // mixed far drive with mid pairs
   int K;              // the run's causal block length (grid path)
   int max_reach;      // the largest reach over the batch
@@ -1206,7 +1207,10 @@ __global__ void lo_rstat_init_kernel(const RunArgs a) {
   a.rstat[3 * b + 2] = 0ull;
   if (a.pfarD) {
     a.amax[2 * b] = a.amax[2 * b + 1] = 0ull;
-    if (b == 0) a.nbad[0] = a.nbad[1] = -1;
+    if (b == 0) {
+      a.nbad[0] = a.nbad[1] = -1;
+      a.npair[0] = a.npair[1] = a.npair[2] = 0ull;
+    }
   }
 }
 
@@ -1236,6 +1240,7 @@ __global__ void __launch_bounds__(256) lo_pairs_kernel(const RunArgs a) {
     const float xm = a.pfarD ? (float)(__longlong_as_double((long long)a.amax[2 * b]) * iL) : 0.f;
     const float vm = a.pfarD ? xm * (float)(__longlong_as_double((long long)a.amax[2 * b + 1]) * a.dt) : 0.f;
     double rmin = 1e300, vmax = 0.0, rmax = 0.0;
+    int nnear = 0, nmid = 0, nfar = 0;
     for (int64_t ij = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ij < NN;
          ij += (int64_t)gridDim.x * blockDim.x) {
       const int i = (int)(ij / N), j = (int)(ij % N);
@@ -1285,6 +1290,8 @@ __global__ void __launch_bounds__(256) lo_pairs_kernel(const RunArgs a) {
           const double k2 = kKe * ir * ir * (3.0 * c1 * c2 - c12);
           a.pfar64[e] = {k2 * ir, k2 * (1.0 / kC), k3, x - fl};
           a.pfarD[e] = far ? (int)fmin(fl, 1073741824.0) : (i == j ? kFarNone : kFarNear);
+          nnear += !far && i != j;
+          nfar += far;
         }
         if (a.pfar) {
           // p_i . E of the far form: k1 X + k2 V + k3 A
@@ -1307,7 +1314,20 @@ __global__ void __launch_bounds__(256) lo_pairs_kernel(const RunArgs a) {
             a.pfar[e] = make_float4(k2 * ir, k2, k3, (float)(x - fl));
           }
           a.pfarD[e] = far ? (int)fmin(fl, kFarMid - 1.0) | (mid ? kFarMid : 0) : (i == j ? kFarNone : kFarNear);
+          nnear += !far && i != j;
+          nmid += far && mid;
+          nfar += far && !mid;
         }
+      }
+    }
+    if (a.pfarD) {
+      nnear = __reduce_add_sync(0xffffffffu, nnear);
+      nmid = __reduce_add_sync(0xffffffffu, nmid);
+      nfar = __reduce_add_sync(0xffffffffu, nfar);
+      if ((threadIdx.x & 31) == 0) {
+        if (nnear) atomicAdd(a.npair, (unsigned long long)nnear);
+        if (nmid) atomicAdd(a.npair + 1, (unsigned long long)nmid);
+        if (nfar) atomicAdd(a.npair + 2, (unsigned long long)nfar);
       }
     }
     s_r[threadIdx.x] = rmin;
@@ -2627,6 +2647,20 @@ static void *coop_kernel_for(const RunArgs &a, bool mixed) {
   if (a.near_L > 0.f) return ring ? (void *)lo_coop_kernel<1, true> : (void *)lo_coop_kernel<1, false>;
   return ring ? (void *)lo_coop_kernel<0, true> : (void *)lo_coop_kernel<0, false>;
 }
+// Whether the far and split drives are the faster ones for a run with npair near, mid and far pairs.  They take a
+// near pair with a warp to itself, whatever the block's length K, where the two-charge drives put 32 / 2 K pairs
+// side by side, and the mixed one's near pairs (pair_drive_f32) are heavier than those of drive_sources_grid: dense
+// clusters lose.  Float64, in units of a near pair: a far one 0.04.  Mixed, in units of a pair of the two-charge
+// drive at K = 16: near 1.5, mid 0.68, far 0.18, that drive at shorter blocks 0.1 + 0.9 / (pairs side by side),
+// and 10 us a block for its graph of kernels where the cooperative loop runs.  Measured, new / old time of a block on
+// lattices of 66 to 4000 oscillators, K = 3, 7 and 16: float64 0.03 to 3.75, mixed 0.17 to 2.58; where this rule
+// takes the new drives 0.03 to 0.87 and 0.17 to 0.94.
+static bool far_pays(const unsigned long long *npair, int K, bool mixed, bool coop) {
+  const double near = (double)npair[0], mid = (double)npair[1], far = (double)npair[2];
+  const double side = std::max(1, 32 / (2 * K)), all = near + mid + far;
+  if (!mixed) return near + 0.04 * far < (coop ? 0.6 : 0.9) * all / side;
+  return 1.5 * near + 0.68 * mid + 0.18 * far < (0.1 + 0.9 / side) * all + (coop ? 48000.0 : 0.0);
+}
 // Receivers per CTA of the cooperative loop, 0 where the loop of graph nodes is faster
 static int coop_recv(const pc_ctx *ctx, size_t nbn, bool mixed) {
   const size_t r = (nbn + ctx->num_sms - 1) / ctx->num_sms;
@@ -2904,6 +2938,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
     a.amax = (unsigned long long *)(f + pf_bytes + pd_bytes + cr_bytes);
     a.nbad = (int *)(f + pf_bytes + pd_bytes + cr_bytes + am_bytes);
     a.bar = (unsigned *)(a.nbad + 16);
+    a.npair = (unsigned long long *)(a.nbad + 32);
     if (!mixed) a.pgeo = (float4 *)(f + pf_bytes + pd_bytes + cr_bytes + am_bytes + 256);
     a.fcp = far_cp;
     a.nsplit = far_split;
@@ -2928,6 +2963,8 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   pc::lo_tables_kernel<<<dp->B, 256, 0, st>>>(a);
   // block lengths and reaches back on the host, and the status of the tables (unit axes)
   std::vector<int> kr(2 * (size_t)dp->B + 1);
+  unsigned long long npair[3] = {0, 0, 0};
+  if (far && cudaMemcpyAsync(npair, a.npair, sizeof(npair), cudaMemcpyDeviceToHost, st) != cudaSuccess) return PC_ERR_CUDA;
   if (cudaMemcpyAsync(kr.data(), a.kblock, 2 * (size_t)dp->B * sizeof(int), cudaMemcpyDeviceToHost, st) !=
           cudaSuccess ||
       cudaMemcpyAsync(kr.data() + 2 * (size_t)dp->B, a.status, sizeof(int), cudaMemcpyDeviceToHost, st) !=
@@ -2968,7 +3005,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   // moving origins in the mixed drive: their float32 mirror (three float4 per half-step sample)
   const size_t om_b = (motion && mixed) ? al(nbn * (size_t)(2 * n_end + 1) * 3 * sizeof(float4)) : 0;
   // (the carried sums sit in lanes K - 2 and K - 1; the float64 run can do without the mirror)
-  if (far && (K < 2 || hs >= ((int64_t)1 << 27) ||
+  if (far && (K < 2 || hs >= ((int64_t)1 << 27) || !far_pays(npair, K, mixed, recv > 0) ||
               (!mixed && !pc::reserve_optional(ctx->run_store, 3 * ring_b + mirror_b + ke_b + om_b, mirror_b)))) {
     far = false;
     a.pfar = nullptr;

@@ -121,6 +121,9 @@ struct Launch {
   // tile's points about its anchor, both in c dt
   const float *rfar;
   float tile_r;
+  // float64 sums of dipoles alone: of the kSplitAsk sampled pairs that split_count_kernel counts in status[1], the
+  // number of near ones from which fields_f64_kernel runs and fields_split64_kernel does not (0: not asked)
+  int near_min;
 };
 
 // the float32 outputs' units: E in k_e e / L^2, B in k_e e / (L^2 c), phi in k_e e / L,
@@ -241,6 +244,7 @@ __device__ __forceinline__ void scale_f64(double iLd, const double (&acc)[10], d
 
 template <int KIND>
 __global__ void __launch_bounds__(128) fields_f64_kernel(const Launch L) {
+  if (L.status[1] < L.near_min) return;
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int f = blockIdx.y;
   if (p >= L.pts.P || f >= L.T) return;
@@ -606,6 +610,7 @@ __global__ void __launch_bounds__(128) fields_split64_kernel(const __grid_consta
     int equal;
   };
   __shared__ Src s_src[kSplitChunk];
+  if (L.status[1] >= L.near_min) return;
   const Sources &s = L.src;
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int f = blockIdx.y;
@@ -660,6 +665,34 @@ __global__ void __launch_bounds__(128) fields_split64_kernel(const __grid_consta
   double E[3] = {0, 0, 0}, B[3] = {0, 0, 0}, A[3] = {0, 0, 0}, phi = 0.0;
   scale_f64(iLd, acc, E, B, phi, A);
   store_f64(L, f, p, E, B, phi, A, mask);
+}
+
+// How many of kSplitAsk pairs, spread over points, dipoles and frames, are near for the split form (its conditions
+// in split_dipole): a pair that is costs it 1.1 (unequal masses) to 1.4 of the two-charge kernel's, for the attempt
+// and the call out of line, and one that is not 0.36.  The choice stays on the device, both kernels are launched and
+// one returns (5 us a call; 64 dipoles whose charges are too fast, 20 000 points: 2.34 -> 1.98 ms).
+constexpr int kSplitAsk = 1024;
+constexpr double kSplitNearMost = 0.65;
+__global__ void __launch_bounds__(128) split_count_kernel(const __grid_constant__ Launch L) {
+  const unsigned k = blockIdx.x * blockDim.x + threadIdx.x;  // < kSplitAsk
+  const Sources &s = L.src;
+  // multiplicative hashing: the three indices independent of one another
+  const int64_t p = (int64_t)(((unsigned long long)(k * 2654435769u) * (unsigned long long)L.pts.P) >> 32);
+  const int j = (int)(((unsigned long long)((k + 1u) * 2246822519u) * (unsigned)s.N) >> 32);
+  const int f = (int)(((unsigned long long)((k + 1u) * 3266489917u) * (unsigned)L.T) >> 32);
+  double r[3];
+  point_at(L.pts, p, r);
+  const double iLd = L.iLd, rx = (r[0] - s.origin[3 * j]) * iLd, ry = (r[1] - s.origin[3 * j + 1]) * iLd,
+               rz = (r[2] - s.origin[3 * j + 2]) * iLd;
+  const double R = sqrt(rx * rx + ry * ry + rz * rz), x = L.uf[f] - R;
+  bool far = s.m1[j] == s.m2[j] && R > L.r_excl * iLd + 1.5 && x > 2.0 && x < (double)(s.Sd - 3);
+  if (far) {
+    const size_t n = (size_t)j * (size_t)s.Sd + (size_t)x;
+    const double iq = 1.0 / s.qd[j], X = fabs(s.d[n] * iq * iLd), V = fabs(s.dd[n] * iq * (1.0 / kC));
+    far = X <= fmin((double)kSplitFieldX * R, (double)kSplitSamples) && V <= (double)kSplitFieldV;
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, !far);
+  if ((threadIdx.x & 31) == 0 && m) atomicAdd(L.status + 1, __popc(m));
 }
 
 // The point of thread tid in tile blockIdx.x (list: 256 consecutive points; plane: a block of rows x
@@ -2068,10 +2101,15 @@ static pc_status fields_impl(pc_ctx *ctx, const pc_charges *ch, const pc_dipole_
     if (precision == PC_F64) {
       dim3 grid((unsigned)((P + 127) / 128), (unsigned)L.T);
       if (split) {
+        // (each launch's frames by themselves: in the first ones the field may not have arrived)
+        if (chunk > 0 && cudaMemsetAsync(L.status + 1, 0, sizeof(int), st) != cudaSuccess) return PC_ERR_CUDA;
+        L.near_min = (int)(kSplitNearMost * kSplitAsk);
+        split_count_kernel<<<kSplitAsk / 128, 128, 0, st>>>(L);
         if (kind == PC_TOTAL) fields_split64_kernel<PC_TOTAL><<<grid, 128, 0, st>>>(L);
         else if (kind == PC_COULOMB) fields_split64_kernel<PC_COULOMB><<<grid, 128, 0, st>>>(L);
         else fields_split64_kernel<PC_RADIATION><<<grid, 128, 0, st>>>(L);
-      } else if (kind == PC_TOTAL) fields_f64_kernel<PC_TOTAL><<<grid, 128, 0, st>>>(L);
+      }
+      if (kind == PC_TOTAL) fields_f64_kernel<PC_TOTAL><<<grid, 128, 0, st>>>(L);
       else if (kind == PC_COULOMB) fields_f64_kernel<PC_COULOMB><<<grid, 128, 0, st>>>(L);
       else fields_f64_kernel<PC_RADIATION><<<grid, 128, 0, st>>>(L);
     } else {

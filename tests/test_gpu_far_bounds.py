@@ -418,3 +418,30 @@ def test_gradients_of_configurations_of_very_unequal_weights(ctx):
     for g, r in zip(got, ref):
         assert float((g[0] - r[0]).abs().max() / r[0].abs().max()) < 1e-12
         assert float((g[1] / 1e-40 - r[1]).abs().max() / r[1].abs().max()) < 1e-12
+
+
+@pytest.mark.parametrize("case", ["fast", "unequal masses", "dense", "not yet there"])
+def test_float64_fields_of_mostly_near_pairs(ctx, case):
+    # a large call whose pairs are nearly all near takes the general kernel, as a small one (below 1e5 pairs) does:
+    # the same bits.  Then 32 frames, a launch's worth, before the field has left any source, and one after that.
+    rng = np.random.default_rng(29)
+    N, P, box = 20, 6000, 1e-7 if case == "dense" else 1e-6
+    dp = W.sinusoidal_dipoles(rng.uniform(0.0, box, (N, 3)), W.unit_vectors(rng, N), OMEGA0, 1e-10 if case == "fast" else 1e-11,
+                              1e-18, 9e-15)
+    if case == "unequal masses":
+        dp.m1 *= 2.0
+    z = 4e-6 if case == "not yet there" else box / 2
+    pts = torch.as_tensor(np.concatenate([rng.uniform(0.0, box, (P, 2)), np.full((P, 1), z)], axis=1), device="cuda")
+    dev = pc.dipoles_to_device(dp)
+    times = list(np.linspace(4e-15, 9e-15, 32)) if case == "not yet there" else [6.2e-15, 6.3e-15]
+    late = [16e-15] if case == "not yet there" else []
+    big = {k: v.clone() for k, v in pc.pc_fields(ctx, dipoles=dev, points=pts, times=times + late).items()}
+    for q in range(0, 300, 100):
+        small = pc.pc_fields(ctx, dipoles=dev, points=pts[q:q + 100], times=times)
+        for k in ("E", "B", "phi", "A"):
+            assert torch.equal(big[k][:len(times), q:q + 100], small[k]), k
+    if late:
+        small = pc.pc_fields(ctx, dipoles=dev, points=pts[:400], times=late)
+        for k in ("E", "B", "phi", "A"):
+            assert float((big[k][len(times), :400] - small[k][0]).abs().max() / small[k].abs().max()) < 1e-10, k
+            assert not torch.equal(big[k][len(times), :400], small[k][0]), k  # the split form's

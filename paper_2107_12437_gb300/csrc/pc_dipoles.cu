@@ -2867,7 +2867,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
   const size_t dl_bytes = al(nbn * dp->N * sizeof(int2));
   const size_t geo_bytes = mixed ? al(nbn * dp->N * sizeof(float4)) : 0;
   const size_t rs_bytes = al(3 * (size_t)dp->B * sizeof(unsigned long long));
-  const size_t k_bytes = al(2 * (size_t)dp->B * sizeof(int));
+  const size_t k_bytes = al((2 * (size_t)dp->B + 6) * sizeof(int));  // block lengths, reaches, three pair counts
   const size_t part_bytes = grid ? al((size_t)pc::kMaxSplit * es_bytes) : es_bytes;
   const size_t blk_bytes = al(2 * sizeof(int64_t));
   const size_t tab_bytes = al(nbn * pc::kTab * sizeof(double));
@@ -2938,7 +2938,7 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
     a.amax = (unsigned long long *)(f + pf_bytes + pd_bytes + cr_bytes);
     a.nbad = (int *)(f + pf_bytes + pd_bytes + cr_bytes + am_bytes);
     a.bar = (unsigned *)(a.nbad + 16);
-    a.npair = (unsigned long long *)(a.nbad + 32);
+    a.npair = (unsigned long long *)(a.kblock + 2 * (size_t)dp->B);
     if (!mixed) a.pgeo = (float4 *)(f + pf_bytes + pd_bytes + cr_bytes + am_bytes + 256);
     a.fcp = far_cp;
     a.nsplit = far_split;
@@ -2961,17 +2961,16 @@ static pc_status run_impl(pc_ctx *ctx, const pc_dipoles *dp, double dt, int64_t 
     if (motion) pc::lo_closest_kernel<<<dim3(gx, gy), 256, 0, st>>>(a);
   }
   pc::lo_tables_kernel<<<dp->B, 256, 0, st>>>(a);
-  // block lengths and reaches back on the host, and the status of the tables (unit axes)
-  std::vector<int> kr(2 * (size_t)dp->B + 1);
-  unsigned long long npair[3] = {0, 0, 0};
-  if (far && cudaMemcpyAsync(npair, a.npair, sizeof(npair), cudaMemcpyDeviceToHost, st) != cudaSuccess) return PC_ERR_CUDA;
-  if (cudaMemcpyAsync(kr.data(), a.kblock, 2 * (size_t)dp->B * sizeof(int), cudaMemcpyDeviceToHost, st) !=
-          cudaSuccess ||
-      cudaMemcpyAsync(kr.data() + 2 * (size_t)dp->B, a.status, sizeof(int), cudaMemcpyDeviceToHost, st) !=
-          cudaSuccess ||
+  // block lengths, reaches and pair counts back on the host, and the status of the tables (unit axes)
+  const size_t nk = 2 * (size_t)dp->B + 6;
+  std::vector<int> kr(nk + 1);
+  if (cudaMemcpyAsync(kr.data(), a.kblock, nk * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaMemcpyAsync(kr.data() + nk, a.status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return PC_ERR_CUDA;
-  if (kr[2 * (size_t)dp->B] == PC_ERR_ARG) return PC_ERR_ARG;
+  if (kr[nk] == PC_ERR_ARG) return PC_ERR_ARG;
+  unsigned long long npair[3];
+  memcpy(npair, kr.data() + 2 * (size_t)dp->B, sizeof(npair));
   int K = pc::kMaxBlock;
   int64_t D = 1;
   for (int b = 0; b < dp->B; ++b) {

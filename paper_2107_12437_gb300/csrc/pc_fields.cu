@@ -682,14 +682,17 @@ __global__ void __launch_bounds__(128) split_count_kernel(const __grid_constant_
   const int f = (int)(((unsigned long long)((k + 1u) * 3266489917u) * (unsigned)L.T) >> 32);
   double r[3];
   point_at(L.pts, p, r);
-  const double iLd = L.iLd, rx = (r[0] - s.origin[3 * j]) * iLd, ry = (r[1] - s.origin[3 * j + 1]) * iLd,
-               rz = (r[2] - s.origin[3 * j + 2]) * iLd;
-  const double R = sqrt(rx * rx + ry * ry + rz * rz), x = L.uf[f] - R;
-  bool far = s.m1[j] == s.m2[j] && R > L.r_excl * iLd + 1.5 && x > 2.0 && x < (double)(s.Sd - 3);
+  const double iLd = L.iLd;
+  // (float32 is enough for a sample, and its latency a fraction)
+  const float rx = (float)((r[0] - s.origin[3 * j]) * iLd), ry = (float)((r[1] - s.origin[3 * j + 1]) * iLd),
+              rz = (float)((r[2] - s.origin[3 * j + 2]) * iLd);
+  const float R2 = fmaf(rz, rz, fmaf(ry, ry, rx * rx)), R = R2 * rsqrt_fast(R2), x = (float)L.uf[f] - R;
+  bool far = s.m1[j] == s.m2[j] && R > (float)(L.r_excl * iLd) + 1.5f && x > 2.f && x < (float)(s.Sd - 3);
   if (far) {
-    const size_t n = (size_t)j * (size_t)s.Sd + (size_t)x;
-    const double iq = 1.0 / s.qd[j], X = fabs(s.d[n] * iq * iLd), V = fabs(s.dd[n] * iq * (1.0 / kC));
-    far = X <= fmin((double)kSplitFieldX * R, (double)kSplitSamples) && V <= (double)kSplitFieldV;
+    const size_t n = (size_t)j * (size_t)s.Sd + (size_t)min((int64_t)x, s.Sd - 1);
+    const float iq = __fdividef((float)kE, (float)s.qd[j]);
+    const float X = fabsf((float)(s.d[n] * (iLd / kE)) * iq), V = fabsf((float)(s.dd[n] * (1.0 / (kC * kE))) * iq);
+    far = X <= fminf(kSplitFieldX * R, kSplitSamples) && V <= kSplitFieldV;
   }
   const unsigned m = __ballot_sync(0xffffffffu, !far);
   if ((threadIdx.x & 31) == 0 && m) atomicAdd(L.status + 1, __popc(m));

@@ -1410,7 +1410,7 @@ __global__ void __launch_bounds__(kRunWarps * 32) lo_drive_kernel(const RunArgs 
 // of 4096 oscillators.
 // A block whose reach holds a sample beyond the limits (a.nbad) goes through lo_drive_kernel's sources
 // altogether; the next far block then forms the carried sums itself.
-// Measured, 4096 oscillators in a 600 nm cube: 3.10 -> 0.38 ms a block of 16 steps, about 11 warp
+// Measured, 4096 oscillators in a 600 nm cube: 3.10 -> 0.42 ms a block of 16 steps, about 11 warp
 // instructions per pair and block against 179; bound by the gathers of the samples from L2 (272 B a pair,
 // 12 TB/s; the pair tables, 20 B a pair, take 0.05 ms from HBM).
 // MID: where the cooperative loop below runs (smaller configurations, whose near pairs are a larger part: 8 %

@@ -601,7 +601,7 @@ __device__ __forceinline__ float kahan_get(const KahanArr &k, int tid, int i) {
 
 // float64, dipoles alone: sources staged in shared memory, each pair in the split form (pc_far_f32.cuh)
 // where it holds, the others, by a bit mask per stage, with the two charges.  64 dipoles of 10 pm, 301 x 517
-// points: 5.20 -> 1.92 ms; the float64 unit is the bound, 70 instructions a pair and 280 a near one.
+// points: 5.20 -> 1.93 ms; the float64 unit is the bound, 70 instructions a pair and 280 a near one.
 constexpr int kSplitChunk = 32;
 template <int KIND>
 __global__ void __launch_bounds__(128) fields_split64_kernel(const __grid_constant__ Launch L) {

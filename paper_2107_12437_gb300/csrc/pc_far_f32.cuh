@@ -264,6 +264,12 @@ __device__ __forceinline__ bool split_dipole(double rx, double ry, double rz, do
   // 1e-14 instead of 1e-15 into the fields of 10 pm dipoles)
   const float dX = (float)(Dd * sx), dV = (float)(Dv * sv), dA = (float)(Da * sa);
   const float Xf = fmaf(thf, dX, h0.x);
+  if (KIND == PC_RADIATION) {
+    // the radiation field's cubic terms are a difference from the Coulomb field's, in float32: where the slow motion
+    // of a charge or a zero of A leaves little of the former, that rounding (1e-7 of (X/R + V)^3) is all of it
+    const float c = fabsf(Xf) * iRf + fmaxf(fabsf(h0.y), fabsf(h1.y));
+    if (!(c * c * c <= 1e-5f * fabsf(fmaf(thf, dA, h0.z)) * Rf)) return false;
+  }
   // a charge whose own retarded time lies off the centre's segment: its state differs from the segment's
   // extension by the overshoot times the second difference of the samples.  The charges' delays are off the
   // centre's by -+ X mu / 2 + (X^2 (1 - mu^2) / 2 - mu^2 X X') / 4 R: the overshoots from those in float64

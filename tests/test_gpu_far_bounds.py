@@ -445,3 +445,30 @@ def test_float64_fields_of_mostly_near_pairs(ctx, case):
         for k in ("E", "B", "phi", "A"):
             assert float((big[k][len(times), :400] - small[k][0]).abs().max() / small[k].abs().max()) < 1e-10, k
             assert not torch.equal(big[k][len(times), :400], small[k][0]), k  # the split form's
+
+
+@pytest.mark.parametrize("dt,amp,omega,z", [(1e-20, 1.5e-12, 1e14, 3e-8), (2.6e-20, 1e-13, 2e13, 4e-9), (1e-18, 1e-11, OMEGA0, 3e-7)])
+def test_float64_radiation_fields_of_slow_charges(ctx, dt, amp, omega, z):
+    # the radiation field alone, a 1e-4 to 1e-8 part of the Coulomb field so close to slow charges (and as much in
+    # the last case): plain errors within 1e-10 of it, at every phase of the moment
+    S = 40001
+    t0 = 0.25 * 2 * math.pi / omega
+    rng = np.random.default_rng(37)
+    s = int(t0 / dt) - S // 2  # samples around the moment's peak, and (shifted) around its zero
+    for shift in (0, int(t0 / dt)):
+        t = (s + shift + np.arange(S)) * dt
+        d = W.E_CHARGE * amp * np.tile(np.sin(omega * t), (3, 1))
+        one = np.ones(3)
+        dp = W.Dipoles(origin=rng.uniform(0.0, z / 20, (3, 3)), axis=W.unit_vectors(rng, 3), q=W.E_CHARGE * one, m1=W.M_E * one,
+                       m2=W.M_E * one, d=d, d_dot=W.E_CHARGE * amp * omega * np.tile(np.cos(omega * t), (3, 1)),
+                       d_ddot=-omega * omega * d, t0=0.0, dt=dt)
+        P = 40003
+        pts = np.concatenate([rng.uniform(0.0, z / 4, (P, 2)), np.full((P, 1), z)], axis=1)
+        times = [float((S // 2 + k) * dt + 1.05 * z / W.C) for k in (-3000, 4.3, 5000.5)]
+        out = pc.pc_fields(ctx, dipoles=pc.dipoles_to_device(dp), points=torch.as_tensor(pts, device="cuda"), times=times,
+                           kind=pc.PC_RADIATION)
+        ref = oracle.fields_x(pts[:60], times, dipoles=dp, kind=pc.PC_RADIATION)
+        scale = oracle.fields(pts[:60], times, dipoles=dp, kind=pc.PC_RADIATION)["scale_source"]["E"]
+        for k, sc in (("E", scale), ("B", scale / W.C)):
+            e = _norm(out[k][:, :60].cpu().numpy() - ref[k]) / np.maximum(_norm(ref[k]), 1e-3 * sc)
+            assert float(np.max(e)) <= 1e-10, (k, shift, float(np.max(e)))

@@ -3857,7 +3857,9 @@ __global__ void __launch_bounds__(kRevWarps * 32, 3) adj_split_kernel(const __gr
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   RevShared &sh = reinterpret_cast<RevShared *>(dyn)[warp];
   const int nbad = *((volatile int *)a.nbad);
-  const bool all_near = nbad >= 0 && n0 - a.max_reach <= nbad;
+  // (the table's row of j says which sources are far for the receiver j: the other way round that is the same pair
+  // but for the masses, which are the source's own condition)
+  const bool all_near = (nbad >= 0 && n0 - a.max_reach <= nbad) || a.m1[bj] != a.m2[bj];
   const int kb_steps = ns / 2, n0i = (int)n0;
   // the float32 part runs on stage adjoints over the configuration's largest so far, in units of k_e e / (c dt)^2
   const double emax = __longlong_as_double((long long)A.ebmax[b]), iemax = emax > 0.0 ? 1.0 / emax : 0.0;

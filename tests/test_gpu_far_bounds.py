@@ -472,3 +472,18 @@ def test_float64_radiation_fields_of_slow_charges(ctx, dt, amp, omega, z):
         for k, sc in (("E", scale), ("B", scale / W.C)):
             e = _norm(out[k][:, :60].cpu().numpy() - ref[k]) / np.maximum(_norm(ref[k]), 1e-3 * sc)
             assert float(np.max(e)) <= 1e-10, (k, shift, float(np.max(e)))
+
+
+@pytest.mark.parametrize("steps", [60, 417])
+@pytest.mark.parametrize("every", [2, 3, 66])
+def test_split_reverse_of_some_unequal_masses(ctx, every, steps):
+    # a pair is far by its source's masses, whatever the receiver's: gradients of configurations with both kinds as
+    # in tests/test_gpu_far.py::test_split_reverse_against_the_two_charge_form
+    cfg = _cloud(66, seed=47)
+    cfg.m1[:, ::every] *= 1.5
+    w = torch.linspace(0.5, 1.5, 66, dtype=torch.float64, device="cuda").view(1, 66)
+    got = pc.pc_dipoles_adjoint(ctx, pc.lo_config_to_device(cfg), cfg.dt, steps, w)
+    cfg.m1 = np.nextafter(cfg.m1, np.inf)
+    ref = pc.pc_dipoles_adjoint(ctx, pc.lo_config_to_device(cfg), cfg.dt, steps, w)
+    for g, r in zip(got, ref):
+        assert float((g - r).abs().max() / r.abs().max()) < 1e-10
